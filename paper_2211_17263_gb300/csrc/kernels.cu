@@ -2785,13 +2785,18 @@ __global__ void __launch_bounds__(kBlock) k_hd_norms(const HdDraws H) {
         s_last = atomicAdd(&N.ctr, 1u) == unsigned(split - 1);
     }
     __syncthreads();
-    if (s_last && threadIdx.x == 0) {
-        __threadfence();
+    if (!s_last) return;
+    // the parts loaded side by side, then added in order by one thread (one thread loading each
+    // part as it adds it waited a round trip to L2 per part: 36 at D = 49,152)
+    __threadfence();
+    __shared__ double2 s_part[kNormSplitMax];
+    if (int(threadIdx.x) < split) s_part[threadIdx.x] = __ldcg(&N.part[threadIdx.x]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
         double z = 0.0, r = 0.0;
         for (int q = 0; q < split; ++q) {
-            const double2 v = __ldcg(&N.part[q]);
-            z += v.x;
-            r += v.y;
+            z += s_part[q].x;
+            r += s_part[q].y;
         }
         N.v = make_float2(float(sqrt(z)), float(sqrt(r)));
         N.ctr = 0u;  // ready for the next launch
@@ -2856,21 +2861,32 @@ __global__ void __launch_bounds__(kBlock) k_hd_perturb(const HdDraws H) {
 }
 
 // a6 + a7 over D parameters: g_d = (1/2P) sum_p w_{2p,d} (L_2p - L_2p+1) (a skinny GEMV,
-// W^T dL, fixed order over p in FP64), then Adam with t = the already advanced step.
-__global__ void __launch_bounds__(kBlock) k_hd_grad(const HdGrad G) {
+// W^T dL, fixed order over p in FP64), then Adam with t = the already advanced step. Bound by the
+// latency of its loads (3 MB of weights at D = 49,152, 16 renders): the losses are read once per
+// CTA, the weights eight at a time, and CTAs of 128 threads spread over every SM.
+constexpr int kGradBlock = 128;
+__global__ void __launch_bounds__(kGradBlock) k_hd_grad(const HdGrad G) {
+    __shared__ double s_dl[kMaxRenders];  // pair differences (antithetic) or losses
     pdl_enter();
-    const int d = int(blockIdx.x) * kBlock + int(threadIdx.x);
+    const int n = G.antithetic ? G.R / 2 : G.R, stride = G.antithetic ? 2 : 1;
+    for (int p = threadIdx.x; p < n; p += kGradBlock)
+        s_dl[p] = G.antithetic ? __ldcg(G.losses + 2 * p) - __ldcg(G.losses + 2 * p + 1) : __ldcg(G.losses + p);
+    __syncthreads();
+    const int d = int(blockIdx.x) * kGradBlock + int(threadIdx.x);
     if (d >= G.D) return;
+    const float* w = G.w + d;
+    const size_t step = size_t(stride) * G.D;
     double g = 0.0;
-    if (G.antithetic) {
-        const int P = G.R / 2;
-        for (int p = 0; p < P; ++p)
-            g += double(G.w[size_t(2 * p) * G.D + d]) * (__ldcg(G.losses + 2 * p) - __ldcg(G.losses + 2 * p + 1));
-        g /= double(2 * P);
-    } else {
-        for (int q = 0; q < G.R; ++q) g += double(G.w[size_t(q) * G.D + d]) * __ldcg(G.losses + q);
-        g /= double(G.R);
+    int p = 0;
+    for (; p + 8 <= n; p += 8) {  // eight weights in flight, then the same sums
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = w[size_t(p + q) * step];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) g += double(v[q]) * s_dl[p + q];
     }
+    for (; p < n; ++p) g += double(w[size_t(p) * step]) * s_dl[p];
+    g /= double(G.antithetic ? 2 * n : n);
     const float gf = float(g);
     if (G.grad_out) G.grad_out[d] = gf;
     if (G.theta) adam_update(G.theta[d], G.m[d], G.v[d], gf, __ldcg(G.step_dev), G.lr, G.b1, G.b2, G.eps);
@@ -2889,7 +2905,7 @@ cudaError_t launch_hd_draws(const HdDraws& H, cudaStream_t stream) {
 
 cudaError_t launch_hd_grad(const HdGrad& G, cudaStream_t stream) {
     if (G.D <= 0) return cudaSuccess;
-    return launch_pdl(k_hd_grad, (G.D + kBlock - 1) / kBlock, kBlock, stream, G);
+    return launch_pdl(k_hd_grad, (G.D + kGradBlock - 1) / kGradBlock, kGradBlock, stream, G);
 }
 
 // ---------------------------------------------------------------------------
