@@ -61,7 +61,9 @@ struct BaseScene {
 
 // Primitive records (4 x float4, grouped: spheres, quads, boxes):
 //   sphere: [0] centre, radius   [1] r^2, 1/r, mat (int bits), prim (int bits)
-//   quad:   [0] centre, mat      [1] unit normal, prim   [2] u, 1/(u.u)   [3] v, 1/(v.v)
+//   quad:   [0] centre, mat | axis << 8   [1] unit normal, prim   [2] u, 1/(u.u)   [3] v, 1/(v.v);
+//           axis-aligned (axis 1..3: the normal along x, y, z): [2].w and [3].w hold the half
+//           extents along the lower and the higher edge axis
 //   box:    [0] min corner, mat  [1] max corner, prim
 // Materials (2 x float4): [0] albedo, type (int bits)  [1] emission, ior.
 // Lights: int4 (kind, record slot, prim, mat) and the emitter's area.
@@ -70,8 +72,8 @@ struct __align__(16) InstScene {
     unsigned seed_lo, seed_hi, step, c3;  // path stream: key and counter words 2, 3
     float4 eye;    // xyz, tan(vfov/2)
     float4 fwd;    // xyz, aspect W/H
-    float4 right;  // xyz, 0
-    float4 up;     // xyz, 0
+    float4 right;  // xyz, 1/(u.u) of the first textured quad (texture scenes)
+    float4 up;     // xyz, its 1/(v.v)
     float4 bg;     // background radiance, 0
     int4 light[kMaxLights];
     float light_area[kMaxLights];
