@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
         J.var_box[(size_t(r) * kMaxVariant + tid) * 2 + 0] = make_float4(lo.x, lo.y, lo.z, 0.0f);
         J.var_box[(size_t(r) * kMaxVariant + tid) * 2 + 1] = make_float4(hi.x, hi.y, hi.z, 0.0f);
     }
-    if (tid == 0) {
+    if (tid == 32) {
         S.tex = texscene ? J.tex_all + size_t(r) * size_t(J.tex_D) : nullptr;
         S.tex_mat = texscene ? B.tex_mat : -1;
         S.tex_res = texscene ? B.tex_res : 0;
@@ -461,14 +461,21 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
         S.right = make_float4(B.right[0], B.right[1], B.right[2], texscene ? s_tex[0] : 0.0f);
         S.up = make_float4(B.up[0], B.up[1], B.up[2], texscene ? s_tex[1] : 0.0f);
         S.bg = make_float4(B.bg[0], B.bg[1], B.bg[2], 0.0f);
-        int nl = 0;
-        for (int i = 0; i < B.n_prims && nl < kMaxLights; ++i) {  // emitters, in primitive order
-            const int mat = B.prim_mat[i];
+    }
+    if (tid < 32) {  // emitters, in primitive order: lane = primitive
+        bool emits = false;
+        int mat = 0;
+        if (tid < B.n_prims) {
+            mat = B.prim_mat[tid];
             const float4 e = S.mat[mat][1];
-            if (!(e.x > 0.0f || e.y > 0.0f || e.z > 0.0f) || B.prim_type[i] == kBox) continue;
-            const int slot = B.prim_slot[i];
+            emits = (e.x > 0.0f || e.y > 0.0f || e.z > 0.0f) && B.prim_type[tid] != kBox;
+        }
+        const unsigned m = __ballot_sync(kFull, emits);
+        const int nl = __popc(m & ((1u << tid) - 1u));
+        if (emits && nl < kMaxLights) {
+            const int slot = B.prim_slot[tid];
             float area;
-            if (B.prim_type[i] == kQuad) {
+            if (B.prim_type[tid] == kQuad) {
                 const float3 u = xyz(S.prim[slot][2]), v = xyz(S.prim[slot][3]);
                 const float3 cr = cross3(u, v);
                 area = sqrtf(dot3(cr, cr));
@@ -476,11 +483,10 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
                 const float rad = S.prim[slot][0].w;
                 area = 4.0f * 3.14159265358979f * rad * rad;
             }
-            S.light[nl] = make_int4(B.prim_type[i], slot, i, mat);
+            S.light[nl] = make_int4(B.prim_type[tid], slot, tid, mat);
             S.light_area[nl] = area;
-            ++nl;
         }
-        S.n_lights = nl;
+        if (tid == 0) S.n_lights = min(__popc(m), kMaxLights);
     }
     __syncthreads();
     {  // write out what the render kernels stage: header, used materials, used primitives
