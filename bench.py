@@ -177,8 +177,8 @@ def _emitter_bound(wl):
 
 def _launches_per_step(wl, sharing):
     """The library's kernel launches in one resident step: sampler, render kernel,
-    finalisation; path sharing adds the per-render and epilogue passes (emitter sharing runs
-    one render kernel); texture scenes add the D-dimensional draws and gradient kernels."""
+    finalisation; path sharing adds the per-render and epilogue passes (replay and
+    render groups run one render kernel); texture scenes add the D-dimensional draws and gradient kernels."""
     import workloads
     n = 5 if sharing and not _emitter_bound(wl) else 3
     if wl.D > 64:
@@ -521,10 +521,12 @@ def main():
         achieved = fp32_counted / (trace_avg_ms * 1e-3) / 1e12 if fp32_counted else model_achieved
         value = world * 1000.0 / step_ms
         traffic = _profiled(wl.name, "dram_bytes_per_step")
-        if sharing and _emitter_bound(wl):
-            kernels = "emitter-sharing kernel k_trace_emit + k_finalize"
-        elif sharing:
+        replayed = (wl.crn and wl.D <= 64 and wl.renders <= 64 and shape["render_groups"] >= 0
+                    and not shape["no_path_sharing"])
+        if sharing and not _emitter_bound(wl):
             kernels = "render pipeline (k_trace shared pass, k_trace_affected, k_shared_epilogue, k_finalize)"
+        elif replayed:
+            kernels = "replay kernel k_trace_replay + k_finalize"
         elif shape["render_groups"] >= 0 and wl.crn and wl.D <= 64:
             kernels = "render-group kernel k_trace_group + k_finalize"
         else:

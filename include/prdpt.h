@@ -138,15 +138,16 @@ typedef struct {
                                   smaller CTAs keep proportionally more; capped at the occupancy
                                   limit); 0 = occupancy limit */
     int32_t no_path_sharing;   /* 0: with crn = 1, trace paths that no perturbation can touch once for
-                                  all renders (geometry-only perturbations), or, when every emitter is
-                                  perturbed and only positions and radii are bound (at most 64
-                                  renders, Eq. 10, no texture), trace each path once with each
-                                  render's own next-event estimates (emitter sharing); same result,
-                                  bit for bit; 1: trace every render */
+                                  all renders (geometry-only perturbations), or, for the other jobs
+                                  without texture or emission bindings (at most 64 renders), trace
+                                  each path once and let every render replay what differs: its own
+                                  next-event estimates, primitives, albedos and tangents (replay);
+                                  same result, bit for bit (Eq. 9's tangents to rounding); 1: trace
+                                  every render */
     int32_t estimator;         /* PRDPT_ESTIMATOR_*: 0 = Eq. 10 (kernel-gradient weights times render
                                   losses); 1 = Eq. 9 (mean over the renders of each render's pathwise
                                   loss gradient: requires sampler = GAUSS, every binding an albedo or
-                                  emission one, D <= 8; no path sharing; single-job steps only) */
+                                  emission one, D <= 8; single-job steps only) */
     int32_t pair_begin;        /* first pair of a shard of a larger estimate (0 normally): this call
                                   computes pairs [pair_begin, pair_begin + pairs) with their global
                                   draw indices (and, with crn = 0, global path-stream fields), and
@@ -157,7 +158,7 @@ typedef struct {
                                   and whose per-render records fit), -1 = off (one render per work
                                   item), or 2, 4, 8, 16, 32. Used with crn = 1, the Eq. 10 estimator
                                   and no texture or emission bindings; ignored otherwise, and when
-                                  emitter sharing applies (see no_path_sharing) */
+                                  replay applies (see no_path_sharing; -1 turns replay off too) */
 } prdpt_grad_opts;
 #define PRDPT_ESTIMATOR_KERNEL_GRADIENT 0 /* Eq. 10: sum_r w_r L_r */
 #define PRDPT_ESTIMATOR_PATHWISE 1        /* Eq. 9: mean_r dL/dtheta (theta + tau_r) */

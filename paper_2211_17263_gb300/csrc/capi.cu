@@ -81,7 +81,8 @@ struct Job {
 struct prdpt_ctx {
     int device = 0;
     int sms = 0;
-    int occ_grad = 1, occ_render = 1, occ_diff = 1, occ_group = 1, occ_emit = 1;
+    int occ_grad = 1, occ_render = 1, occ_diff = 1, occ_group = 1;
+    std::map<unsigned long long, int> occ_replay;  // resident CTAs per SM by kernel variant and shared memory
     uint64_t budget = 0, used = 0;
     std::map<void*, size_t> allocs;
     std::vector<Scene*> scenes;
@@ -125,6 +126,10 @@ struct prdpt_ctx {
     size_t s_norms_n = 0;
     double* s_gpart = nullptr;    // pathwise estimator: [R][tiles][D] gradient partials
     size_t s_gpart_n = 0;
+    double* s_psums = nullptr;    // replay mode: sums of the blocks' parts, and their finished parts (zero)
+    size_t s_psums_n = 0;
+    unsigned* s_pdone = nullptr;
+    size_t s_pdone_n = 0;
     double* s_rgrads = nullptr;   // pathwise estimator: [R][kMaxDiff] per-render gradients
     size_t s_rgrads_n = 0;
     // packed launches
@@ -134,8 +139,10 @@ struct prdpt_ctx {
     size_t batch_cap = 0;
     int batch_blocks = 0;
     // the packed arrays hold the path-sharing jobs, then the render-group jobs, then the
-    // per-render ones: jobs and work items of each kind (one render launch per kind)
+    // per-render ones, then the replay jobs: jobs and work items of each kind (one render
+    // launch per kind)
     int batch_jobs[4] = {0, 0, 0, 0}, batch_items[4] = {0, 0, 0, 0};
+    TraceLaunch batch_replay{};  // variant, table and pool of the packed replay launch
     // optional CUDA-event timing of the render kernel, recorded on its launch stream
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_used, ev_free;
@@ -394,7 +401,6 @@ void block_release(prdpt_ctx* c, void* p, cudaEvent_t ready) {
     c->pending.push_back({p, ready});
 }
 
-bool is_emissive(const float* mp) { return mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f; }
 
 double radial_constant(int D) { return std::sqrt(2.0) * std::exp(std::lgamma(0.5 * (D + 1)) - std::lgamma(0.5 * D)); }
 
@@ -428,6 +434,37 @@ int choose_block(prdpt_ctx* c, int requested, int R, int W, int H, bool render) 
         if (items >= 2 * warps) return px;
     }
     return 8;
+}
+
+// Pixels per block in replay mode when the caller does not say: the most that give every resident
+// warp eight items, while each still fills two batches of paths (32 each). A small image would
+// otherwise end in a half-empty round (GI box walls 256 x 256 at 32 spp, 24 warps per SM: blocks of 8
+// pixels 1.55 ms, of 4 pixels 1.25 ms).
+int choose_replay_block(prdpt_ctx* c, int requested, int W, int H, int spp) {
+    if (requested == 8 || requested == 16 || requested == 32) return requested;
+    const long long warps = (long long)c->sms * kReplayWarpsPerSm;
+    int px = 32;
+    for (; px > 1; px /= 2) {
+        int bw, bh;
+        block_shape(px, &bw, &bh);
+        const long long items = (long long)((W + bw - 1) / bw) * ((H + bh - 1) / bh);
+        if (items >= 8 * warps || px / 2 * spp < 64) break;
+    }
+    return px;
+}
+
+// Work items per block in replay mode: the fewest that do the same for the block size a caller asked
+// for (caustic 237 x 141 at 20 spp, 24 renders, blocks of 32 pixels: 0.68 ms whole, 0.27 ms in 8
+// parts; their sums meet in memory, which costs small blocks 5 %, so the choice above comes first).
+int replay_parts(prdpt_ctx* c, int px, int tiles, int spp) {
+    const long long warps = (long long)c->sms * kReplayWarpsPerSm;
+    int parts = 1;
+    while (2 * parts <= px && (long long)tiles * parts < 8 * warps && (long long)px / (2 * parts) * spp >= 64) parts *= 2;
+    return parts;
+}
+
+size_t replay_part_sums(const TraceJob& J, int tiles) {  // doubles of a replay job's part sums
+    return J.parts > 1 ? size_t(tiles) * J.parts * J.R * (1 + J.nd) : 0;
 }
 
 // The render kernels number their work items (render x pixel block) with 32-bit integers.
@@ -480,18 +517,37 @@ int grid_for_group(prdpt_ctx* c, int items, int ctas_per_sm) {
     return need < cap ? need : cap;
 }
 
-// Persistent grid of the emitter-sharing kernel: one work item per CTA of kGroupBlock threads
-// (ctas_per_sm counts 256-thread CTAs, as above).
-int grid_for_emit(prdpt_ctx* c, int items, int ctas_per_sm) {
-    const int per_sm = (ctas_per_sm > 0 && 2 * ctas_per_sm < c->occ_emit) ? 2 * ctas_per_sm : c->occ_emit;
+// Persistent grid of the replay kernel: one work item per warp of CTAs of kGroupBlock threads
+// (ctas_per_sm counts 256-thread CTAs, as above). 0: the kernel cannot run with its shared memory.
+int grid_for_replay(prdpt_ctx* c, const TraceLaunch& L, int ctas_per_sm) {
+    const unsigned long long key = (unsigned long long)replay_smem(L) << 9 | (L.halves > 1 ? 256u : 0u) | unsigned(L.diff_nd) << 4 |
+                                   (L.replay_mat ? 8u : 0u) | (L.counters ? 4u : 0u) | unsigned(L.replay_move);
+    auto it = c->occ_replay.find(key);
+    if (it == c->occ_replay.end()) it = c->occ_replay.emplace(key, trace_replay_blocks_per_sm(L)).first;
+    const int occ = it->second;
+    const int per_sm = (ctas_per_sm > 0 && 2 * ctas_per_sm < occ) ? 2 * ctas_per_sm : occ;
     const int cap = c->sms * per_sm;
-    return items < cap ? items : cap;
+    const int need = (L.total_items + kGroupBlock / 32 - 1) / (kGroupBlock / 32);
+    return need < cap ? need : cap;
 }
 
-// Work items of a gradient job's render launch: pixel blocks (path sharing, emitter sharing),
+// Add a job to a replay launch: the variant, table and pool that cover every job of it.
+void replay_cover(TraceLaunch& L, const TraceJob& J) {
+    L.replay_mat |= J.var_mats ? 1 : 0;
+    L.replay_move = std::max(L.replay_move, J.n_var > 0 ? (J.black ? 1 : 2) : 0);
+    L.halves = std::max(L.halves, J.R > 32 ? 2 : 1);
+    L.tab_rows = std::max(L.tab_rows, J.R * J.gstride);
+    L.pixels = std::max(L.pixels, J.bw * J.bh / J.parts);
+    L.pool = std::max(L.pool, replay_path_granules(J.depth, J.n_var > 0));
+    if (J.diff) L.diff_nd = J.nd;
+    L.pool = replay_pool(L);
+}
+
+// Work items of a gradient job's render launch: pixel blocks (path sharing, replay),
 // (block, group of gsize renders) (render-group mode) or (render, block).
 long long job_items(const TraceJob& J) {
-    if (J.share || J.emit) return J.tiles;
+    if (J.emit) return (long long)J.tiles * J.parts;
+    if (J.share) return J.tiles;
     if (J.gsize > 0) return (long long)J.tiles * (J.R / J.gsize);
     return (long long)J.R * J.tiles;
 }
@@ -518,8 +574,8 @@ cudaError_t timed_trace(prdpt_ctx* c, const TraceLaunch* Ls, int nL, const Trace
     }
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < nL; ++i) {
-        const int grid = Ls[i].diff_nd ? grid_for_diff(c, Ls[i].total_items, ctas_per_sm)
-                         : (Ls[i].group == 2 && !render) ? grid_for_emit(c, Ls[i].total_items, ctas_per_sm)
+        const int grid = (Ls[i].group == 2 && !render) ? grid_for_replay(c, Ls[i], ctas_per_sm)
+                         : Ls[i].diff_nd ? grid_for_diff(c, Ls[i].total_items, ctas_per_sm)
                          : (Ls[i].group && !render) ? grid_for_group(c, Ls[i].total_items, ctas_per_sm)
                                                     : grid_for(c, Ls[i].total_items, render, ctas_per_sm);
         e = launch_trace(Ls[i], render, grid, stream);
@@ -571,7 +627,6 @@ prdpt_status prdpt_create(prdpt_ctx** out, int32_t device, uint64_t hbm_budget_b
     c->occ_render = trace_blocks_per_sm(true);
     c->occ_diff = trace_diff_blocks_per_sm();
     c->occ_group = trace_group_blocks_per_sm();
-    c->occ_emit = trace_emit_blocks_per_sm();
     e = cudaStreamCreateWithFlags(&c->io, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         delete c;
@@ -758,6 +813,13 @@ static void fill_share(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         J.var_slot[J.n_var++] = B.prim_slot[i];
         J.var_prims |= 1u << B.prim_slot[i];
     }
+    // Only albedos bound: path sharing would trace every path that meets a bound material again
+    // in every render; replay (fill_group) traces it once.
+    if (J.n_var == 0 && o->render_groups >= 0 && 2 * o->pairs <= 64 && B.n_prims <= kGroupPrims &&
+        B.n_mats <= kGroupMats) {
+        J.var_mats = 0u;
+        return;
+    }
     J.share = 1;
     if (I) {
         I->n_var = J.n_var;
@@ -772,12 +834,15 @@ static void fill_share(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
 // renders' paths then agree until a perturbed primitive intervenes), the Eq. 10 estimator,
 // no texture and no emission bindings (those change which primitives emit).
 static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o) {
+    J.black = 0;
+    J.parts = 1;
     J.gsize = 0;
     J.gstride = 0;
     J.emit = 0;
-    if (J.share || o->render_groups < 0 || !o->crn || o->estimator != PRDPT_ESTIMATOR_KERNEL_GRADIENT ||
-        B.tex_mat >= 0 || B.n_prims > kGroupPrims || B.n_mats > kGroupMats)
+    if (J.share || o->render_groups < 0 || !o->crn || B.tex_mat >= 0 || B.n_prims > kGroupPrims ||
+        B.n_mats > kGroupMats)
         return;
+    const bool pathwise = o->estimator == PRDPT_ESTIMATOR_PATHWISE;
     unsigned prims = 0u, mats = 0u;
     bool radius = false;
     for (int d = 0; d < B.D; ++d) {
@@ -789,24 +854,57 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     }
     const int n = __builtin_popcount(prims), nm = __builtin_popcount(mats);
     if (n > kMaxVariant) return;
-    // per render: the perturbed primitives' records (4 float4 each), the bound materials'
-    // albedo rows, and the 8 emitter areas when a radius binding can change one
-    const int stride = 4 * n + nm + (radius ? 2 : 0);
-    if (stride == 0) return;
+    // per render: the rows of the perturbed primitives' records that a binding changes (a quad's
+    // centre row, a sphere's and a box's two rows), the bound materials' albedo rows, and the 8
+    // emitter areas when a radius binding can change one
+    int rows = 0;
+    unsigned offs = 0u;
+    unsigned char src[2 * kMaxVariant] = {};
+    for (int slot = 0, k = 0; slot < B.n_prims; ++slot) {
+        if (!((prims >> slot) & 1u)) continue;
+        offs |= unsigned(rows) << (8 * k++);
+        const bool quad = slot >= B.n_sph && slot < B.n_sph + B.n_quad;
+        for (int q = 0; q < (quad ? 1 : 2); ++q) src[rows++] = (unsigned char)(2 * slot + q);
+    }
+    J.var_rows = rows;
+    J.var_offs = offs;
+    std::memcpy(J.row_src, src, sizeof(src));
+    const int stride = rows + nm + (radius ? 2 : 0);
+    if (n + nm == 0) return;
     const int R = J.R;
-    // Emitter sharing (k_trace_emit): every emitter perturbed, no bound material, at most 64
-    // renders; paths are traced once for all renders (path sharing's switch turns it off)
-    bool emitters_perturbed = n > 0 && mats == 0u && R >= 1 && R <= 64 && R * stride <= kEmitTabRows;
-    for (int i = 0; i < B.n_prims && emitters_perturbed; ++i)
-        if (is_emissive(B.mat_param[B.prim_mat[i]]) && !((prims >> B.prim_slot[i]) & 1u)) emitters_perturbed = false;
-    if (emitters_perturbed && !o->no_path_sharing) {
+    // Replay (k_trace_replay): at most 64 renders whose rows fit; every path is traced once and
+    // each render replays what differs (path sharing's switch turns it off). The pathwise
+    // estimator's rows also hold the parameters' clamp derivatives, by tangent slot.
+    int per_channel[3] = {0, 0, 0};
+    J.nd = 0;
+    for (int k = 0; k < kReplayTangents; ++k) J.slot_param[k] = -1;
+    for (int m = 0; m < kGroupMats; ++m) J.mat_slots[m] = 0;
+    for (int d = 0; pathwise && d < B.D; ++d) {  // tangent slots: 3 i + channel
+        const int slot = 3 * per_channel[B.bind_comp[d]]++ + B.bind_comp[d];
+        J.nd = std::max(J.nd, slot / 3 + 1);
+        if (slot >= kReplayTangents) continue;
+        J.slot_param[slot] = (signed char)(d);
+        J.mat_slots[B.bind_index[d]] |= (unsigned short)(1u << slot);
+    }
+    J.nd = J.nd <= 2 ? 3 * J.nd : (J.nd <= 4 ? 12 : 0);  // 0, 3, 6 or 12
+    const int rstride = stride + (J.nd + 3) / 4;
+    if (!o->no_path_sharing && (!pathwise || J.nd > 0) && R >= 1 && R <= 64 && R * rstride <= kReplayTabRows) {
         J.emit = 1;
-        J.gstride = stride;
+        J.black = 1;
+        for (int i = 0; i < B.n_prims; ++i) {
+            const int m = B.prim_mat[i];
+            const float* mp = B.mat_param[m];
+            if (((prims >> B.prim_slot[i]) & 1u) &&
+                (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f))
+                J.black = 0;
+        }
+        J.gstride = rstride;
         J.n_var = n;
         J.var_prims = prims;
-        J.var_mats = 0u;
+        J.var_mats = mats;
         return;
     }
+    if (pathwise) return;
     int G = 0;
     if (o->render_groups > 0) {
         const int g = o->render_groups;
@@ -1042,10 +1140,11 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
     TraceJob probe{};
     if (prdpt_status st = fill_diff(probe, s->host, o)) return st;
     probe.R = R;
-    fill_share(probe, s->host, o);  // path or emitter sharing: items are blocks, not (render, block)
+    fill_share(probe, s->host, o);  // path sharing or replay: items are blocks, not (render, block)
     fill_group(probe, s->host, o);
     const bool per_block = probe.share || probe.emit;
-    const int px = choose_block(c, o->block_pixels, per_block ? 1 : R, o->width, o->height, false);
+    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp)
+                              : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
     if (prdpt_status st = check_items(per_block ? (long long)tiles : (long long)R * tiles)) return st;
@@ -1064,6 +1163,13 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
         return st;
     if (prdpt_status st = grow(c, &c->s_partials, &c->s_partials_n, (size_t)R * tiles)) return st;
     if (prdpt_status st = grow(c, &c->s_losses, &c->s_losses_n, (size_t)R)) return st;
+    if (probe.emit) {
+        probe.parts = replay_parts(c, px, tiles, o->spp);
+        if (probe.parts > 1 &&  // (without room for the parts' sums the blocks stay whole)
+            (grow(c, &c->s_psums, &c->s_psums_n, replay_part_sums(probe, tiles)) != PRDPT_OK ||
+             grow_zeroed(c, &c->s_pdone, &c->s_pdone_n, (size_t)tiles) != PRDPT_OK))
+            probe.parts = 1;
+    }
     if (probe.diff) {
         if (prdpt_status st = grow(c, &c->s_gpart, &c->s_gpart_n, (size_t)R * tiles * D)) return st;
         if (prdpt_status st = grow(c, &c->s_rgrads, &c->s_rgrads_n, (size_t)R * kMaxDiff)) return st;
@@ -1148,10 +1254,17 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
         J.b2 = adam->b2;
         J.eps = adam->eps;
     }
-    TL.diff_nd = diff_slots(J);
+    J.parts = probe.parts;
     TL.total_items = int(job_items(J));
     TL.share = J.share;
     TL.group = J.emit ? 2 : (J.gsize > 0 ? 1 : 0);
+    TL.diff_nd = diff_slots(J);
+    if (J.emit) {
+        J.queue = c->s_ctl + 0;
+        J.part_sums = c->s_psums;
+        J.part_done = c->s_pdone;
+        replay_cover(TL, J);
+    }
     TL.queue = c->s_ctl + 0;
     TL.counters = c->counting ? c->counters : nullptr;
     TL.status = c->status;
@@ -1328,7 +1441,8 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     j->R = 2 * o->pairs;
     const int D = j->D, R = j->R, W = o->width, H = o->height;
     const bool per_block = probe.share || probe.emit;
-    const int px = choose_block(c, o->block_pixels, per_block ? 1 : R, W, H, false);
+    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp)
+                              : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
     int bw, bh, tiles_x, tiles;
     tiles_for(px, W, H, &bw, &bh, &tiles_x, &tiles);
     if (prdpt_status st = check_items(per_block ? (long long)tiles : (long long)R * tiles)) {
@@ -1365,11 +1479,25 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     const size_t off_tx = (off_hs + (tex ? sizeof(float) * 5 * (size_t)D : 0) + 255) & ~size_t(255);
     const size_t off_nr = (off_tx + (tex ? sizeof(float) * (size_t)R * D : 0) + 255) & ~size_t(255);
     const size_t off_bs = (off_nr + (tex ? sizeof(HdNorm) * (size_t)R : 0) + 255) & ~size_t(255);
-    const size_t total = off_bs + sizeof(BaseScene);  // the job's own copy of its scene
+    const size_t off_ps = (off_bs + sizeof(BaseScene) + 255) & ~size_t(255);  // after the job's own copy of its scene
+    // replay mode: the sums of the blocks' parts and their counters
+    if (probe.emit) probe.parts = replay_parts(c, px, tiles, o->spp);
+    const size_t off_pd = (off_ps + sizeof(double) * replay_part_sums(probe, tiles) + 255) & ~size_t(255);
+    size_t total = off_bs + sizeof(BaseScene);
     void* base = nullptr;
-    if (prdpt_status st = block_alloc(c, &base, total)) {
-        delete j;
-        return st;
+    if (probe.parts > 1) {
+        total = off_pd + sizeof(unsigned) * (size_t)tiles;
+        if (block_alloc(c, &base, total) != PRDPT_OK) {  // without room for them the blocks stay whole
+            probe.parts = 1;
+            base = nullptr;
+            total = off_bs + sizeof(BaseScene);
+        }
+    }
+    if (!base) {
+        if (prdpt_status st = block_alloc(c, &base, total)) {
+            delete j;
+            return st;
+        }
     }
     j->last = take_event(c);
     if (!j->last) {
@@ -1434,6 +1562,7 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
         else  // rendered later on the device (prdpt_job_render_target)
             e = zero_async(c, j->target, sizeof(float4) * (size_t)W * H, io);
     }
+    if (e == cudaSuccess && probe.parts > 1) e = zero_async(c, b + off_pd, sizeof(unsigned) * (size_t)tiles, io);
     if (e == cudaSuccess && probe.share)
         e = zero_async(c, j->accaff, sizeof(unsigned long long) * 3 * (size_t)R * pix, io);
     if (e == cudaSuccess) e = cudaStreamSynchronize(io);
@@ -1497,6 +1626,13 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     }
     fill_share(T, s->host, o, &I);
     fill_group(T, s->host, o);
+    T.queue = j->queue;
+    I.queue_reset = j->queue;
+    if (T.emit) {
+        T.parts = probe.parts;
+        T.part_sums = reinterpret_cast<double*>(b + off_ps);
+        T.part_done = reinterpret_cast<unsigned*>(b + off_pd);
+    }
     if (T.share) {
         T.share_acc = j->share;
         T.acc_aff = j->accaff;
@@ -1583,6 +1719,7 @@ prdpt_status prdpt_step(prdpt_ctx* c, int32_t job_id, void* stream) {
     TL.share = j->trace.share;
     TL.group = j->trace.emit ? 2 : (j->trace.gsize > 0 ? 1 : 0);
     TL.diff_nd = diff_slots(j->trace);
+    if (j->trace.emit) replay_cover(TL, j->trace);
     TL.queue = j->queue;
     TL.counters = c->counting ? c->counters : nullptr;
     TL.status = c->status;
@@ -1623,6 +1760,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
         std::vector<InstJob> inst(n);
         std::vector<TraceJob> trace(n);
         int blocks = 0, jobs_of[4] = {0, 0, 0, 0}, items_of[4] = {0, 0, 0, 0};
+        TraceLaunch cover{};  // the replay launch's variant, table and pool
         for (int i = 0; i < n; ++i) {
             Job* j = order[i];
             const int kd = kind(j);
@@ -1634,6 +1772,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
             trace[i].fin_begin = blocks - j->R;  // same prefix as the sampler CTAs
             const long long it = job_items(j->trace);
             if (prdpt_status st = check_items((long long)items_of[kd] + it)) return st;
+            if (kd == 3) replay_cover(cover, j->trace);
             items_of[kd] += int(it);
             jobs_of[kd]++;
         }
@@ -1683,6 +1822,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
         PRDPT_CUDA(cudaEventRecord(c->h_desc_ev[k], st_));
         c->batch_ids = ids;
         c->batch_blocks = blocks;
+        c->batch_replay = cover;
         for (int q = 0; q < 4; ++q) {
             c->batch_jobs[q] = jobs_of[q];
             c->batch_items[q] = items_of[q];
@@ -1700,7 +1840,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
     TraceLaunch TL[4] = {};
     int nL = 0, first = 0;
     unsigned* queues[4] = {c->s_ctl + 2, c->s_ctl + 3, c->s_ctl + 8, c->s_ctl + 9};
-    for (int kd = 0; kd < 4; ++kd) {  // path-sharing, render-group, per-render, emitter-sharing jobs
+    for (int kd = 0; kd < 4; ++kd) {  // path-sharing, render-group, per-render, replay jobs
         if (c->batch_jobs[kd] > 0) {
             TraceLaunch& T = TL[nL++];
             T.jobs = c->d_trace + first;
@@ -1708,6 +1848,14 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
             T.total_items = c->batch_items[kd];
             T.share = kd == 0 ? 1 : 0;
             T.group = kd == 1 ? 1 : (kd == 3 ? 2 : 0);
+            if (kd == 3) {
+                T.replay_mat = c->batch_replay.replay_mat;
+                T.replay_move = c->batch_replay.replay_move;
+                T.tab_rows = c->batch_replay.tab_rows;
+                T.pool = c->batch_replay.pool;
+                T.halves = c->batch_replay.halves;
+                T.pixels = c->batch_replay.pixels;
+            }
             T.queue = queues[kd];
         }
         first += c->batch_jobs[kd];

@@ -33,6 +33,9 @@ constexpr int kMaxVariant = 4;   // path sharing: perturbed primitives
 constexpr int kMaxShareSpp = 64; // path sharing: samples per pixel (6 bits of a path code)
 constexpr int kSeg = 4;          // path sharing: touching segments kept per path
 constexpr int kMaxDiff = 8;      // pathwise estimator (Eq. 9): differentiated parameters
+constexpr int kGroupPrims = 16;  // render-group and replay mode: at most 16 primitives ...
+constexpr int kGroupMats = 16;   // ... and 16 materials (the staged copy is smaller)
+constexpr int kReplayTangents = 12;  // pathwise estimator in replay mode: tangent slots at most
 
 constexpr unsigned kTagPerturb = 1u;
 constexpr unsigned kTagPath = 2u;
@@ -105,6 +108,7 @@ struct InstJob {
     int hd;                   // high-dimensional parameters: draws made by k_perturb_hd, skip a1 here
     const float* tex_all;     // texture scenes: [R][tex_D] per-render textures, or null
     int tex_D;
+    unsigned* queue_reset;    // replay mode: the job's own item queue, zeroed by its first CTA, or null
     unsigned* share_reset;    // [4] path-sharing counters of the job, zeroed by its first CTA, or null
     // path sharing: bounds of each perturbed primitive in each render, [R][kMaxVariant][2]
     // (min, max corner, inflated), written by the render's CTA; null when not sharing
@@ -174,23 +178,43 @@ struct TraceJob {
     unsigned var_prims;       // record-slot bitmask of perturbed primitives
     unsigned var_mats;        // bitmask of materials whose parameters are bound
     // Render-group mode (k_trace_group): gsize renders per work item (0: per-render items);
-    // each render's row of the per-warp table holds gstride float4 (its records of the
-    // n_var perturbed primitives, the albedo rows of the bound materials, and its emitter
-    // areas when a radius binding can change them)
-    int gsize, gstride;
-    // Emitter-sharing mode (k_trace_emit): 1 when the job's paths are traced once for all its
-    // renders, each render adding its own next-event estimates (gstride as above; items are
-    // pixel blocks of all renders)
-    int emit;
+    // each render's row of the per-warp table holds gstride float4 (the record rows of its
+    // perturbed primitives that a binding changes, the albedo rows of the bound materials, and its
+    // emitter areas when a radius binding can change them). var_rows: the former; row_src[q]: record
+    // slot * 2 + row of the q-th; var_offs: the k-th perturbed primitive's first (bits 8 k .. 8 k + 7)
+    int gsize, gstride, var_rows;
+    unsigned var_offs;
+    unsigned char row_src[2 * kMaxVariant];
+    // Replay mode (k_trace_replay): 1 when the job's paths are traced once for all its renders
+    // and each render replays what differs (gstride as above, plus two rows of clamp derivatives
+    // for the pathwise estimator; items are pixel blocks of all renders, taken from `queue`);
+    // black: every perturbed primitive's material is diffuse and black (and not bound)
+    // a block is `parts` work items (a power of two, at most its pixels), whose sums go through
+    // part_sums [tiles][parts][R][1 + nd] when there are several; part_done counts a block's finished
+    // parts (zero between launches).
+    int emit, black, parts;
+    double* part_sums;
+    unsigned* part_done;
+    // pathwise estimator in replay mode: tangent slot k holds parameter slot_param[k] (-1: none) of
+    // channel k mod 3; mat_slots[m]: the slots of material m's parameters
+    int nd;
+    signed char slot_param[kReplayTangents];
+    unsigned short mat_slots[kGroupMats];
+    unsigned* queue;
 };
 struct TraceLaunch {
     TraceJob job0;            // used when jobs == null (single job, passed by value)
     const TraceJob* jobs;     // packed launch: [njobs] in device memory
     int njobs, total_items;
     int share;                // 1: every job of the launch shares paths (selects the kernel variant)
-    int diff_nd;              // pathwise estimator: tangent slots of the kernel variant (0, 4 or 8)
+    int diff_nd;              // pathwise estimator: tangent slots of the kernel variant (0; k_trace 4, 6, 8;
+                              // k_trace_replay 3, 6, 12)
     int group;                // 1: every job of the launch runs in render-group mode (k_trace_group),
-                              // 2: in emitter-sharing mode (k_trace_emit)
+                              // 2: in replay mode (k_trace_replay)
+    // replay mode, covering every job of the launch: bound materials, perturbed primitives (1 only
+    // black ones, 2 any), float4 of the per-render table, entries of a warp's pool, 32-render
+    // halves of a warp's sums, pixels of a work item at most
+    int replay_mat, replay_move, tab_rows, pool, halves, pixels;
     int fin_total;            // packed launch: finalisation CTAs (sum of R over jobs)
     unsigned* queue;          // work-queue head, zeroed by the instantiation launch
     unsigned long long* counters;  // [8] or null (null: the uncounted kernel variant runs)
@@ -270,18 +294,25 @@ cudaError_t launch_philox(unsigned long long seed, unsigned c0, unsigned c1, uns
 // kDiffBlock threads.
 int trace_blocks_per_sm(bool render_mode);
 int trace_group_blocks_per_sm();
-int trace_emit_blocks_per_sm();
+// Resident CTAs per SM of a replay launch's kernel variant with its shared memory (0: it does
+// not fit).
+int trace_replay_blocks_per_sm(const TraceLaunch& L);
+constexpr int kReplayWarpsPerSm = 20;  // resident warps of the replay kernel
+size_t replay_smem(const TraceLaunch& L);
+int replay_pool(const TraceLaunch& L);  // pool of a launch that needs at least L.pool granules
 constexpr int kGroupBlock = 128;    // render-group CTAs: 4 warps (their per-warp tables fit 48 KB)
-constexpr int kGroupPrims = 16;     // render-group mode: at most 16 primitives ...
-constexpr int kGroupMats = 16;      // ... and 16 materials (the staged copy is smaller)
 constexpr int kGroupTabRows = 192;  // float4 of a warp's per-render record table (render-group mode)
-constexpr int kEmitTabRows = 256;   // float4 of a CTA's per-render record table (emitter-sharing mode)
+constexpr int kReplayTabRows = 1024;  // float4 of a CTA's per-render record table (replay mode), at most
+// Granules (float4) of a warp's pool that one path may need in replay mode with and without
+// perturbed primitives: per vertex a segment (3), emission (1) and estimate (3; without perturbed
+// primitives 1), and one prefix (2).
+constexpr int replay_path_granules(int depth, bool move) { return (move ? 7 : 2) * depth + 2; }
 constexpr int kDiffBlock = 128;
 int trace_diff_blocks_per_sm();
 
-// Pixel block of one warp work item for 8, 16 or 32 pixels.
+// Pixel block of one warp work item for 8, 16 or 32 pixels (replay mode: also 1, 2 or 4).
 inline void block_shape(int pixels, int* bw, int* bh) {
-    *bw = (pixels >= 16) ? 8 : 4;
+    *bw = (pixels >= 16) ? 8 : (pixels < 4 ? pixels : 4);
     *bh = pixels / *bw;
 }
 

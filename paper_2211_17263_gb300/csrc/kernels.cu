@@ -21,6 +21,10 @@
 //                   recorded paths that may meet its own primitives, resuming where
 //                   the renders part, and adds its radiance minus the shared one.
 //   k_shared_epilogue path sharing: the blocks with recorded paths, all renders.
+//   k_trace_group   render groups: the renders of a path sample traced side by side.
+//   k_trace_replay  replay: each path traced once for all renders of a job, recording the
+//                   events that can differ; each render replays them with its own
+//                   primitives, albedos and (Eq. 9) tangents.
 //   k_finalize      one CTA per render: L_r from the block partials (fixed order); the
 //                   CTA completing a job's last render forms the gradient of Eq. 10
 //                   (or the mean of Eq. 9's pathwise gradients) and applies Adam.
@@ -161,7 +165,8 @@ __device__ __forceinline__ float sigma_at(const InstJob& J, int d, int t) {
 // Axis-aligned bounds of a primitive record, inflated by 1e-3 scene units plus 1e-5
 // relative, so that a slab test against them is conservative for the exact FP32
 // intersection tests of the primitive (path sharing).
-__device__ __forceinline__ void prim_bounds(const float4* P, int type, float3& lo, float3& hi) {
+template <class Rec>
+__device__ __forceinline__ void prim_bounds(const Rec& P, int type, float3& lo, float3& hi) {
     if (type == kSphere) {
         const float4 c = P[0];
         const float rad = fabsf(c.w);
@@ -276,6 +281,7 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
         if (L.queue_reset3) *L.queue_reset3 = 0u;
         if (L.queue_reset4) *L.queue_reset4 = 0u;
     }
+    if (r == 0 && tid == 0 && J.queue_reset) *J.queue_reset = 0u;
     if (r == 0 && tid == 0 && J.share_reset)
         for (int i = 0; i < 4; ++i) J.share_reset[i] = 0u;
     if (tid == 0 && J.aff_cursor) J.aff_cursor[r] = 0u;
@@ -439,7 +445,7 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
     if (J.var_box && tid < J.n_var) {  // path sharing: this render's bounds of a perturbed primitive
         const int i = J.var_prim[tid];
         float3 lo, hi;
-        prim_bounds(S.prim[B.prim_slot[i]], B.prim_type[i], lo, hi);
+        prim_bounds(static_cast<const float4*>(S.prim[B.prim_slot[i]]), B.prim_type[i], lo, hi);
         J.var_box[(size_t(r) * kMaxVariant + tid) * 2 + 0] = make_float4(lo.x, lo.y, lo.z, 0.0f);
         J.var_box[(size_t(r) * kMaxVariant + tid) * 2 + 1] = make_float4(hi.x, hi.y, hi.z, 0.0f);
     }
@@ -684,25 +690,29 @@ __device__ __forceinline__ bool occluded(const Scn& S, float3 o, float3 d, float
 // perturbed primitive intervenes, so the lanes stay coherent). The invariant part of the
 // scene is the warp's staged InstScene; each lane reads what differs between renders from
 // its row of a per-warp table:
-//   [4 k .. 4 k + 3]   record of the k-th perturbed primitive (in record-slot order)
-//   [4 n + j]          albedo row (albedo, type) of the j-th bound material (only albedos
-//                      are bound in this mode; the emission row is the staged scene's)
-//   [4 n + m .. + 1]   the render's emitter areas (8 floats), only when a radius binding
-//                      can change an emitter's area (m = bound materials)
+//   [0 .. n - 1]  the rows of the perturbed primitives' records that a position or radius
+//                 binding changes (a quad's centre row; a sphere's and a box's two rows), in
+//                 record-slot order; the other rows are the staged scene's
+//   [n + j]       albedo row (albedo, type) of the j-th bound material (only albedos are bound
+//                 in this mode; the emission row is the staged scene's)
+//   [n + m .. + 1]  the render's emitter areas (8 floats), only when a radius binding can
+//                 change an emitter's area (m = bound materials)
 // A record in a per-render table kept field-major (field j of every render contiguous), so
 // that lanes reading their own renders' fields load consecutive float4 without bank
-// conflicts: field j at p[j * s].
+// conflicts: row j at p[j * s] for the first n rows, in the staged scene's record for the others.
 struct SRec {
     const float4* p;
-    int s;
-    __device__ __forceinline__ float4 operator[](int j) const { return p[j * s]; }
+    int s, n;
+    const float4* base;
+    __device__ __forceinline__ float4 operator[](int j) const { return *(j < n ? p + j * s : base + j); }
 };
 
 struct GroupLane {
     const float4* rec;  // this lane's row: field q at rec[q * rs]
     unsigned prims;     // record-slot mask of the perturbed primitives
     unsigned mats;      // mask of the bound materials
-    int n_var;          // perturbed primitives
+    unsigned offs;      // first field of the k-th perturbed primitive's own rows: bits 8 k .. 8 k + 7
+    int var_rows;       // fields of all of them
     int areas;          // 1: the row holds the emitter areas
     const uint4* rng;   // the sample group's Philox blocks: [0] jitter, [1 + 2 b + k] vertex b, slot k
     int bpre;           // vertices b < bpre have their blocks in `rng`
@@ -714,8 +724,10 @@ struct GroupLane {
 template <bool kGroup, class Scn>
 __device__ __forceinline__ auto prim_rec(const Scn& S, int slot, const GroupLane* g) {
     if constexpr (kGroup) {
-        if ((g->prims >> slot) & 1u) return SRec{g->rec + 4 * __popc(g->prims & ((1u << slot) - 1u)) * g->rs, g->rs};
-        return SRec{S.prim[slot], 1};
+        const bool quad = slot >= S.n_sph && slot < S.n_sph + S.n_quad;
+        const int k = __popc(g->prims & ((1u << slot) - 1u));
+        const bool own = (g->prims >> slot) & 1u;
+        return SRec{g->rec + ((g->offs >> (8 * k)) & 255u) * g->rs, g->rs, own ? (quad ? 1 : 2) : 0, S.prim[slot]};
     } else {
         return static_cast<const float4*>(S.prim[slot]);
     }
@@ -725,7 +737,7 @@ __device__ __forceinline__ auto prim_rec(const Scn& S, int slot, const GroupLane
 template <bool kGroup, class Scn>
 __device__ __forceinline__ float4 mat_albedo(const Scn& S, int m, const GroupLane* g) {
     if constexpr (kGroup) {
-        if ((g->mats >> m) & 1u) return g->rec[(4 * g->n_var + __popc(g->mats & ((1u << m) - 1u))) * g->rs];
+        if ((g->mats >> m) & 1u) return g->rec[(g->var_rows + __popc(g->mats & ((1u << m) - 1u))) * g->rs];
     }
     return S.mat[m][0];
 }
@@ -734,7 +746,7 @@ template <bool kGroup, class Scn>
 __device__ __forceinline__ float light_area(const Scn& S, int li, const GroupLane* g) {
     if constexpr (kGroup) {
         if (g->areas)
-            return reinterpret_cast<const float*>(g->rec + (4 * g->n_var + __popc(g->mats) + (li >> 2)) * g->rs)[li & 3];
+            return reinterpret_cast<const float*>(g->rec + (g->var_rows + __popc(g->mats) + (li >> 2)) * g->rs)[li & 3];
     }
     return S.light_area[li];
 }
@@ -746,22 +758,23 @@ __device__ __forceinline__ void group_hit(const Scn& S, const GroupLane& g, floa
                                           Counters& cnt) {
     const float3 inv = rcp3(d);
     unsigned m = g.prims;
-    for (int k = 0; m; ++k) {
+#pragma unroll 1
+    for (unsigned offs = g.offs; m; offs >>= 8) {
         const int slot = __ffs(m) - 1;
         m &= m - 1u;
-        const SRec P{g.rec + 4 * k * g.rs, g.rs};
+        const float4* own = g.rec + (offs & 255u) * g.rs;
         float t;
         int type;
         if (slot < S.n_sph) {
-            t = sphere_t(P, o, d);
+            t = sphere_t(SRec{own, g.rs, 2, S.prim[slot]}, o, d);
             type = kSphere;
             if (kCount) ++cnt.sph;
         } else if (slot < S.n_sph + S.n_quad) {
-            t = quad_any_t(P, o, d, inv);
+            t = quad_any_t(SRec{own, g.rs, 1, S.prim[slot]}, o, d, inv);
             type = kQuad;
             if (kCount) ++cnt.quad;
         } else {
-            t = box_t(P, o, inv);
+            t = box_t(SRec{own, g.rs, 2, S.prim[slot]}, o, inv);
             type = kBox;
             if (kCount) ++cnt.box;
         }
@@ -775,20 +788,21 @@ __device__ __forceinline__ bool group_occluded(const Scn& S, const GroupLane& g,
                                                int light, Counters& cnt) {
     const float3 inv = rcp3(d);
     unsigned m = g.prims;
-    for (int k = 0; m; ++k) {
+#pragma unroll 1
+    for (unsigned offs = g.offs; m; offs >>= 8) {
         const int slot = __ffs(m) - 1;
         m &= m - 1u;
+        const float4* own = g.rec + (offs & 255u) * g.rs;
         if (slot == light) continue;
-        const SRec P{g.rec + 4 * k * g.rs, g.rs};
         float t;
         if (slot < S.n_sph) {
-            t = sphere_t(P, o, d);
+            t = sphere_t(SRec{own, g.rs, 2, S.prim[slot]}, o, d);
             if (kCount) ++cnt.sph;
         } else if (slot < S.n_sph + S.n_quad) {
-            t = quad_any_t(P, o, d, inv);
+            t = quad_any_t(SRec{own, g.rs, 1, S.prim[slot]}, o, d, inv);
             if (kCount) ++cnt.quad;
         } else {
-            t = box_t(P, o, inv);
+            t = box_t(SRec{own, g.rs, 2, S.prim[slot]}, o, inv);
             if (kCount) ++cnt.box;
         }
         if (t < dist) return true;
@@ -996,22 +1010,22 @@ __device__ __forceinline__ void tan_reset(Tangents<kND>& t) {
 }
 
 // L += beta * E (background or emitter seen on a camera or specular ray); E may be bound.
-template <int kND, class Scn>
-__device__ __forceinline__ void tan_emit(Tangents<kND>& t, const TraceJob& J, const Scn& S, float3 beta,
+template <int kND, class Clamp>
+__device__ __forceinline__ void tan_emit(Tangents<kND>& t, const TraceJob& J, const Clamp& dclamp, float3 beta,
                                          float3 E, int mat) {
 #pragma unroll
     for (int k = 0; k < kND; ++k) {
         if (k >= J.diff_n) break;
         const int c = J.diff_comp[k];
         float d = t.dB[k] * comp3(E, c);
-        if (J.diff_kind[k] == kBindEmission && J.diff_mat[k] == mat) d = fmaf(comp3(beta, c), S.dclamp[k], d);
+        if (J.diff_kind[k] == kBindEmission && J.diff_mat[k] == mat) d = fmaf(comp3(beta, c), dclamp[k], d);
         t.dL[k] += d;
     }
 }
 
 // L += beta * albedo * Le * g (next-event estimation at a vertex of material mat).
-template <int kND, class Scn>
-__device__ __forceinline__ void tan_nee(Tangents<kND>& t, const TraceJob& J, const Scn& S, float3 beta,
+template <int kND, class Clamp>
+__device__ __forceinline__ void tan_nee(Tangents<kND>& t, const TraceJob& J, const Clamp& dclamp, float3 beta,
                                         float3 albedo, int mat, float3 Le, int lmat, float g) {
 #pragma unroll
     for (int k = 0; k < kND; ++k) {
@@ -1019,22 +1033,22 @@ __device__ __forceinline__ void tan_nee(Tangents<kND>& t, const TraceJob& J, con
         const int c = J.diff_comp[k];
         const float bc = comp3(beta, c), rc = comp3(albedo, c), ec = comp3(Le, c);
         float d = t.dB[k] * rc * ec;
-        if (J.diff_kind[k] == kBindAlbedo && J.diff_mat[k] == mat) d = fmaf(bc * S.dclamp[k], ec, d);
-        if (J.diff_kind[k] == kBindEmission && J.diff_mat[k] == lmat) d = fmaf(bc * rc, S.dclamp[k], d);
+        if (J.diff_kind[k] == kBindAlbedo && J.diff_mat[k] == mat) d = fmaf(bc * dclamp[k], ec, d);
+        if (J.diff_kind[k] == kBindEmission && J.diff_mat[k] == lmat) d = fmaf(bc * rc, dclamp[k], d);
         t.dL[k] = fmaf(d, g, t.dL[k]);
     }
 }
 
 // beta <- beta * albedo (scattering at a vertex of material mat); beta is the old value.
-template <int kND, class Scn>
-__device__ __forceinline__ void tan_scatter(Tangents<kND>& t, const TraceJob& J, const Scn& S, float3 beta,
+template <int kND, class Clamp>
+__device__ __forceinline__ void tan_scatter(Tangents<kND>& t, const TraceJob& J, const Clamp& dclamp, float3 beta,
                                             float3 albedo, int mat) {
 #pragma unroll
     for (int k = 0; k < kND; ++k) {
         if (k >= J.diff_n) break;
         const int c = J.diff_comp[k];
         float d = t.dB[k] * comp3(albedo, c);
-        if (J.diff_kind[k] == kBindAlbedo && J.diff_mat[k] == mat) d = fmaf(comp3(beta, c), S.dclamp[k], d);
+        if (J.diff_kind[k] == kBindAlbedo && J.diff_mat[k] == mat) d = fmaf(comp3(beta, c), dclamp[k], d);
         t.dB[k] = d;
     }
 }
@@ -1063,6 +1077,7 @@ __device__ __forceinline__ bool occluded_set(const Scn& S, float3 o, float3 d, f
     if (kCount) ++cnt.shadow;
     const int ns = S.n_sph, nsq = S.n_sph + S.n_quad;
     const float3 inv = rcp3(d);
+#pragma unroll 1
     while (cand) {
         const int i = __ffs(cand) - 1;
         cand &= cand - 1u;
@@ -1116,7 +1131,7 @@ __device__ __forceinline__ bool nee_to(const Scn& S, float3 po, float3 ns, float
         const int np = S.n_sph + S.n_quad + S.n_box;
         const unsigned all = np >= 32 ? 0xffffffffu : (1u << np) - 1u;
         blocked = occluded_set<kCount>(S, po, wi, dist, all & ~(gl->prims | skip | (1u << lt.y)), cnt) ||
-                  group_occluded<kCount>(S, *gl, po, wi, dist, lt.y, cnt);
+                  ((gl->prims & ~(1u << lt.y)) != 0u && group_occluded<kCount>(S, *gl, po, wi, dist, lt.y, cnt));
     } else {
         blocked = occluded<kCount, kShared>(S, po, wi, dist, lt.y, cnt, skip);
     }
@@ -1139,100 +1154,71 @@ __device__ __forceinline__ bool nee_visible(const Scn& S, float3 po, float3 ns, 
 __device__ __forceinline__ float3 nee_add(float3 L, float3 ba, float3 Le, float g) { return L + ba * Le * g; }
 __device__ __forceinline__ float3 bg_add(float3 L, float3 beta, float3 bg) { return L + beta * bg; }
 
-// Emitter-sharing mode (k_trace_emit): a path is traced once in the invariant scene for all
-// renders; its diffuse vertices are kept (up to kEmitCap) so that each render evaluates its
-// own next-event estimate there, and a path whose ray could meet a perturbed primitive (its
-// segment touches their union bounds) stops so that each render traces it on from there.
-#ifndef PRDPT_EMIT_CAP
-#define PRDPT_EMIT_CAP 2
-#endif
-constexpr int kEmitCap = PRDPT_EMIT_CAP;  // diffuse vertices kept per path
-constexpr int kEmitFields = 13;  // po, ns, beta * albedo, the emitter point (lu, lv), emitter li, cull mask
-struct EmitLane {
-    const float4* ulo;  // union over the renders of each perturbed primitive's bounds
-    const float4* uhi;
-    int n_var;
-    unsigned skip;      // record slots of the perturbed primitives
-    float* ent;         // the warp's kept vertices: ent[(k * kEmitFields + field) * 32 + lane]
-    int lane;
-    int n;              // vertices kept by this lane's path
-    bool miss;          // the path ended by leaving the scene
-};
-
-// Invariant primitives that no render's shadow ray from po to its emitter li can meet, as a
-// record-slot mask: every such ray lies
-// in the cone from po over the emitter's union bounds (centre b, half-diagonal rb: the ray
-// to a point y deviates from the axis po -> b by at most t rb at parameter t). A primitive
-// is left out when its bounding sphere (a sphere itself; a quad's or box's enclosing one)
-// keeps clear of that cone, or when a quad's plane has po and the whole union box strictly
-// on one side. The margins exceed the FP32 rounding of the intersection tests, so leaving
-// these primitives out never changes a shadow ray's outcome.
-template <class Scn>
-__device__ __forceinline__ unsigned shadow_cull(const Scn& S, const EmitLane& E, float3 po, int li) {
-    const int slot = S.light[li].y;
-    if (!((E.skip >> slot) & 1u)) return 0u;
-    const int k = __popc(E.skip & ((1u << slot) - 1u));
-    const float3 lo = xyz(E.ulo[k]), hi = xyz(E.uhi[k]);
-    const float3 bc = (lo + hi) * 0.5f, bh = (hi - lo) * 0.5f;
-    const float rb = sqrtf(dot3(bh, bh));
-    const float3 v = bc - po;
-    const float vv = dot3(v, v), lv = sqrtf(vv);
-    unsigned m = 0u;
-    const int ns = S.n_sph, nq = S.n_quad, np = ns + nq + S.n_box;
-    for (int i = 0; i < np; ++i) {
-        if ((E.skip >> i) & 1u) continue;
-        const float4* P = S.prim[i];
-        float3 c;
-        float rad;
-        if (i < ns) {
-            c = xyz(P[0]);
-            rad = fabsf(P[0].w);
-        } else if (i < ns + nq) {
-            c = xyz(P[0]);
-            const float3 n = xyz(P[1]), pc = po - c;
-            const float mg = (1e-5f + 2e-6f * sqrtf(dot3(pc, pc))) * sqrtf(dot3(n, n));
-            const float sp = dot3(pc, n), sb = dot3(bc - c, n);
-            const float eb = fabsf(n.x) * bh.x + fabsf(n.y) * bh.y + fabsf(n.z) * bh.z;
-            if ((sp > mg && sb - eb > mg) || (sp < -mg && sb + eb < -mg)) {
-                m |= 1u << i;
-                continue;
-            }
-            const float3 u = xyz(P[2]), w = xyz(P[3]);
-            rad = 0.5f * (sqrtf(dot3(u, u)) + sqrtf(dot3(w, w)));
-        } else {
-            const float3 a = xyz(P[0]), b = xyz(P[1]);
-            c = (a + b) * 0.5f;
-            const float3 e = (b - a) * 0.5f;
-            rad = sqrtf(dot3(e, e));
-        }
-        const float R = rad + 1e-3f + 1e-5f * (fabsf(c.x) + fabsf(c.y) + fabsf(c.z));
-        const float3 w = c - po;
-        const float t0 = vv > 0.0f ? dot3(w, v) / vv : 0.0f;
-        const float tc = fminf(fmaxf(t0, 0.0f), 1.0f);
-        const float3 q = w - v * tc;
-        const float dc = sqrtf(dot3(q, q));
-        const float thi = lv > 0.0f ? fminf(1.0f, t0 + (R + rb) / lv) : 1.0f;
-        if (dc > R + fmaxf(thi, 0.0f) * rb) m |= 1u << i;
+// Normal and material of the hit at pt (surfaces' own orientation).
+template <class Rec>
+__device__ __forceinline__ float3 surface_normal(const Rec& P, int type, float3 pt, float3 o, float3 d, int& mat) {
+    float3 ng;
+    if (type == kSphere) {
+        const float4 a = P[0];
+        ng = (pt - xyz(a)) * P[1].y;
+        mat = as_int(P[1].z);
+    } else if (type == kQuad) {
+        ng = xyz(P[1]);
+        mat = as_int(P[0].w) & 255;
+    } else {
+        ng = box_normal(P, o, d, rcp3(d));
+        mat = as_int(P[0].w) & 255;
     }
-    return m;
+    return ng;
 }
 
-// Does the segment o + t d, 0 <= t <= tmax, touch a union box of the perturbed primitives?
-template <bool kCount>
-__device__ __forceinline__ bool emit_touch(const EmitLane& E, float3 o, float3 d, float tmax, Counters& cnt) {
-    const float3 inv = rcp3(d);
-    const float tm = tmax * 1.0001f + 1e-3f;
-    bool hit = false;
-    for (int k = 0; k < E.n_var; ++k) hit = hit || slab_touch(xyz(E.ulo[k]), xyz(E.uhi[k]), o, inv, tm);
-    if (kCount) cnt.box += E.n_var;
-    return hit;
+// Cosine-distributed direction around ns (not normalised to the last bit).
+__device__ __forceinline__ float3 diffuse_dir(float3 ns, float u1, float u2) {
+    const float rad = u1 * rsqrt_fast(u1);
+    float sp, cp;
+    sincospif(2.0f * u2, &sp, &cp);
+    float3 t1, t2;
+    onb(ns, t1, t2);
+    const float cz2 = fmaxf(0.0f, 1.0f - u1);
+    return t1 * (rad * cp) + t2 * (rad * sp) + ns * (cz2 * rsqrt_fast(fmaxf(cz2, 1e-30f)));
 }
 
-template <bool kCount, bool kShared, int kND = 0, bool kGroup = false, bool kEmit = false, class Scn>
+// Smooth dielectric (exact unpolarised Fresnel): reflect or refract the path's ray at pt.
+__device__ __forceinline__ void dielectric(Path& p, float3 pt, float3 ng, float ior, float u) {
+    float ci = -dot3(p.d, ng);
+    float eta;
+    float3 n;
+    if (ci > 0.0f) {
+        eta = rcp_fast(ior);
+        n = ng;
+    } else {
+        eta = ior;
+        n = ng * -1.0f;
+        ci = -ci;
+    }
+    const float s2t = eta * eta * (1.0f - ci * ci);
+    float F, ct = 0.0f;
+    if (s2t >= 1.0f) {
+        F = 1.0f;
+    } else {
+        ct = sqrtf(1.0f - s2t);
+        const float rs = div_fast(eta * ci - ct, eta * ci + ct);
+        const float rp = div_fast(ci - eta * ct, ci + eta * ct);
+        F = 0.5f * (rs * rs + rp * rp);
+    }
+    if (u < F) {
+        p.d = normalized(p.d + n * (2.0f * ci));
+        p.o = pt + n * kEps;
+    } else {
+        p.d = normalized(p.d * eta + n * (eta * ci - ct));
+        p.o = pt - n * kEps;
+    }
+}
+
+template <bool kCount, bool kShared, int kND = 0, bool kGroup = false, class Scn>
 __device__ __forceinline__ int advance(const Scn& S, int depth, int rr_start, Path& p, Counters& cnt,
                                        const VarBoxes* V = nullptr, Tangents<kND>* tn = nullptr,
-                                       const TraceJob* Jd = nullptr, const GroupLane* gl = nullptr,
-                                       EmitLane* el = nullptr) {
+                                       const TraceJob* Jd = nullptr, const GroupLane* gl = nullptr) {
     if (kShared && p.seg == 0u) {
         const int t = threadIdx.x;
         s_stash[0][t] = p.o.x;
@@ -1243,10 +1229,7 @@ __device__ __forceinline__ int advance(const Scn& S, int depth, int rr_start, Pa
         s_stash[5][t] = p.d.z;
     }
     Hit h;
-    if constexpr (kEmit) {  // the invariant scene; a ray that could meet a perturbed primitive stops here
-        h = closest_hit<kCount, true>(S, p.o, p.d, cnt, el->skip);
-        if (emit_touch<kCount>(*el, p.o, p.d, h.slot < 0 ? 3.0e38f : h.t, cnt)) return kAffected;
-    } else if constexpr (kGroup) {  // the staged scene without the perturbed primitives, then the lane's own
+    if constexpr (kGroup) {  // the staged scene without the perturbed primitives, then the lane's own
         h = closest_hit<kCount, true>(S, p.o, p.d, cnt, gl->prims);
         group_hit<kCount>(S, *gl, p.o, p.d, h, cnt);
     } else {
@@ -1257,30 +1240,15 @@ __device__ __forceinline__ int advance(const Scn& S, int depth, int rr_start, Pa
         if (p.seg & kSegAll) return kAffected;
     }
     if (h.slot < 0) {
-        if constexpr (kEmit) {
-            el->miss = true;  // the background term is added per render, after its vertex terms
-            return kEnded;
-        }
-        if (kND > 0) tan_emit(*tn, *Jd, S, p.beta, xyz(S.bg), -1);
+        if (kND > 0) tan_emit(*tn, *Jd, S.dclamp, p.beta, xyz(S.bg), -1);
         p.L = bg_add(p.L, p.beta, xyz(S.bg));
         return kEnded;
     }
     if (kCount) ++cnt.vertices;
     const float3 pt = p.o + p.d * h.t;
     const auto P = prim_rec<kGroup>(S, h.slot, gl);
-    float3 ng;
     int mat;
-    if (h.type == kSphere) {
-        const float4 a = P[0];
-        ng = (pt - xyz(a)) * P[1].y;
-        mat = as_int(P[1].z);
-    } else if (h.type == kQuad) {
-        ng = xyz(P[1]);
-        mat = as_int(P[0].w) & 255;
-    } else {
-        ng = box_normal(P, p.o, p.d, rcp3(p.d));
-        mat = as_int(P[0].w) & 255;
-    }
+    const float3 ng = surface_normal(P, h.type, pt, p.o, p.d, mat);
     if (kShared && ((V->mats >> mat) & 1u)) {  // every render from here (state: this vertex)
         p.seg = (p.seg == 0u ? open_group<false>(*V, p) : p.seg) | kSegAll;
         return kAffected;
@@ -1291,8 +1259,7 @@ __device__ __forceinline__ int advance(const Scn& S, int depth, int rr_start, Pa
     float3 albedo = xyz(m0);
     if (mat == S.tex_mat && h.type == kQuad) albedo = tex_albedo(S, P, pt);
     if (p.specular && (emission.x > 0.f || emission.y > 0.f || emission.z > 0.f) && dot3(p.d, ng) < 0.0f) {
-        if constexpr (kEmit) return kAffected;  // an invariant emitter: not in this mode's jobs
-        if (kND > 0) tan_emit(*tn, *Jd, S, p.beta, emission, mat);
+        if (kND > 0) tan_emit(*tn, *Jd, S.dclamp, p.beta, emission, mat);
         p.L = p.L + p.beta * emission;
     }
     const bool last = (p.b + 1 >= depth);
@@ -1301,91 +1268,44 @@ __device__ __forceinline__ int advance(const Scn& S, int depth, int rr_start, Pa
     if (mtype == kDiffuse) {
         const float3 ns = dot3(ng, p.d) < 0.0f ? ng : ng * -1.0f;
         const float3 po = pt + ns * kEps;
-        const uint4 w0 = vertex_words<kGroup, kGroup || kEmit>(S, p, 0, gl);
-        if (S.n_lights > 1 || rr) w1 = vertex_words<kGroup, kGroup || kEmit>(S, p, 1, gl);
+        const uint4 w0 = vertex_words<kGroup, kGroup>(S, p, 0, gl);
+        if (S.n_lights > 1 || rr) w1 = vertex_words<kGroup, kGroup>(S, p, 1, gl);
         if (S.n_lights > 0) {  // next-event estimation: one emitter, uniform area sample
-            if constexpr (kEmit) {  // kept for the renders' own estimates (the renders' emitters differ)
-                if (el->n == kEmitCap) return kAffected;
-                float* e = el->ent + el->n * kEmitFields * 32 + el->lane;
-                const float3 ba = p.beta * albedo;
-                e[0] = po.x; e[32] = po.y; e[64] = po.z;
-                e[96] = ns.x; e[128] = ns.y; e[160] = ns.z;
-                e[192] = ba.x; e[224] = ba.y; e[256] = ba.z;
-                const int li = nee_light(S, w1.x);
-                e[288] = u01(w0.x); e[320] = u01(w0.y); e[352] = __int_as_float(li);
-                e[384] = __uint_as_float(shadow_cull(S, *el, po, li));
-                ++el->n;
-            } else {
-                float3 wi;
-                float dist, g;
-                int lmat;
-                if (nee_visible<kCount, kShared, kGroup>(S, po, ns, w0.x, w0.y, w1.x, cnt, kShared ? V->skip : 0u, gl,
-                                                         wi, dist, g, lmat)) {
-                    if (kShared) {
-                        note_touch<kCount, true>(*V, po, wi, dist, p, cnt);
-                        if (p.seg & kSegAll) return kAffected;
-                    }
-                    const float3 Le = xyz(S.mat[lmat][1]);
-                    if (kND > 0) tan_nee(*tn, *Jd, S, p.beta, albedo, mat, Le, lmat, g);
-                    p.L = nee_add(p.L, p.beta * albedo, Le, g);
+            float3 wi;
+            float dist, g;
+            int lmat;
+            if (nee_visible<kCount, kShared, kGroup>(S, po, ns, w0.x, w0.y, w1.x, cnt, kShared ? V->skip : 0u, gl,
+                                                     wi, dist, g, lmat)) {
+                if (kShared) {
+                    note_touch<kCount, true>(*V, po, wi, dist, p, cnt);
+                    if (p.seg & kSegAll) return kAffected;
                 }
+                const float3 Le = xyz(S.mat[lmat][1]);
+                if (kND > 0) tan_nee(*tn, *Jd, S.dclamp, p.beta, albedo, mat, Le, lmat, g);
+                p.L = nee_add(p.L, p.beta * albedo, Le, g);
             }
         }
         if (last) return kEnded;
-        const float u1 = u01(w0.z), u2 = u01(w0.w);
-        const float rad = u1 * rsqrt_fast(u1);
-        float sp, cp;
-        sincospif(2.0f * u2, &sp, &cp);
-        float3 t1, t2;
-        onb(ns, t1, t2);
-        const float cz2 = fmaxf(0.0f, 1.0f - u1);
-        const float3 wo = t1 * (rad * cp) + t2 * (rad * sp) + ns * (cz2 * rsqrt_fast(fmaxf(cz2, 1e-30f)));
-        if (kND > 0) tan_scatter(*tn, *Jd, S, p.beta, albedo, mat);
+        const float3 wo = diffuse_dir(ns, u01(w0.z), u01(w0.w));
+        if (kND > 0) tan_scatter(*tn, *Jd, S.dclamp, p.beta, albedo, mat);
         p.beta = p.beta * albedo;
         p.o = po;
         p.d = normalized(wo);
         p.specular = false;
     } else if (mtype == kMirror) {
         if (last) return kEnded;
-        if (rr) w1 = vertex_words<kGroup, kGroup || kEmit>(S, p, 1, gl);
+        if (rr) w1 = vertex_words<kGroup, kGroup>(S, p, 1, gl);
         const float3 ns = dot3(ng, p.d) < 0.0f ? ng : ng * -1.0f;
         p.d = normalized(p.d - ns * (2.0f * dot3(p.d, ns)));
         p.o = pt + ns * kEps;
-        if (kND > 0) tan_scatter(*tn, *Jd, S, p.beta, albedo, mat);
+        if (kND > 0) tan_scatter(*tn, *Jd, S.dclamp, p.beta, albedo, mat);
         p.beta = p.beta * albedo;
         p.specular = true;
     } else {  // smooth dielectric: exact unpolarised Fresnel, reflect or refract
         if (last) return kEnded;
-        w1 = vertex_words<kGroup, kGroup || kEmit>(S, p, 1, gl);
-        float ci = -dot3(p.d, ng);
-        float eta;
-        float3 n;
-        if (ci > 0.0f) {
-            eta = rcp_fast(m1.w);
-            n = ng;
-        } else {
-            eta = m1.w;
-            n = ng * -1.0f;
-            ci = -ci;
-        }
-        const float s2t = eta * eta * (1.0f - ci * ci);
-        float F, ct = 0.0f;
-        if (s2t >= 1.0f) {
-            F = 1.0f;
-        } else {
-            ct = sqrtf(1.0f - s2t);
-            const float rs = div_fast(eta * ci - ct, eta * ci + ct);
-            const float rp = div_fast(ci - eta * ct, ci + eta * ct);
-            F = 0.5f * (rs * rs + rp * rp);
-        }
-        if (u01(w1.z) < F) {
-            p.d = normalized(p.d + n * (2.0f * ci));
-            p.o = pt + n * kEps;
-        } else {
-            p.d = normalized(p.d * eta + n * (eta * ci - ct));
-            p.o = pt - n * kEps;
-        }
-        if (kND > 0) tan_scatter(*tn, *Jd, S, p.beta, albedo, mat);
+        w1 = vertex_words<kGroup, kGroup>(S, p, 1, gl);
+        dielectric(p, pt, ng, m1.w, u01(w1.z));
+        if (kND > 0) tan_scatter(*tn, *Jd, S.dclamp, p.beta, albedo, mat);
         p.beta = p.beta * albedo;
         p.specular = true;
     }
@@ -1961,18 +1881,17 @@ __global__ void __launch_bounds__(kGroupBlock, kGroupMinBlocks) k_trace_group(co
         }
         if (g != cur_item_g) {  // stage render g G's scene and the group's per-render records
             stage_group_scene(W.scene, J, g * G, lane);
-            const int n = J.n_var, nm = __popc(J.var_mats);
+            const int n = J.var_rows, nm = __popc(J.var_mats);
             for (int i = lane; i < G * stride; i += 32) {
                 const int gi = i / stride, q = i - gi * stride;
                 const InstScene& R = J.scenes[g * G + gi];
                 float4 v;
-                if (q < 4 * n) {  // record of the (q / 4)-th perturbed primitive
-                    const int slot = nth_set_bit(J.var_prims, q >> 2);
-                    v = __ldg(&R.prim[slot][q & 3]);
-                } else if (q < 4 * n + nm) {  // albedo row of a bound material
-                    v = __ldg(&R.mat[nth_set_bit(J.var_mats, q - 4 * n)][0]);
+                if (q < n) {  // own row of a perturbed primitive
+                    v = __ldg(&R.prim[J.row_src[q] >> 1][J.row_src[q] & 1]);
+                } else if (q < n + nm) {  // albedo row of a bound material
+                    v = __ldg(&R.mat[nth_set_bit(J.var_mats, q - n)][0]);
                 } else {  // emitter areas
-                    v = __ldg(reinterpret_cast<const float4*>(R.light_area) + (q - 4 * n - nm));
+                    v = __ldg(reinterpret_cast<const float4*>(R.light_area) + (q - n - nm));
                 }
                 W.tab[q * G + gi] = v;  // field-major: the lanes' loads of one field are contiguous
             }
@@ -1984,8 +1903,8 @@ __global__ void __launch_bounds__(kGroupBlock, kGroupMinBlocks) k_trace_group(co
         // blocks, so the group's lanes draw them ahead, one block each: the jitter and
         // slots 0 and 1 of vertices b < bpre.
         const int bpre = (G - 1) >> 1;
-        const GroupLane gl{W.tab + gi, J.var_prims, J.var_mats, J.n_var,
-                           stride > 4 * J.n_var + __popc(J.var_mats) ? 1 : 0, W.rng + ks * G, bpre, G};
+        const GroupLane gl{W.tab + gi, J.var_prims, J.var_mats, J.var_offs, J.var_rows,
+                           stride > J.var_rows + __popc(J.var_mats) ? 1 : 0, W.rng + ks * G, bpre, G};
         const unsigned gmask = G == 32 ? kFull : ((1u << G) - 1u) << (ks * G);
         const int x0 = (t % J.tiles_x) * J.bw, y0 = (t / J.tiles_x) * J.bh;
         const int vw = min(J.bw, J.W - x0), vh = min(J.bh, J.H - y0);
@@ -2040,292 +1959,952 @@ __global__ void __launch_bounds__(kGroupBlock, kGroupMinBlocks) k_trace_group(co
     }
 }
 
-// ---------------------------------------------------------------------------
-// k_trace_emit: emitter-sharing variant of the per-render kernel (a3-a5)
-// ---------------------------------------------------------------------------
-// For a job whose perturbed primitives include every emitter and whose materials are not
-// bound (e.g. a moving light): under common random numbers the renders' paths agree until
-// one of their rays could meet a perturbed primitive, and differ before that only in the
-// next-event estimates. A work item is one pixel block of all R <= 64 renders, taken by a
-// CTA of kEmitWarps warps; warp w takes the pixel slots of positions q = 8w .. 8w + 7 of
-// the bit-reversed order. For each pixel, 32 samples at a time:
-//   phase A  lane = sample: the path is traced once in the invariant scene, keeping its
-//            diffuse vertices (EmitLane) and its end: left the scene (the background term),
-//            ended, or stopped where a ray could meet a perturbed primitive;
-//   phase B  lane = render (lane and lane + 32; with R <= 16, render lane mod G of sample
-//            group lane / G, G the power of two >= R): for each sample that adds anything,
-//            the render's own next-event estimates at the kept vertices (occlusion tested
-//            against the primitives the vertex's cull mask leaves), then the background term
-//            or, for a stopped path, the rest of the path traced in the render's scene (as in
-//            k_trace_group).
-// Each render's radiance is the same sum, term by term and in the same order, as tracing
-// the path in that render alone, so with the same block shape every partial is
-// bit-identical to the per-render kernel's; the warps' subtrees of the pairwise pixel sum
-// are combined as that sum's top two levels.
-constexpr int kEmitWarps = kGroupBlock / 32;
-constexpr int kEmitTab = kEmitTabRows;
-static_assert(32 % kEmitWarps == 0, "each warp takes 32 / kEmitWarps pixel slots");
-constexpr int kEmitSlots = 32 / kEmitWarps;
-static_assert(kEmitSlots == 8, "the warps' subtrees are the pairwise sum's levels 0-2");
+// Replay mode (k_trace_replay): a path is traced once in the invariant scene for all renders.
+// What is the same in every render -- the path up to its first event that can differ -- is its
+// lane's own radiance; from there on the path is recorded as a chain of groups of entries (one
+// group per vertex) in a per-warp pool of float4 granules, which every render replays with its
+// own primitives and albedos. The first granule's w is the entry's info word:
+//   bits 0-1 kind, 16: last entry of its group
+//   kVert      a vertex: bits 2-3 the next-event estimate, 4 Russian roulette, 5-7 light, 8-11
+//              material, 12-15 surface slot, 17 flipped normal, 18 normal kept in full, 19-31 the
+//              estimate's cull mask. With bound materials (throughput replayed per render):
+//                0 none                (-, u_rr, -, info)
+//                1 perturbed emitter   (po, info) (light u, v, u_rr, -) [(ns, -)]: each render's
+//                                      own point on it, occlusion and geometry term
+//                2 fixed emitter       (g, u_rr, -, info): seen by every render
+//                3 fixed emitter       (po, info) (wi, distance) (g, u_rr, -, -): the render's own
+//                                      primitives may hide it
+//              without: 1 (po, info) (ba, light u) (ns, light v), 2 (-, info) - (ba, g),
+//              3 (po, info) (wi, distance) (ba, g), with ba = beta * albedo
+//   kSegment   a ray that could meet a perturbed primitive: (o, info) (d, t) [(beta, -) without
+//              bound materials], t the invariant scene's closest hit; bit 4 emission counts, 8-14
+//              vertex index. A render whose own primitive is closer parts from the path here
+//   kEmission  emission seen on a camera or specular ray: (beta, info), bits 8-11 material, 5 the
+//              background
+//   kPrefix    radiance (and throughput) before the first entry: (L, info) [(beta, -)]
+enum : unsigned { kVert = 0u, kSegment = 1u, kEmission = 2u, kPrefix = 3u };
+constexpr unsigned kLastEntry = 1u << 16;
+constexpr int kNoEntry = 0xffff;  // end of a chain
+constexpr int kCullBits = 13;
 
-struct EmitWarp {
-    float ent[kEmitCap * kEmitFields * 32];  // kept vertices of the warp's 32 paths
-    float st[10][32];                        // end state: o, d, beta, vertex b (bits)
-    int n[32];                               // vertices kept
-    int kind[32];                            // 0 ended, 1 left the scene, 2 stopped (specular flag: 4)
-    double pair[2][3][32];                   // pairwise-sum stacks of the lane's two renders
+struct ReplayLane {
+    const float4* ulo;   // union over the renders of each perturbed primitive's bounds
+    const float4* uhi;
+    const float4* amax;  // per bound material: the largest albedo over the renders
+    const float4* ball;  // per record slot: an enclosing ball, inflated
+    int n_var;
+    unsigned skip;       // record slots of the perturbed primitives
+    unsigned mats;       // bound materials
+    float4* ent;         // the warp's pool
+    unsigned short* nxt; // per group (its first granule): the chain's next group
+    unsigned* ctr;       // granules claimed
+    int cap;
+    int first, last;     // this lane's chain
+    bool rec;            // recording (the renders may differ from here on)
+    bool varied;         // a bound material was met: p.beta is an upper bound over the renders
+    bool full;           // the pool ran out: the path is traced again in a later batch
 };
-struct EmitSmem {
+
+// Enclosing ball of a primitive record, inflated beyond the FP32 rounding of its test.
+__device__ __forceinline__ float4 prim_ball(const float4* P, int type) {
+    float3 c;
+    float rad;
+    if (type == kSphere) {
+        c = xyz(P[0]);
+        rad = fabsf(P[0].w);
+    } else if (type == kQuad) {
+        const float3 u = xyz(P[2]), w = xyz(P[3]);
+        c = xyz(P[0]);
+        rad = 0.5f * (sqrtf(dot3(u, u)) + sqrtf(dot3(w, w)));
+    } else {
+        const float3 a = xyz(P[0]), b = xyz(P[1]), e = (b - a) * 0.5f;
+        c = (a + b) * 0.5f;
+        rad = sqrtf(dot3(e, e));
+    }
+    return make_float4(c.x, c.y, c.z, rad * 1.00001f + 1e-3f + 1e-5f * (fabsf(c.x) + fabsf(c.y) + fabsf(c.z)));
+}
+
+// Invariant primitives that no render's shadow ray from po to its emitter in record slot `slot`
+// can meet, as a mask of the first kCullBits record slots: every such ray lies in the cone from
+// po over the emitter's union bounds (centre b, half-diagonal rb: the ray to a point y deviates
+// from the axis po -> b by at most t rb at parameter t). A primitive is left out when its
+// enclosing ball keeps clear of that cone, or when a quad's plane has po and the whole union
+// box strictly on one side. The margins exceed the FP32 rounding of the intersection tests and
+// of the approximate roots and quotients here, so leaving these primitives out never changes a
+// shadow ray's outcome.
+__device__ __forceinline__ unsigned shadow_cull(const GroupScene& S, const ReplayLane& E, float3 po, int slot) {
+    const int k = __popc(E.skip & ((1u << slot) - 1u));
+    const float3 lo = xyz(E.ulo[k]), hi = xyz(E.uhi[k]);
+    const float3 bc = (lo + hi) * 0.5f, bh = (hi - lo) * 0.5f;
+    const float bb = dot3(bh, bh), rb = bb * rsqrt_fast(bb) * 1.0001f;  // the bounds are inflated: bb > 0
+    const float3 v = bc - po;
+    const float vv = dot3(v, v);
+    if (!(vv > 1e-12f)) return 0u;
+    const float ilv = rsqrt_fast(vv) * 1.0001f, ivv = rcp_fast(vv);
+    unsigned m = 0u;
+    const int ns = S.n_sph, nq = S.n_quad, np = min(ns + nq + S.n_box, kCullBits);
+#pragma unroll 1
+    for (int i = 0; i < np; ++i) {
+        if ((E.skip >> i) & 1u) continue;
+        const float4 ball = E.ball[i];
+        const float3 w = xyz(ball) - po;
+        const float t0 = dot3(w, v) * ivv;
+        const float3 q = w - v * fminf(fmaxf(t0, 0.0f), 1.0f);
+        const float lim = ball.w + fmaxf(fminf(1.0f, t0 + (ball.w + rb) * ilv), 0.0f) * rb;
+        bool clear = dot3(q, q) > lim * lim * 1.0001f;
+        if (!clear && i >= ns && i < ns + nq) {
+            const float4* P = S.prim[i];
+            const float3 c = xyz(P[0]), n = xyz(P[1]), pc = po - c;
+            const float pp = dot3(pc, pc), mg = 1.1e-5f + 2.1e-6f * pp * rsqrt_fast(fmaxf(pp, 1e-30f));
+            const float sp = dot3(pc, n), sb = dot3(bc - c, n);
+            const float eb = fabsf(n.x) * bh.x + fabsf(n.y) * bh.y + fabsf(n.z) * bh.z;
+            clear = (sp > mg && sb - eb > mg) || (sp < -mg && sb + eb < -mg);
+        }
+        if (clear) m |= 1u << i;
+    }
+    return m;
+}
+
+// Does the segment o + t d, 0 <= t <= tmax, touch a union box of the perturbed primitives?
+template <bool kCount>
+__device__ __forceinline__ bool replay_touch(const ReplayLane& E, float3 o, float3 d, float tmax, Counters& cnt) {
+    const float3 inv = rcp3(d);
+    const float tm = tmax * 1.0001f + 1e-3f;
+    bool hit = false;
+#pragma unroll 1
+    for (int k = 0; k < E.n_var; ++k) hit = hit || slab_touch(xyz(E.ulo[k]), xyz(E.uhi[k]), o, inv, tm);
+    if (kCount) cnt.box += E.n_var;
+    return hit;
+}
+
+// One vertex of a path of a replay job (as advance), recording what can differ between the
+// renders. kMat: the job binds albedos; kMove: it perturbs primitives.
+template <bool kCount, bool kMat, bool kMove>
+__device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int rr_start, Path& p, ReplayLane& E,
+                                             Counters& cnt) {
+    const Hit h = closest_hit<kCount, kMove>(S, p.o, p.d, cnt, kMove ? E.skip : 0u);
+    const bool miss = h.slot < 0;
+    const bool touch = kMove && replay_touch<kCount>(E, p.o, p.d, miss ? 3.0e38f : h.t, cnt);
+    bool rec = E.rec || touch, bound = false, last = true, rr = false;
+    unsigned emis = 0u, vert = 0u;  // info words of the entries to record (emission: 0 none)
+    int nvert = 0;                  // granules of the vertex entry
+    float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0, v2 = v0;
+    float3 pt = p.o, ng = p.d, ns = p.d, po = p.o, albedo = p.d;
+    int mtype = kDiffuse;
+    float ior = 1.0f;
+    uint4 w0 = make_uint4(0u, 0u, 0u, 0u), w1 = w0;
+    if (miss) {
+        if (!rec) p.L = bg_add(p.L, p.beta, xyz(S.bg));
+        else if (S.bg.x != 0.0f || S.bg.y != 0.0f || S.bg.z != 0.0f) emis = kEmission | 32u;
+    } else {
+        if (kCount) ++cnt.vertices;
+        pt = p.o + p.d * h.t;
+        int mat = 0;
+        ng = surface_normal(static_cast<const float4*>(S.prim[h.slot]), h.type, pt, p.o, p.d, mat);
+        const float4 m0 = S.mat[mat][0], m1 = S.mat[mat][1];
+        mtype = as_int(m0.w);
+        ior = m1.w;
+        const float3 emission = xyz(m1);
+        albedo = xyz(m0);
+        if (p.specular && (emission.x > 0.f || emission.y > 0.f || emission.z > 0.f) && dot3(p.d, ng) < 0.0f) {
+            if (rec) emis = kEmission | (unsigned(mat) << 8);
+            else p.L = p.L + p.beta * emission;
+        }
+        if (kMat && ((E.mats >> mat) & 1u)) {
+            bound = rec = true;
+            albedo = xyz(E.amax[mat]);
+        }
+        last = p.b + 1 >= depth;
+        rr = !last && rr_start >= 0 && p.b >= rr_start;
+        const bool flip = !(dot3(ng, p.d) < 0.0f);
+        ns = flip ? ng * -1.0f : ng;
+        po = pt + ns * kEps;
+        const bool diffuse = mtype == kDiffuse;
+        if (diffuse) w0 = path_words<true>(S, p.pixel, p.s, p.b, 0);
+        if (diffuse ? (S.n_lights > 1 || rr) : (!last && (rr || mtype == kDielectric)))
+            w1 = path_words<true>(S, p.pixel, p.s, p.b, 1);
+        const float urr = u01(w1.y);
+        unsigned est = 0u;
+        int li = 0;
+        if (diffuse && S.n_lights > 0) {  // next-event estimation: one emitter, uniform area sample
+            const float3 ba = p.beta * albedo;
+            if (maxc(ba) > 0.0f || bound) {  // (a black vertex adds nothing, nor has it derivatives unless bound)
+                li = nee_light(S, w1.x);
+                const int lslot = S.light[li].y;
+                const float lu = u01(w0.x), lv = u01(w0.y);
+                if (kMove && ((E.skip >> lslot) & 1u)) {  // each render's own estimate
+                    est = 1u;
+                    rec = true;
+                    vert = shadow_cull(S, E, po, lslot) << (32 - kCullBits);
+                    v0 = make_float4(po.x, po.y, po.z, 0.f);
+                    if (kMat) {
+                        v1 = make_float4(lu, lv, urr, 0.f);
+                        v2 = make_float4(ns.x, ns.y, ns.z, 0.f);
+                        vert |= (flip ? 1u << 17 : 0u) | (h.type != kQuad ? 1u << 18 : 0u) | (unsigned(h.slot) << 12);
+                        nvert = h.type != kQuad ? 3 : 2;
+                    } else {
+                        v1 = make_float4(ba.x, ba.y, ba.z, lu);
+                        v2 = make_float4(ns.x, ns.y, ns.z, lv);
+                        nvert = 3;
+                    }
+                } else {
+                    float3 wi;
+                    float dist, g;
+                    int lmat;
+                    if (nee_to<kCount, kMove, false>(S, po, ns, lu, lv, li, cnt, kMove ? E.skip : 0u, nullptr, wi, dist,
+                                                     g, lmat)) {
+                        const bool own = kMove && replay_touch<kCount>(E, po, wi, dist, cnt);
+                        rec = rec || own;
+                        if (!rec) {
+                            p.L = nee_add(p.L, ba, xyz(S.mat[lmat][1]), g);
+                        } else if (own) {
+                            est = 3u;
+                            v0 = make_float4(po.x, po.y, po.z, 0.f);
+                            v1 = make_float4(wi.x, wi.y, wi.z, dist);
+                            v2 = kMat ? make_float4(g, urr, 0.f, 0.f) : make_float4(ba.x, ba.y, ba.z, g);
+                            nvert = 3;
+                        } else {
+                            est = 2u;
+                            v0 = make_float4(g, urr, 0.f, 0.f);
+                            v2 = make_float4(ba.x, ba.y, ba.z, g);
+                            nvert = kMat ? 1 : 3;
+                        }
+                    }
+                }
+            }
+        }
+        if (kMat && rec && est == 0u) {
+            v0 = make_float4(0.f, urr, 0.f, 0.f);
+            nvert = 1;
+        }
+        vert |= kVert | (est << 2) | (rr ? 16u : 0u) | (unsigned(li) << 5) | (unsigned(mat) << 8);
+    }
+    // ---- record the vertex's group: prefix, segment, emission, vertex ------------------------
+    const bool pre = rec && !E.rec &&
+                     (p.L.x != 0.0f || p.L.y != 0.0f || p.L.z != 0.0f ||
+                      (kMat && (p.beta.x != 1.0f || p.beta.y != 1.0f || p.beta.z != 1.0f)));
+    const int npre = pre ? (kMat ? 2 : 1) : 0, nseg = touch ? (kMat ? 2 : 3) : 0;
+    const int total = npre + nseg + (emis ? 1 : 0) + nvert;
+    E.rec = rec;
+    if (total) {
+        int i = int(atomicAdd(E.ctr, unsigned(total)));
+        if (i + total > E.cap) {
+            E.full = true;
+            return kEnded;
+        }
+        E.nxt[i] = (unsigned short)(kNoEntry);
+        if (E.first == kNoEntry) E.first = i;
+        else E.nxt[E.last] = (unsigned short)(i);
+        E.last = i;
+        const int end = i + total;
+        if (pre) {
+            E.ent[i] = make_float4(p.L.x, p.L.y, p.L.z, __uint_as_float(kPrefix | (i + npre == end ? kLastEntry : 0u)));
+            if (kMat) E.ent[i + 1] = make_float4(p.beta.x, p.beta.y, p.beta.z, 0.f);
+            i += npre;
+        }
+        if (kMove && touch) {
+            const unsigned info = kSegment | (p.specular ? 16u : 0u) | (unsigned(p.b) << 8) |
+                                  (i + nseg == end ? kLastEntry : 0u);
+            E.ent[i] = make_float4(p.o.x, p.o.y, p.o.z, __uint_as_float(info));
+            E.ent[i + 1] = make_float4(p.d.x, p.d.y, p.d.z, miss ? INFINITY : h.t);
+            if (!kMat) E.ent[i + 2] = make_float4(p.beta.x, p.beta.y, p.beta.z, 0.f);
+            i += nseg;
+        }
+        if (emis) {
+            E.ent[i] = make_float4(p.beta.x, p.beta.y, p.beta.z, __uint_as_float(emis | (i + 1 == end ? kLastEntry : 0u)));
+            ++i;
+        }
+        if (nvert) {
+            v0.w = __uint_as_float(vert | kLastEntry);
+            E.ent[i] = v0;
+            if (kMove && nvert > 1) E.ent[i + 1] = v1;
+            if (kMove && nvert > 2) E.ent[i + 2] = v2;
+        }
+    }
+    if (miss || last) return kEnded;
+    // ---- the next ray ---------------------------------------------------------------------------
+    if (mtype == kDiffuse) {
+        p.d = normalized(diffuse_dir(ns, u01(w0.z), u01(w0.w)));
+        p.o = po;
+        p.specular = false;
+    } else {
+        if (mtype == kMirror) {
+            p.d = normalized(p.d - ns * (2.0f * dot3(p.d, ns)));
+            p.o = po;
+        } else {
+            dielectric(p, pt, ng, ior, u01(w1.z));
+        }
+        p.specular = true;
+    }
+    p.beta = p.beta * albedo;
+    if (kMat) E.varied = E.varied || bound;
+    if (maxc(p.beta) <= 0.0f) return kEnded;
+    if (rr) {  // Russian roulette on slot 1's second uniform
+        if (kMat && E.varied) {
+            // A render survives when u < q_r = min(0.95, max beta_r), and q_r <= q here; its
+            // largest throughput is then max(1, max beta_r / 0.95) up to rounding.
+            const float bm = maxc(p.beta);
+            if (u01(w1.y) >= fminf(0.95f, bm * 1.000001f)) return kEnded;
+            const float nb = fmaxf(1.0f, bm * 1.0527f) * 1.00001f;
+            p.beta = f3(nb, nb, nb);
+        } else {
+            const float q = fminf(0.95f, maxc(p.beta));
+            if (u01(w1.y) >= q) return kEnded;
+            p.beta = p.beta * rcp_fast(q);
+        }
+    }
+    ++p.b;
+    return kLive;
+}
+
+// ---------------------------------------------------------------------------
+// k_trace_replay: every path traced once, replayed by each render (a3-a5)
+// ---------------------------------------------------------------------------
+// Under common random numbers the renders of a job differ only where a perturbed primitive
+// meets a ray, where an emitter that moved is sampled, and in the albedos that are bound. A
+// work item is one of a pixel block's J.parts parts (1/parts of the positions of the bit-reversed
+// slot order) for all R <= 64 renders, taken by one warp, which takes the part's (pixel, sample)
+// tasks in batches of 32, pixels in that order:
+//   phase A  lane = task: the path is traced once in the invariant scene (replay_vertex). What
+//            is the same in every render goes into the pixel's common sum, the rest into a
+//            chain of entries in the warp's pool. A batch whose pool runs out keeps the paths
+//            before the first one that did not fit, and the next batch starts there (with that
+//            path alone if it was the batch's first: the pool holds any one path);
+//   phase B  lane = render (lane and lane + 32; with R < 32 the lanes hold floor(32 / R)
+//            samples side by side): each render replays the chains with its own primitives,
+//            albedos and tangents (replay_sample). A render that parts from the path (its own
+//            primitive is hit first) traces the rest as k_trace_group does, unless that
+//            primitive is black (most emitters), where the path ends.
+// Each render's radiance is the same sum, term by term and in the same order, as tracing the
+// path in that render alone, and the pairwise pixel sum is the shuffle tree of the per-render
+// epilogue (see k_trace_group): with the same block shape every partial is bit-identical to
+// the per-render kernel's; a part's sum is a subtree, and the warp that finishes a block's last
+// part adds them. The warps of a CTA share the staged scene and the per-render table
+// and meet only when the launch goes on to another job.
+//
+// Tracing a path once instead of once per render leaves per render only its estimates (light
+// sample, occlusion by the few primitives the cull leaves, geometry term) and products of
+// albedos. Before, the GI box's renders retraced every path side by side (k_trace_group) and Eq. 9
+// traced each render alone (k_trace): GI box 512 x 512, 32 renders at 32 spp 40.9 -> 16.2 ms, its
+// walls by Eq. 9 87.6 -> 7.5 ms, by Eq. 10 at 256 x 256 11.3 -> 1.26 ms, caustic 512 x 512, 64 renders at
+// 64 spp 7.8 -> 7.3 ms (caustic 237 x 141, 24 renders at 20 spp: 250 -> 258 us, the larger code's
+// cold start). Bound by instruction issue (60 % of cycles, 20 warps per SM): fixed-latency
+// dependencies and instruction fetch are the largest stalls, phase A takes about a quarter of the
+// GI box's time and half of Eq. 9's. Groups of entries are 16-byte granules because the pool's
+// shared memory sets how many paths fit a batch.
+constexpr int kReplayWarps = kGroupBlock / 32;
+
+// Shared memory of a CTA: this head, the per-render table, and per warp (replay_warp_bytes)
+//   double pair[halves][levels][32]   pairwise-sum stacks of the lane's renders
+//   u64 acc[halves][3][32]            radiance of the current pixel, 2^-32 fixed point
+//   u64 dacc[halves][nd][32]          Eq. 9: its tangent sums
+//   double gsum[halves][nd][32]       Eq. 9: the block's gradient partials
+//   u64 common[pixels][3]             radiance common to all renders, per pixel of the block
+//   float4 ent[pool], u16 nxt[pool], u16 first[32], unsigned ctr
+struct ReplayHead {
     GroupScene scene;  // the invariant part (render 0's records of the other primitives)
     TraceJob job;
-    float4 tab[kEmitTab];  // per-render rows (as k_trace_group's), R x gstride
     float4 ulo[kMaxVariant], uhi[kMaxVariant];
-    double sub[kEmitWarps][64];
-    EmitWarp w[kEmitWarps];
-    unsigned item;
-    int job_index;
+    float4 amax[kGroupMats];   // largest albedo of each bound material over the renders
+    float4 ball[kGroupPrims];  // enclosing balls of the invariant primitives
+    unsigned left, pad[3];     // has the job items left?
+};
+static_assert(sizeof(ReplayHead) % 16 == 0, "float4 arrays follow");
+
+__host__ __device__ constexpr int replay_levels(int pixels) {
+    return pixels <= 1 ? 0 : (pixels <= 2 ? 1 : (pixels <= 4 ? 2 : (pixels <= 8 ? 3 : (pixels <= 16 ? 4 : 5))));
+}
+__host__ __device__ constexpr size_t replay_warp_bytes(int pool, int halves, int pixels, int nd) {
+    return size_t(halves) * (replay_levels(pixels) + 3 + 2 * nd) * 256 + ((size_t(pixels) * 24 + 15) & ~size_t(15)) + size_t(pool) * 18 + 80;
+}
+size_t replay_smem(const TraceLaunch& L) {
+    return sizeof(ReplayHead) + size_t(L.tab_rows) * 16 +
+           kReplayWarps * replay_warp_bytes(L.pool, L.halves, L.pixels, L.diff_nd);
+}
+
+// Resident CTAs per SM that a variant is compiled for: 6 (<= 80 registers, 24 warps), or 5 (<= 102)
+// with perturbed primitives, where the pool needs the shared memory (the GI box with only its
+// light moving, 32 renders at 16 spp: 8.4 ms with 5, 15.6 ms with 6; the GI box's walls, 256 x 256:
+// 1.33 ms with 5, 1.25 ms with 6).
+constexpr int replay_min_blocks(bool move) { return move ? 5 : 6; }
+
+// The pool takes the shared memory that replay_min_blocks CTAs per SM (the registers' limit) leave,
+// up to kReplayPoolMax granules: a pool that runs out costs part of a batch's phase A (GI box at
+// 32 renders, 224 granules of 3 float4 instead of 128: 73 -> 27 ms), a CTA less per SM more.
+constexpr int kReplayPoolMax = 512;
+int replay_pool(const TraceLaunch& L) {
+    const size_t kCta = 227 * 1024 / replay_min_blocks(L.replay_move != 0) - 1024;  // 1 KB is the system's
+    const size_t head = sizeof(ReplayHead) + size_t(L.tab_rows) * 16;
+    const size_t rest = replay_warp_bytes(0, L.halves, L.pixels, L.diff_nd);
+    int fits = 0;
+    if (kCta > head + kReplayWarps * rest) fits = int((kCta - head - kReplayWarps * rest) / (18 * kReplayWarps));
+    fits = fits < kReplayPoolMax ? fits : kReplayPoolMax;
+    const int need = (L.pool + 7) & ~7;
+    return fits > need ? fits & ~7 : need;
+}
+
+// A render's clamp derivatives (Eq. 9) in its row of the table.
+struct ClampRow {
+    const float4* p;
+    int s;
+    __device__ __forceinline__ float operator[](int k) const {
+        return reinterpret_cast<const float*>(p + (k >> 2) * s)[k & 3];
+    }
 };
 
-// The rest of a stopped path in one render's scene (as k_trace_group traces it).
+// Sum of non-negative floats below 2^14 in 2^-32 fixed point, as to_fixed adds them, without
+// 64-bit arithmetic: hi counts units of 2^-9 (the bits that an addition of 2^14 rounded toward
+// zero keeps), lo the rest in units of 2^-32. The sum is (hi << 23) + lo; 32 terms fit.
+__device__ __forceinline__ void fix_add(unsigned& hi, unsigned& lo, float v) {
+    const float s = __fadd_rz(v, 16384.0f);
+    hi += __float_as_uint(s) - 0x46800000u;
+    const float r = v - (s - 16384.0f);  // exact, in [0, 2^-9)
+    lo += __float_as_uint(__fadd_rz(r, 0x1p-9f)) - 0x3b000000u;
+}
+__device__ __forceinline__ unsigned long long fix_sum(unsigned hi, unsigned lo) {
+    return ((unsigned long long)hi << 23) + lo;
+}
+// The same for |v| < 2^13 (tangents): rounded down to 2^-32, hi signed.
+__device__ __forceinline__ void fix_add_signed(unsigned& hi, unsigned& lo, float v) {
+    const float s = __fadd_rz(v, 24576.0f);
+    hi += __float_as_uint(s) - 0x46c00000u;
+    const float r = v - (s - 24576.0f);
+    lo += __float_as_uint(__fadd_rz(r, 0x1p-9f)) - 0x3b000000u;
+}
+__device__ __forceinline__ unsigned long long fix_sum_signed(unsigned hi, unsigned lo) {
+    return (unsigned long long)((long long)int(hi) << 23) + lo;
+}
+
+// The rest of a path in one render's scene (as k_trace_group traces it).
 template <bool kCount>
-__device__ __forceinline__ float3 emit_continue(const GroupScene& S, int depth, int rr_start, const GroupLane& gl,
-                                                Path p, Counters& cnt) {
+__device__ __forceinline__ float3 replay_alone(const GroupScene& S, int depth, int rr_start, const GroupLane& gl,
+                                               Path p, Counters& cnt) {
     while (advance<kCount, false, 0, true>(S, depth, rr_start, p, cnt, nullptr, nullptr, nullptr, &gl) == kLive) {
     }
     return p.L;
 }
 
-#ifndef PRDPT_EMIT_MIN_BLOCKS
-#define PRDPT_EMIT_MIN_BLOCKS 5  // <= 102 registers: 20 resident warps per SM
-#endif
-constexpr int kEmitMinBlocks = PRDPT_EMIT_MIN_BLOCKS;
+// One render's radiance from a path's chain (without the common part). kMove: 0 no perturbed primitive, 1 only black ones (a render that meets its own
+// primitive ends there), 2 any. Tangent slot k is a parameter of channel k mod 3 (kND: 0 or a
+// multiple of 3); J.mat_slots[m] holds the slots of material m's parameters.
+template <bool kCount, bool kMat, int kMove, int kND>
+__device__ __forceinline__ float3 replay_sample(const GroupScene& S, const TraceJob& J, const GroupLane& gl,
+                                                const float4* ent, const unsigned short* nxt, int i, unsigned pixel,
+                                                int s, int slot, Counters& cnt, Tangents<kND>& tn) {
+    float3 Lr = f3(0.f, 0.f, 0.f), beta = f3(1.f, 1.f, 1.f);
+    const ClampRow dclamp{gl.rec + (gl.var_rows + __popc(gl.mats)) * gl.rs, gl.rs};
+    bool on = true, parted = false;  // on the shared path; left it to go on alone
+    Path p;
+    int next = nxt[i];
+#pragma unroll 1
+    while (i != kNoEntry) {
+        const float4 a = ent[i];
+        const unsigned info = __float_as_uint(a.w), kind = info & 3u;
+        const int mat = int(info >> 8) & 15;
+        int size = 1;
+        if (kind == kVert) {
+            const unsigned est = (info >> 2) & 3u;
+            size = !kMove ? 1 : (!kMat || est == 3u || (info & (1u << 18)) ? 3 : (est == 1u ? 2 : 1));
+            if ((!kMat && !kMove) || on) {
+                float3 ba, albedo = f3(0.f, 0.f, 0.f);
+                float urr = 0.0f;
+                if (kMat) {
+                    albedo = xyz(mat_albedo<true>(S, mat, &gl));
+                    ba = beta * albedo;
+                    urr = a.y;
+                    if (kND > 0) {  // tangents of beta * albedo
+                        const unsigned ms = J.mat_slots[mat];
+#pragma unroll
+                        for (int k = 0; k < kND; ++k) {
+                            tn.dB[k] *= comp3(albedo, k % 3);
+                            if ((ms >> k) & 1u) tn.dB[k] = fmaf(comp3(beta, k % 3), dclamp[k], tn.dB[k]);
+                        }
+                    }
+                }
+                if (est) {
+                    const int li = int(info >> 5) & 7;
+                    bool seen = true;
+                    float g;
+                    int lmat;
+                    if (kMove && est == 1u) {
+                        const float4 b = ent[i + 1];
+                        float3 ns;
+                        float lu, lv;
+                        if (kMat) {
+                            urr = b.z;
+                            lu = b.x;
+                            lv = b.y;
+                            if (info & (1u << 18)) {
+                                ns = xyz(ent[i + 2]);
+                            } else {  // a quad's normal, from its record
+                                ns = xyz(S.prim[(info >> 12) & 15u][1]);
+                                if (info & (1u << 17)) ns = ns * -1.0f;
+                            }
+                        } else {
+                            const float4 c = ent[i + 2];
+                            ba = xyz(b);
+                            ns = xyz(c);
+                            lu = b.w;
+                            lv = c.w;
+                        }
+                        float3 wi;
+                        float dist;
+                        seen = nee_to<kCount, false, true>(S, xyz(a), ns, lu, lv, li, cnt, info >> (32 - kCullBits), &gl,
+                                                           wi, dist, g, lmat);
+                    } else {
+                        const int4 lt = S.light[li];
+                        lmat = lt.w;
+                        g = a.x;
+                        if (kMove && (est == 3u || !kMat)) {
+                            const float4 c = ent[i + 2];
+                            g = kMat ? c.x : c.w;
+                            if (kMat) urr = c.y;
+                            else ba = xyz(c);
+                            if (est == 3u) {
+                                const float4 b = ent[i + 1];
+                                seen = !group_occluded<kCount>(S, gl, xyz(a), xyz(b), b.w, lt.y, cnt);
+                            }
+                        }
+                    }
+                    if (seen) {
+                        const float3 Le = xyz(S.mat[lmat][1]);
+                        if (kND > 0) {
+                            const float3 leg = Le * g;
+#pragma unroll
+                            for (int k = 0; k < kND; ++k) tn.dL[k] = fmaf(tn.dB[k], comp3(leg, k % 3), tn.dL[k]);
+                        }
+                        Lr = nee_add(Lr, ba, Le, g);
+                    }
+                }
+                if (kMat) {
+                    const float mb = maxc(ba);
+                    on = mb > 0.0f;
+                    beta = ba;
+                    if (info & 16u) {  // Russian roulette
+                        const float q = fminf(0.95f, mb);
+                        on = on && urr < q;
+                        const float inv_q = rcp_fast(q);
+                        beta = beta * inv_q;
+#pragma unroll
+                        for (int k = 0; k < kND; ++k) tn.dB[k] *= inv_q;
+                    }
+                }
+            }
+        } else if (kMove && kind == kSegment) {
+            size = kMat ? 2 : 3;
+            if (on) {
+                const float4 b = ent[i + 1];
+                Hit h{b.w, -1, 0};
+                group_hit<kCount>(S, gl, xyz(a), xyz(b), h, cnt);
+                if (h.slot >= 0) {  // this render's own primitive comes first
+                    on = false;
+                    const float3 bt = kMat ? beta : xyz(ent[i + 2]);
+                    const auto P = prim_rec<true>(S, h.slot, &gl);
+                    const int hm = as_int(h.type == kSphere ? P[1].z : P[0].w) & 255;
+                    const float4 al = mat_albedo<true>(S, hm, &gl);
+                    if (kMove == 1 || (as_int(al.w) == kDiffuse && al.x == 0.0f && al.y == 0.0f && al.z == 0.0f)) {
+                        // a black surface: its emission, and the path ends
+                        const float3 em = xyz(S.mat[hm][1]);
+                        if ((info & 16u) && (em.x > 0.f || em.y > 0.f || em.z > 0.f)) {
+                            const float3 d = xyz(b), pt = xyz(a) + d * h.t;
+                            const float3 ng = h.type == kSphere ? (pt - xyz(P[0])) * P[1].y : xyz(P[1]);
+                            if (dot3(d, ng) < 0.0f) Lr = Lr + bt * em;
+                        }
+                    } else {
+                        parted = true;
+                        p.o = xyz(a);
+                        p.d = xyz(b);
+                        p.beta = bt;
+                        p.specular = (info & 16u) != 0u;
+                        p.b = int(info >> 8) & 127;
+                    }
+                }
+            }
+        } else if (kind == kEmission) {
+            if ((!kMat && !kMove) || on) {
+                const float3 E = (info & 32u) ? xyz(S.bg) : xyz(S.mat[mat][1]);
+#pragma unroll
+                for (int k = 0; k < kND; ++k) tn.dL[k] = fmaf(tn.dB[k], comp3(E, k % 3), tn.dL[k]);
+                Lr = Lr + (kMat ? beta : xyz(a)) * E;
+            }
+        } else if (kind == kPrefix) {
+            Lr = xyz(a);
+            if (kMat) {
+                beta = xyz(ent[i + 1]);
+                size = 2;
+            }
+        }
+        if (info & kLastEntry) {
+            i = next;
+            if (i != kNoEntry) next = nxt[i];
+        } else {
+            i += size;
+        }
+    }
+    if (kMove == 2 && parted) {
+        p.L = Lr;
+        p.pixel = pixel;
+        p.s = s;
+        p.slot = slot;
+        p.seg = 0u;
+        Lr = replay_alone<kCount>(S, J.depth, J.rr_start, gl, p, cnt);
+    }
+    return Lr;
+}
 
-template <bool kCount>
-__global__ void __launch_bounds__(kGroupBlock, kEmitMinBlocks) k_trace_emit(const __grid_constant__ TraceLaunch L) {
-    __shared__ EmitSmem E;
+// Sum number k (0 the squared error, 1 + slot a tangent slot's) of work item `item` in render r. Out
+// of line, like replay_combine: both run once per item, and inlined they cost the loops registers.
+template <int kND>
+__device__ __noinline__ void replay_store(const TraceJob& J, unsigned item, int r, int k, double v) {
+    if (J.parts > 1) {
+        J.part_sums[(size_t(item) * J.R + r) * (1 + kND) + k] = v;
+    } else if (k == 0) {
+        J.partials[size_t(r) * J.tiles + item] = v;
+    } else if (J.slot_param[k - 1] >= 0) {
+        J.gpartials[(size_t(r) * J.tiles + item) * J.diff_n + J.slot_param[k - 1]] = v;
+    }
+}
+
+// The warp that finishes a block's last part adds the parts' subtrees in the pairwise sum's order.
+template <int kND>
+__device__ __noinline__ void replay_combine(const TraceJob& J, unsigned item, int lane) {
+    const int parts = J.parts, t = int(item) / parts;
+    unsigned done = 0;
+    __threadfence();  // the part's sums before its count
+    __syncwarp();
+    if (lane == 0) {
+        done = atomicAdd(J.part_done + t, 1u);
+        __threadfence();
+    }
+    done = __shfl_sync(kFull, done, 0);
+    if (done != unsigned(parts - 1)) return;
+    const int n = J.R * (1 + kND);
+    for (int i = lane; i < n; i += 32) {
+        const int r = i / (1 + kND), k = i - r * (1 + kND);
+        const int param = k > 0 ? J.slot_param[k - 1] : 0;
+        if (param < 0) continue;
+        double s[5], v = 0.0;
+        for (int p = 0; p < parts; ++p) {
+            v = __ldcg(J.part_sums + (size_t(t) * parts + p) * n + i);
+            int l = 0;
+            for (; (p >> l) & 1; ++l) v = s[l] + v;
+            if (p + 1 < parts) s[l] = v;
+        }
+        if (k == 0) J.partials[size_t(r) * J.tiles + t] = v;
+        else J.gpartials[(size_t(r) * J.tiles + t) * J.diff_n + param] = v;
+    }
+    if (lane == 0) J.part_done[t] = 0u;  // ready for the next launch
+}
+
+template <bool kCount, bool kMat, int kMove, int kND>
+__global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_trace_replay(const __grid_constant__ TraceLaunch L) {
+    extern __shared__ __align__(16) unsigned char s_replay[];
+    ReplayHead& E = *reinterpret_cast<ReplayHead*>(s_replay);
+    float4* tab = reinterpret_cast<float4*>(s_replay + sizeof(ReplayHead));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    EmitWarp& Wp = E.w[warp];
+    const int levels = replay_levels(L.pixels), halves = L.halves;
+    unsigned char* wbase = s_replay + sizeof(ReplayHead) + size_t(L.tab_rows) * 16 +
+                           size_t(warp) * replay_warp_bytes(L.pool, halves, L.pixels, kND);
+    double (*pair)[32] = reinterpret_cast<double (*)[32]>(wbase);
+    unsigned long long (*acc)[32] = reinterpret_cast<unsigned long long (*)[32]>(pair + halves * levels);
+    unsigned long long (*dacc)[32] = acc + halves * 3;
+    double (*gsum)[32] = reinterpret_cast<double (*)[32]>(dacc + halves * kND);
+    unsigned long long (*common)[3] = reinterpret_cast<unsigned long long (*)[3]>(gsum + halves * kND);
+    float4* ent = reinterpret_cast<float4*>(common + L.pixels + (L.pixels & 1));
+    unsigned short* nxt = reinterpret_cast<unsigned short*>(ent + L.pool);
+    unsigned short* firsts = nxt + L.pool;
+    unsigned* ctr = reinterpret_cast<unsigned*>(firsts + 32);
     const TraceJob& J = E.job;
-    int cur_job = -1;
     Counters cnt{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    if (!L.jobs) {  // a single job's descriptor is host data: copied before the wait
-        const unsigned* src = reinterpret_cast<const unsigned*>(&L.job0);
+    const int njobs = L.jobs ? L.njobs : 1;
+    for (int jb = 0; jb < njobs; ++jb) {  // a packed launch's jobs one after another, each CTA from another one
+    {  // job descriptors are host data: the first is copied before the wait on the previous kernel
+        const unsigned* src =
+            reinterpret_cast<const unsigned*>(L.jobs ? L.jobs + (int(blockIdx.x) + jb) % njobs : &L.job0);
         unsigned* dst = reinterpret_cast<unsigned*>(&E.job);
+        __syncthreads();  // every warp is done with the previous job
         for (int i = threadIdx.x; i < int(sizeof(TraceJob) / 4); i += kGroupBlock) dst[i] = src[i];
+        if (jb == 0) pdl_enter();
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) E.left = __ldcg(J.queue) < unsigned(J.tiles * J.parts) ? 1u : 0u;
+    __syncthreads();
+    if (!E.left) continue;
+    const int n = J.n_var, nr = J.var_rows, nm = __popc(J.var_mats), stride = J.gstride, ncl = (kND + 3) / 4;
+    if (J.R < 1 || J.R > 32 * halves || J.R * stride > L.tab_rows || stride < nr + nm + ncl || n < 0 ||
+        n > kMaxVariant || J.n_prims > kGroupPrims || J.n_mats > kGroupMats || (!kMat && nm) || (!kMove && n) ||
+        (kMove == 1 && !J.black && n) || J.parts < 1 || J.parts > J.bw * J.bh ||
+        J.bw * J.bh > L.pixels * J.parts || (J.parts & (J.parts - 1)) != 0 || replay_path_granules(J.depth, kMove != 0) > L.pool) {
+        if (threadIdx.x == 0) atomicOr(L.status, kStatusBadItem);
+        continue;
+    }
+    // ---- stage the job: invariant scene, per-render rows, union bounds --------------------------
+    if (warp == 0) stage_group_scene(E.scene, J, 0, lane);
+    for (int i = threadIdx.x; i < J.R * stride; i += kGroupBlock) {
+        const int r = i / stride, q = i - r * stride;
+        const InstScene& R = J.scenes[r];
+        float4 v;
+        if (q < nr) {
+            v = __ldg(&R.prim[J.row_src[q] >> 1][J.row_src[q] & 1]);
+        } else if (q < nr + nm) {
+            v = __ldg(&R.mat[nth_set_bit(J.var_mats, q - nr)][0]);
+        } else if (kND > 0) {  // clamp derivatives by tangent slot
+            const int k = 4 * (q - nr - nm);
+            auto dc = [&](int slot) { return slot < kND && J.slot_param[slot] >= 0 ? __ldg(R.dclamp + J.slot_param[slot]) : 0.0f; };
+            v = make_float4(dc(k), dc(k + 1), dc(k + 2), dc(k + 3));
+        } else {
+            v = __ldg(reinterpret_cast<const float4*>(R.light_area) + (q - nr - nm));
+        }
+        tab[q * J.R + r] = v;  // field-major, as k_trace_group's table
     }
     __syncthreads();
-    pdl_enter();
-    for (;;) {
-        if (threadIdx.x == 0) {
-            const unsigned item = atomicAdd(L.queue, 1u);
-            int j = 0;
-            if (item < unsigned(L.total_items) && L.jobs) {
-                int lo = 0, hi = L.njobs - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) / 2;
-                    if (L.jobs[mid].item_begin <= int(item)) lo = mid; else hi = mid - 1;
-                }
-                j = lo;
-            }
-            E.item = item;
-            E.job_index = j;
+    if (kMat && int(threadIdx.x) < nm) {
+        float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int r = 0; r < J.R; ++r) {
+            const float4 v = tab[(nr + int(threadIdx.x)) * J.R + r];
+            m = make_float4(fmaxf(m.x, v.x), fmaxf(m.y, v.y), fmaxf(m.z, v.z), 0.f);
         }
-        __syncthreads();
-        const unsigned item = E.item;
-        const int j = E.job_index;
-        if (item >= unsigned(L.total_items)) break;
-        if (j != cur_job) {  // stage the job, its invariant scene, per-render rows and union bounds
-            if (L.jobs) {
-                const unsigned* src = reinterpret_cast<const unsigned*>(L.jobs + j);
-                unsigned* dst = reinterpret_cast<unsigned*>(&E.job);
-                for (int i = threadIdx.x; i < int(sizeof(TraceJob) / 4); i += kGroupBlock) dst[i] = src[i];
-                __syncthreads();
+        E.amax[nth_set_bit(J.var_mats, int(threadIdx.x))] = m;
+    }
+    if (kMove && warp == 1 && lane < J.n_prims && lane < kCullBits)
+        E.ball[lane] = prim_ball(E.scene.prim[lane], lane < E.scene.n_sph ? kSphere
+                                                     : (lane < E.scene.n_sph + E.scene.n_quad ? kQuad : kBox));
+    if (kMove && warp == 0) {
+        for (int k = 0; k < n; ++k) {
+            const int slot = nth_set_bit(J.var_prims, k);
+            const int type = slot < E.scene.n_sph ? kSphere : (slot < E.scene.n_sph + E.scene.n_quad ? kQuad : kBox);
+            float3 lo = f3(INFINITY, INFINITY, INFINITY), hi = f3(-INFINITY, -INFINITY, -INFINITY);
+            for (int r = lane; r < J.R; r += 32) {
+                float3 a, c;
+                const SRec own{tab + ((J.var_offs >> (8 * k)) & 255u) * J.R + r, J.R, type == kQuad ? 1 : 2, E.scene.prim[slot]};
+                prim_bounds(own, type, a, c);
+                lo = f3(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z));
+                hi = f3(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
             }
-            if (J.R < 1 || J.R > 64 || J.R * J.gstride > kEmitTab || J.gstride < 4 * J.n_var || J.n_var < 1 ||
-                J.n_var > kMaxVariant || J.n_prims > kGroupPrims || J.n_mats > kGroupMats) {
-                if (threadIdx.x == 0) atomicOr(L.status, kStatusBadItem);
-                break;
-            }
-            if (warp == 0) stage_group_scene(E.scene, J, 0, lane);
-            const int stride = J.gstride, n = J.n_var;
-            for (int i = threadIdx.x; i < J.R * stride; i += kGroupBlock) {
-                const int r = i / stride, q = i - r * stride;
-                const InstScene& R = J.scenes[r];
-                float4 v;
-                if (q < 4 * n) v = __ldg(&R.prim[nth_set_bit(J.var_prims, q >> 2)][q & 3]);
-                else v = __ldg(reinterpret_cast<const float4*>(R.light_area) + (q - 4 * n));  // emitter areas
-                E.tab[q * J.R + r] = v;  // field-major, as k_trace_group's table
-            }
-            __syncthreads();
-            if (warp == 0) {
-                for (int k = 0; k < n; ++k) {
-                    const int slot = nth_set_bit(J.var_prims, k);
-                    const int type = slot < E.scene.n_sph ? kSphere : (slot < E.scene.n_sph + E.scene.n_quad ? kQuad : kBox);
-                    float3 lo = f3(INFINITY, INFINITY, INFINITY), hi = f3(-INFINITY, -INFINITY, -INFINITY);
-                    for (int r = lane; r < J.R; r += 32) {
-                        float3 a, c;
-                        const float4 rec[4] = {E.tab[(4 * k) * J.R + r], E.tab[(4 * k + 1) * J.R + r],
-                                               E.tab[(4 * k + 2) * J.R + r], E.tab[(4 * k + 3) * J.R + r]};
-                        prim_bounds(rec, type, a, c);
-                        lo = f3(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z));
-                        hi = f3(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
-                    }
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        lo.x = fminf(lo.x, __shfl_xor_sync(kFull, lo.x, o));
-                        lo.y = fminf(lo.y, __shfl_xor_sync(kFull, lo.y, o));
-                        lo.z = fminf(lo.z, __shfl_xor_sync(kFull, lo.z, o));
-                        hi.x = fmaxf(hi.x, __shfl_xor_sync(kFull, hi.x, o));
-                        hi.y = fmaxf(hi.y, __shfl_xor_sync(kFull, hi.y, o));
-                        hi.z = fmaxf(hi.z, __shfl_xor_sync(kFull, hi.z, o));
-                    }
-                    if (lane == 0) {
-                        E.ulo[k] = make_float4(lo.x, lo.y, lo.z, 0.f);
-                        E.uhi[k] = make_float4(hi.x, hi.y, hi.z, 0.f);
-                    }
-                }
+            for (int o = 16; o > 0; o >>= 1) {
+                lo.x = fminf(lo.x, __shfl_xor_sync(kFull, lo.x, o));
+                lo.y = fminf(lo.y, __shfl_xor_sync(kFull, lo.y, o));
+                lo.z = fminf(lo.z, __shfl_xor_sync(kFull, lo.z, o));
+                hi.x = fmaxf(hi.x, __shfl_xor_sync(kFull, hi.x, o));
+                hi.y = fmaxf(hi.y, __shfl_xor_sync(kFull, hi.y, o));
+                hi.z = fmaxf(hi.z, __shfl_xor_sync(kFull, hi.z, o));
             }
-            __syncthreads();
-            cur_job = j;
+            if (lane == 0) {
+                E.ulo[k] = make_float4(lo.x, lo.y, lo.z, 0.f);
+                E.uhi[k] = make_float4(hi.x, hi.y, hi.z, 0.f);
+            }
         }
-        const int t = int(item) - J.item_begin;
-        if (t < 0 || t >= J.tiles) {
-            if (threadIdx.x == 0) atomicOr(L.status, kStatusBadItem);
-            break;
-        }
-        const int R = J.R, nh = R > 32 ? 2 : 1, stride = J.gstride;
-        // phase B lanes: render gi = lane mod G of sample group ks = lane / G (G the power of
-        // two >= R, at most 32): with few renders a warp takes 32 / G samples at a time
-        const int G = R >= 32 ? 32 : (R <= 1 ? 1 : 1 << (32 - __clz(R - 1)));
-        const int nsg = 32 / G, gi = lane % G, ks = lane / G;
-        const int areas = stride > 4 * J.n_var ? 1 : 0;
+    }
+    __syncthreads();
+    // Positions of the bit-reversed order that can hold a pixel of a block of 2^k pixels are
+    // multiples of 2^(5 - k): the other levels of the pairwise sum would add zeros.
+    const int qshift = 5 - replay_levels(J.bw * J.bh), qend = (32 / J.parts) >> qshift;
+    for (;;) {  // ---- the warp's work items ------------------------------------------------------
+        unsigned item = 0;
+        if (lane == 0) item = atomicAdd(J.queue, 1u);
+        item = __shfl_sync(kFull, item, 0);
+        if (item >= unsigned(J.tiles * J.parts)) break;
+        const int t = int(item) / J.parts, q0 = (int(item) - t * J.parts) * (qend << qshift);
+        const int R = J.R, nh = R > 32 ? 2 : 1, spp = J.spp;
+        // phase B lanes: render gi of sample group ks; with R < 32, nsg = floor(32 / R) samples
+        // side by side (lanes beyond nsg R idle)
+        const int G = R < 32 ? R : 32, nsg = 32 / G, gi = lane % G, ks = lane / G;
+        const int areas = !kND && J.gstride > J.var_rows + __popc(J.var_mats) ? 1 : 0;
         const int x0 = (t % J.tiles_x) * J.bw, y0 = (t / J.tiles_x) * J.bh;
         const int vw = min(J.bw, J.W - x0), vh = min(J.bh, J.H - y0);
         const int npx = vw * vh;
         const unsigned magic_w = 0xffffffffu / unsigned(vw) + 1u;
-        const float inv = mean_scale(J.spp);
-        EmitLane el{E.ulo, E.uhi, J.n_var, J.var_prims, Wp.ent, lane, 0, false};
-        const bool bg_nonzero = E.scene.bg.x != 0.0f || E.scene.bg.y != 0.0f || E.scene.bg.z != 0.0f;
-        double sub[2] = {0.0, 0.0};
+        const float inv = mean_scale(spp);
+        // the part's positions that hold a pixel (bit q: position q0 + q)
+        const unsigned vm = __ballot_sync(kFull, lane < (qend << qshift) && brev5(q0 + lane) < npx);
+        const int npix = __popc(vm);
+        auto pixel_of = [&](int k, int& slot) {  // k-th pixel of the block
+            slot = brev5(q0 + nth_set_bit(vm, k));
+            const int row = div_magic(slot, vw, magic_w);
+            return unsigned((y0 + row) * J.W + x0 + slot - row * vw);
+        };
+        if (lane < npix)
+            for (int i = 0; i < 3; ++i) common[lane][i] = 0ull;
+#pragma unroll 1
+        for (int i = 0; i < 3 * nh; ++i) acc[i][lane] = 0ull;
+#pragma unroll 1
+        for (int i = 0; i < kND * nh; ++i) {
+            dacc[i][lane] = 0ull;
+            gsum[i][lane] = 0.0;
+        }
+        auto push_pair = [&](int h, int q, double v) {  // position q << qshift of the pairwise sum
+            double (*s)[32] = pair + h * levels;
+            int l = 0;
+#pragma unroll 1
+            for (; (q >> l) & 1; ++l) v = s[l][lane] + v;
+            if (q + 1 < qend) s[l][lane] = v;
+            else if (ks == 0 && gi + 32 * h < R) replay_store<kND>(J, item, gi + 32 * h, 0, v);  // a5
+        };
+        int k0 = 0, s0 = 0;    // the next task: pixel k0 of the block, sample s0
+        int nextq = 0;         // positions below are summed
+        bool alone = false;    // the next batch holds one path only
         // The loops below stay rolled: unrolled copies of the tracer overflow the instruction
         // cache (measured on the caustic step: 13.1 ms unrolled, 11.0 ms rolled).
 #pragma unroll 1
-        for (int qq = 0; qq < kEmitSlots; ++qq) {
-            const int slot = brev5(warp * kEmitSlots + qq);  // pixels in bit-reversed slot order
-            double e[2] = {0.0, 0.0};
-            if (slot < npx) {
-                const int row = div_magic(slot, vw, magic_w);
-                const int px = x0 + slot - row * vw, py = y0 + row;
-                unsigned long long acc[2][3] = {{0ull, 0ull, 0ull}, {0ull, 0ull, 0ull}};
-                for (int s0 = 0; s0 < J.spp; s0 += 32) {
-                    // ---- phase A: one path per lane, traced once for all renders ----------
-                    __syncwarp();  // phase B of the previous samples is done with the table
-                    bool work = false;  // does the sample add anything to a render?
-                    if (s0 + lane < J.spp) {
-                        Path p;
-                        start_path<true>(E.scene, J.W, J.H, px, py, s0 + lane, slot, p);
-                        if (kCount) ++cnt.paths;
-                        el.n = 0;
-                        el.miss = false;
-                        int res;
-                        while ((res = advance<kCount, false, 0, false, true>(E.scene, J.depth, J.rr_start, p, cnt,
-                                                                             nullptr, nullptr, nullptr, nullptr,
-                                                                             &el)) == kLive) {
-                        }
-                        Wp.n[lane] = el.n;
-                        Wp.kind[lane] = (res == kAffected ? 2 : (el.miss ? 1 : 0)) | (p.specular ? 4 : 0);
-                        Wp.st[0][lane] = p.o.x;
-                        Wp.st[1][lane] = p.o.y;
-                        Wp.st[2][lane] = p.o.z;
-                        Wp.st[3][lane] = p.d.x;
-                        Wp.st[4][lane] = p.d.y;
-                        Wp.st[5][lane] = p.d.z;
-                        Wp.st[6][lane] = p.beta.x;
-                        Wp.st[7][lane] = p.beta.y;
-                        Wp.st[8][lane] = p.beta.z;
-                        Wp.st[9][lane] = __int_as_float(p.b);
-                        work = el.n > 0 || res == kAffected || (el.miss && bg_nonzero);
-                    }
-                    // ---- phase B: each render's terms of each sample, in sample order -----
-                    // (samples that add nothing to any render -- no kept vertex, not stopped,
-                    // no background term -- are passed over: their sums would add zero)
-                    __syncwarp();
-                    unsigned todo = __ballot_sync(kFull, work);
+        while (k0 < npix) {
+            // ---- phase A: one path per lane, traced once for all renders ----------------------
+            __syncwarp();  // phase B of the previous batch is done with the pool
+            if (lane == 0) *ctr = 0u;
+            __syncwarp();
+            int kp = k0, sp = s0 + lane;  // this lane's task
+            while (sp >= spp && kp < npix) {
+                sp -= spp;
+                ++kp;
+            }
+            const bool have = kp < npix && (!alone || lane == 0);
+            ReplayLane el{E.ulo,    E.uhi,    E.amax, E.ball, J.n_var, J.var_prims, J.var_mats, ent, nxt, ctr,
+                          L.pool, kNoEntry, kNoEntry, false,  false,   false};
+            Path p;
+            p.L = f3(0.f, 0.f, 0.f);
+            if (have) {
+                int slot;
+                const unsigned pixel = pixel_of(kp, slot);
+                const int py = int(pixel) / J.W, px = int(pixel) - py * J.W;
+                start_path<true>(E.scene, J.W, J.H, px, py, sp, slot, p);
+            }
+            bool live = have;
+#pragma unroll 1
+            while (__any_sync(kFull, live)) {
+                if (live) live = replay_vertex<kCount, kMat, (kMove != 0)>(E.scene, J.depth, J.rr_start, p, el, cnt) == kLive;
+            }
+            const unsigned fm = __ballot_sync(kFull, el.full), hm = __ballot_sync(kFull, have);
+            const int nb = fm ? __ffs(fm) - 1 : __popc(hm);  // the batch: tasks of lanes 0 .. nb - 1
+            if (nb == 0) {
+                if (alone) {  // cannot happen: the host sizes the pool for any one path
+                    if (lane == 0) atomicOr(L.status, kStatusBadItem);
+                    break;
+                }
+                alone = true;
+                continue;
+            }
+            alone = false;
+            if (lane < nb) {
+                if (kCount) ++cnt.paths;
+                firsts[lane] = (unsigned short)(el.first);
+                if (!el.rec && (p.L.x != 0.0f || p.L.y != 0.0f || p.L.z != 0.0f)) {
+                    smem_add_u64(&common[kp][0], to_fixed(p.L.x));
+                    smem_add_u64(&common[kp][1], to_fixed(p.L.y));
+                    smem_add_u64(&common[kp][2], to_fixed(p.L.z));
+                }
+            }
+            const unsigned work = __ballot_sync(kFull, lane < nb && el.first != kNoEntry);
+            __syncwarp();
+            // ---- phase B: each render's terms, pixel by pixel ---------------------------------
+            int i0 = 0;  // first task of the current pixel in the batch
+#pragma unroll 1
+            while (i0 < nb) {
+                const int i1 = min(nb, i0 + spp - s0);
+                const unsigned in = (i1 >= 32 ? kFull : (1u << i1) - 1u) & ~((1u << i0) - 1u);
+                int slot;
+                const unsigned pixel = pixel_of(k0, slot);
+                const bool ends = s0 + (i1 - i0) == spp;  // the pixel's last samples
+#pragma unroll 1
+                for (int h = 0; h < nh; ++h) {
+                    const int r = gi + 32 * h;
+                    const GroupLane gl{tab + (r < R ? r : 0), J.var_prims, J.var_mats, J.var_offs, J.var_rows, areas,
+                                       nullptr, 0, R};
+                    unsigned hi0 = 0u, hi1 = 0u, hi2 = 0u, lo0 = 0u, lo1 = 0u, lo2 = 0u;
+                    unsigned dhi[kND > 0 ? kND : 1], dlo[kND > 0 ? kND : 1];
+#pragma unroll
+                    for (int k = 0; k < kND; ++k) dhi[k] = dlo[k] = 0u;
+                    unsigned todo = work & in;
 #pragma unroll 1
                     while (todo) {
-                        int jj = -1;  // sample group ks takes the ks-th of the next nsg samples
-                        for (int i = 0; i < nsg && todo; ++i) {
-                            if (i == ks) jj = __ffs(todo) - 1;
+                        int jj = __ffs(todo) - 1;
+                        todo &= todo - 1u;
+#pragma unroll 1
+                        for (int i = 1; i < nsg; ++i) {  // sample group ks takes the ks-th of the next nsg tasks
+                            if (i <= ks) jj = __ffs(todo) - 1;
                             todo &= todo - 1u;
                         }
-                        if (jj < 0) continue;
-                        const int nk = Wp.n[jj], kind = Wp.kind[jj];
+                        if (jj < 0 || r >= R) continue;
+                        Tangents<kND> tn;
+                        if (kND > 0) tan_reset(tn);
+                        const float3 v = replay_sample<kCount, kMat, kMove, kND>(
+                            E.scene, J, gl, ent, nxt, firsts[jj], pixel, s0 + jj - i0, slot, cnt, tn);
+                        if (v.x + v.y + v.z < 16384.0f && fminf(v.x, fminf(v.y, v.z)) >= 0.0f) {
+                            fix_add(hi0, lo0, v.x);
+                            fix_add(hi1, lo1, v.y);
+                            fix_add(hi2, lo2, v.z);
+                        } else {
 #pragma unroll 1
-                        for (int h = 0; h < nh; ++h) {
-                            const int r = gi + 32 * h;
-                            if (r >= R) continue;
-                            const GroupLane gl{E.tab + r, J.var_prims, 0u, J.n_var, areas, nullptr, 0, R};
-                            float3 Lr = f3(0.f, 0.f, 0.f);
-#pragma unroll 1
-                            for (int k = 0; k < nk; ++k) {
-                                const float* en = Wp.ent + k * kEmitFields * 32 + jj;
-                                const float3 po = f3(en[0], en[32], en[64]), nsv = f3(en[96], en[128], en[160]);
-                                float3 wi;
-                                float dist, g;
-                                int lmat;
-                                if (nee_to<kCount, false, true>(E.scene, po, nsv, en[288], en[320],
-                                                                __float_as_int(en[352]), cnt, __float_as_uint(en[384]),
-                                                                &gl, wi, dist, g, lmat))
-                                    Lr = nee_add(Lr, f3(en[192], en[224], en[256]), xyz(E.scene.mat[lmat][1]), g);
-                            }
-                            const float3 beta = f3(Wp.st[6][jj], Wp.st[7][jj], Wp.st[8][jj]);
-                            if ((kind & 3) == 1) {
-                                Lr = bg_add(Lr, beta, xyz(E.scene.bg));
-                            } else if ((kind & 3) == 2) {  // the rest of the path in render r's scene
-                                Path p;
-                                p.o = f3(Wp.st[0][jj], Wp.st[1][jj], Wp.st[2][jj]);
-                                p.d = f3(Wp.st[3][jj], Wp.st[4][jj], Wp.st[5][jj]);
-                                p.beta = beta;
-                                p.L = Lr;
-                                p.pixel = unsigned(py * J.W + px);
-                                p.s = s0 + jj;
-                                p.b = __float_as_int(Wp.st[9][jj]);
-                                p.slot = slot;
-                                p.specular = (kind & 4) != 0;
-                                p.seg = 0u;
-                                Lr = emit_continue<kCount>(E.scene, J.depth, J.rr_start, gl, p, cnt);
-                            }
-                            if (Lr.x != 0.0f || Lr.y != 0.0f || Lr.z != 0.0f) {
-                                acc[h][0] += to_fixed(Lr.x);
-                                acc[h][1] += to_fixed(Lr.y);
-                                acc[h][2] += to_fixed(Lr.z);
-                            }
+                            for (int c = 0; c < 3; ++c) acc[3 * h + c][lane] += to_fixed(comp3(v, c));
+                        }
+#pragma unroll
+                        for (int k = 0; k < kND; ++k) {
+                            if (fabsf(tn.dL[k]) < 8192.0f) fix_add_signed(dhi[k], dlo[k], tn.dL[k]);
+                            else dacc[h * kND + k][lane] += to_fixed_signed(tn.dL[k]);
                         }
                     }
+                    unsigned long long a0 = acc[3 * h][lane] + fix_sum(hi0, lo0),
+                                       a1 = acc[3 * h + 1][lane] + fix_sum(hi1, lo1),
+                                       a2 = acc[3 * h + 2][lane] + fix_sum(hi2, lo2);
+                    acc[3 * h][lane] = ends ? 0ull : a0;
+                    acc[3 * h + 1][lane] = ends ? 0ull : a1;
+                    acc[3 * h + 2][lane] = ends ? 0ull : a2;
+                    if (!ends) {
+#pragma unroll
+                        for (int k = 0; k < kND; ++k) dacc[h * kND + k][lane] += fix_sum_signed(dhi[k], dlo[k]);
+                        continue;
+                    }
+                    // the pixel is complete: add its sample groups and the common part, form the error
+                    auto groups = [&](unsigned long long v) {
+                        unsigned long long sum = v;
+                        _Pragma("unroll 1") for (int q = 1; q < nsg; ++q) sum += __shfl_sync(kFull, v, (lane + q * G) & 31);
+                        return sum;
+                    };
+                    if (nsg > 1) {  // valid in the lanes of sample group 0
+                        a0 = groups(a0);
+                        a1 = groups(a1);
+                        a2 = groups(a2);
+                    }
+                    a0 += common[k0][0];
+                    a1 += common[k0][1];
+                    a2 += common[k0][2];
+                    const float4 T = __ldg(J.target + pixel);
+                    const int q = nth_set_bit(vm, k0) >> qshift;
+                    _Pragma("unroll 1") for (int z = nextq; z < q; ++z) push_pair(h, z, 0.0);
+                    if (kND > 0) {
+                        const float3 res = f3(fixed_diff(a0, T.x, unsigned(spp), inv), fixed_diff(a1, T.y, unsigned(spp), inv),
+                                              fixed_diff(a2, T.z, unsigned(spp), inv));
+                        push_pair(h, q, double(fmaf(res.x, res.x, fmaf(res.y, res.y, res.z * res.z))));
+#pragma unroll
+                        for (int k = 0; k < kND; ++k) {
+                            unsigned long long d = dacc[h * kND + k][lane] + fix_sum_signed(dhi[k], dlo[k]);
+                            dacc[h * kND + k][lane] = 0ull;
+                            if (nsg > 1) d = groups(d);
+                            gsum[h * kND + k][lane] += double(comp3(res, k % 3) * (signed_word_to_float((long long)d) * inv));
+                        }
+                    } else {
+                        push_pair(h, q, pixel_sq_error(a0, a1, a2, T, unsigned(spp), inv));
+                    }
                 }
-                for (int o = G; o < 32; o <<= 1) {  // the render's other sample groups
-                    acc[0][0] += __shfl_xor_sync(kFull, acc[0][0], o);
-                    acc[0][1] += __shfl_xor_sync(kFull, acc[0][1], o);
-                    acc[0][2] += __shfl_xor_sync(kFull, acc[0][2], o);
+                if (ends) {
+                    nextq = (nth_set_bit(vm, k0) >> qshift) + 1;
+                    ++k0;
+                    s0 = 0;
+                } else {
+                    s0 += i1 - i0;
                 }
-                const float4 T = __ldg(J.target + size_t(py) * J.W + px);
-                for (int h = 0; h < nh; ++h)
-                    e[h] = pixel_sq_error(acc[h][0], acc[h][1], acc[h][2], T, unsigned(J.spp), inv);
-            }
-            for (int h = 0; h < 2; ++h) {  // levels 0-2 of the pairwise sum over this warp's slots
-                double v = e[h];
-                int l = 0;
-                for (; (qq >> l) & 1; ++l) v = Wp.pair[h][l][lane] + v;
-                if (l < 3) Wp.pair[h][l][lane] = v;
-                else sub[h] = v;
+                i0 = i1;
             }
         }
-        for (int h = 0; h < nh; ++h)
-            if (ks == 0 && gi + 32 * h < R) E.sub[warp][gi + 32 * h] = sub[h];
-        __syncthreads();
-        for (int r = threadIdx.x; r < R; r += kGroupBlock)  // a5: levels 3 and 4
-            J.partials[size_t(r) * J.tiles + t] = (E.sub[0][r] + E.sub[1][r]) + (E.sub[2][r] + E.sub[3][r]);
-        __syncthreads();
+        for (int h = 0; h < nh; ++h) {
+            _Pragma("unroll 1") for (int z = nextq; z < qend; ++z) push_pair(h, z, 0.0);
+            if (kND > 0 && ks == 0 && gi + 32 * h < R) {
+#pragma unroll
+                for (int k = 0; k < kND; ++k) replay_store<kND>(J, item, gi + 32 * h, 1 + k, gsum[h * kND + k][lane]);
+            }
+        }
+        __syncwarp();
+        if (J.parts > 1) replay_combine<kND>(J, item, lane);
+    }
     }
     if (kCount) {
         const unsigned v[kNumCounters] = {warp_sum_u(cnt.sph), warp_sum_u(cnt.quad), warp_sum_u(cnt.box),
@@ -2710,11 +3289,12 @@ __global__ void k_philox(unsigned long long seed, unsigned c0, unsigned c1, unsi
 // ---------------------------------------------------------------------------
 // Launch with the programmatic-stream-serialisation attribute (see pdl_enter).
 template <typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(Args...), int grid, int block, cudaStream_t stream, const Args&... args) {
+static cudaError_t launch_pdl_smem(void (*kernel)(Args...), int grid, int block, size_t smem, cudaStream_t stream,
+                                   const Args&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(grid));
     cfg.blockDim = dim3(unsigned(block));
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -2722,6 +3302,10 @@ static cudaError_t launch_pdl(void (*kernel)(Args...), int grid, int block, cuda
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... Args>
+static cudaError_t launch_pdl(void (*kernel)(Args...), int grid, int block, cudaStream_t stream, const Args&... args) {
+    return launch_pdl_smem(kernel, grid, block, 0, stream, args...);
 }
 
 cudaError_t launch_instantiate(const InstLaunch& L, cudaStream_t stream) {
@@ -2750,17 +3334,43 @@ int trace_group_blocks_per_sm() {
     return n > 0 ? n : 1;
 }
 
-int trace_emit_blocks_per_sm() {
+// Kernel variant of a replay launch: bound materials, perturbed primitives, tangent slots. A
+// packed launch runs the variant that covers all of its jobs.
+constexpr size_t kReplaySmemMax = 160 * 1024;
+static_assert(sizeof(ReplayHead) + kReplayTabRows * 16 +
+                      kReplayWarps * replay_warp_bytes(replay_path_granules(64, true), 2, 32, 12) <= kReplaySmemMax,
+              "the largest table, pool (depth 64) and tangent sums fit");
+using ReplayKernel = void (*)(const TraceLaunch);
+template <bool kCount>
+static ReplayKernel replay_kernel_of(const TraceLaunch& L) {
+    if (L.diff_nd == 3) return k_trace_replay<kCount, true, 0, 3>;
+    if (L.diff_nd == 6) return k_trace_replay<kCount, true, 0, 6>;
+    if (L.diff_nd == 12) return k_trace_replay<kCount, true, 0, 12>;
+    if (!L.replay_mat) return L.replay_move == 2 ? k_trace_replay<kCount, false, 2, 0> : k_trace_replay<kCount, false, 1, 0>;
+    return L.replay_move == 2 ? k_trace_replay<kCount, true, 2, 0>
+                              : (L.replay_move ? k_trace_replay<kCount, true, 1, 0> : k_trace_replay<kCount, true, 0, 0>);
+}
+static ReplayKernel replay_kernel(const TraceLaunch& L) {
+    return L.counters ? replay_kernel_of<true>(L) : replay_kernel_of<false>(L);
+}
+
+int trace_replay_blocks_per_sm(const TraceLaunch& L) {
+    const ReplayKernel k = replay_kernel(L);
+    const size_t smem = replay_smem(L);
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_emit<false>, kGroupBlock, 0);
-    return n > 0 ? n : 1;
+    // the same bound for every launch of the kernel: a later one may need more than this one
+    if (smem > kReplaySmemMax ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kReplaySmemMax)) != cudaSuccess)
+        return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kGroupBlock, smem) != cudaSuccess) return 0;
+    return n;
 }
 
 cudaError_t launch_trace(const TraceLaunch& L, bool render_mode, int grid, cudaStream_t stream) {
     if (L.total_items <= 0) return cudaSuccess;
     const bool count = L.counters != nullptr;
     if (L.group == 2 && !render_mode)
-        return launch_pdl(count ? k_trace_emit<true> : k_trace_emit<false>, grid, kGroupBlock, stream, L);
+        return launch_pdl_smem(replay_kernel(L), grid, kGroupBlock, replay_smem(L), stream, L);
     if (L.group && !render_mode)
         return launch_pdl(count ? k_trace_group<true> : k_trace_group<false>, grid, kGroupBlock, stream, L);
     const bool share = !render_mode && L.share;
