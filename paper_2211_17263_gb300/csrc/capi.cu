@@ -583,9 +583,16 @@ cudaError_t timed_trace(prdpt_ctx* c, const TraceLaunch* Ls, int nL, const Trace
     }
     for (int i = 0; i < nL && !render; ++i) {
         if (!Ls[i].share) continue;  // affected paths per render, then their blocks' errors
-        e = launch_trace_affected(Ls[i], grid_for(c, 1 << 30, false, ctas_per_sm), stream);
+        // Every warp of the per-render pass claims entries from some render's list until it has seen
+        // all of them used up, which a small job's full grid spends its time on: at most one warp
+        // per 64 (render, path) pairs (64 x 64 x 4 spp, 8 renders: 456 CTAs 43.1 us a step, 256 38.9,
+        // 171 41.6; larger jobs reach the cap and keep their times), one epilogue warp per block.
+        const TraceJob& J = Ls[i].job0;
+        const long long pairs = (long long)J.W * J.H * J.spp * J.R;
+        const int claims = Ls[i].jobs || pairs / 64 > (1 << 30) ? 1 << 30 : std::max(int(pairs / 64), 1);
+        e = launch_trace_affected(Ls[i], grid_for(c, claims, false, ctas_per_sm), stream);
         if (e != cudaSuccess) return e;
-        e = launch_shared_epilogue(Ls[i], grid_for(c, 1 << 30, false, 0), stream);
+        e = launch_shared_epilogue(Ls[i], grid_for(c, Ls[i].jobs ? 1 << 30 : J.tiles, false, 0), stream);
         if (e != cudaSuccess) return e;
     }
     if (fin) {  // per-render losses, gradient, Adam
