@@ -901,6 +901,7 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         for (int i = 0; i < B.n_prims; ++i) {
             const int m = B.prim_mat[i];
             const float* mp = B.mat_param[m];
+            if ((mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f) && !((prims >> B.prim_slot[i]) & 1u)) J.black = 0;
             if (((prims >> B.prim_slot[i]) & 1u) &&
                 (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f))
                 J.black = 0;

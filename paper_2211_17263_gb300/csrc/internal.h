@@ -188,7 +188,8 @@ struct TraceJob {
     // Replay mode (k_trace_replay): 1 when the job's paths are traced once for all its renders
     // and each render replays what differs (gstride as above, plus two rows of clamp derivatives
     // for the pathwise estimator; items are pixel blocks of all renders, taken from `queue`);
-    // black: every perturbed primitive's material is diffuse and black (and not bound)
+    // black: every perturbed primitive's material is diffuse and black (and not bound), and every
+    // emitter is perturbed
     // a block is `parts` work items (a power of two, at most its pixels), whose sums go through
     // part_sums [tiles][parts][R][1 + nd] when there are several; part_done counts a block's finished
     // parts (zero between launches).

@@ -2078,11 +2078,11 @@ __device__ __forceinline__ bool replay_touch(const ReplayLane& E, float3 o, floa
 }
 
 // One vertex of a path of a replay job (as advance), recording what can differ between the
-// renders. kMat: the job binds albedos; kMove: it perturbs primitives.
-template <bool kCount, bool kMat, bool kMove>
+// renders. kMat: the job binds albedos; kMove: it perturbs primitives (1: every emitter is one).
+template <bool kCount, bool kMat, int kMove>
 __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int rr_start, Path& p, ReplayLane& E,
                                              Counters& cnt) {
-    const Hit h = closest_hit<kCount, kMove>(S, p.o, p.d, cnt, kMove ? E.skip : 0u);
+    const Hit h = closest_hit<kCount, (kMove != 0)>(S, p.o, p.d, cnt, kMove ? E.skip : 0u);
     const bool miss = h.slot < 0;
     const bool touch = kMove && replay_touch<kCount>(E, p.o, p.d, miss ? 3.0e38f : h.t, cnt);
     bool rec = E.rec || touch, bound = false, last = true, rr = false;
@@ -2132,7 +2132,7 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
                 li = nee_light(S, w1.x);
                 const int lslot = S.light[li].y;
                 const float lu = u01(w0.x), lv = u01(w0.y);
-                if (kMove && ((E.skip >> lslot) & 1u)) {  // each render's own estimate
+                if (kMove == 1 || (kMove && ((E.skip >> lslot) & 1u))) {  // each render's own estimate
                     est = 1u;
                     rec = true;
                     vert = shadow_cull(S, E, po, lslot) << (32 - kCullBits);
@@ -2151,7 +2151,7 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
                     float3 wi;
                     float dist, g;
                     int lmat;
-                    if (nee_to<kCount, kMove, false>(S, po, ns, lu, lv, li, cnt, kMove ? E.skip : 0u, nullptr, wi, dist,
+                    if (nee_to<kCount, (kMove != 0), false>(S, po, ns, lu, lv, li, cnt, kMove ? E.skip : 0u, nullptr, wi, dist,
                                                      g, lmat)) {
                         const bool own = kMove && replay_touch<kCount>(E, po, wi, dist, cnt);
                         rec = rec || own;
@@ -2287,8 +2287,9 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
 // albedos. Before, the GI box's renders retraced every path side by side (k_trace_group) and Eq. 9
 // traced each render alone (k_trace): GI box 512 x 512, 32 renders at 32 spp 40.9 -> 16.2 ms, its
 // walls by Eq. 9 87.6 -> 7.5 ms, by Eq. 10 at 256 x 256 11.3 -> 1.26 ms, caustic 512 x 512, 64 renders at
-// 64 spp 7.8 -> 7.3 ms (caustic 237 x 141, 24 renders at 20 spp: 250 -> 258 us, the larger code's
-// cold start). Bound by instruction issue (60 % of cycles, 20 warps per SM): fixed-latency
+// 64 spp 7.8 -> 7.3 ms. Leaving fixed emitters out of the variant for jobs whose emitters all move
+// (80 -> 74 KB of code: instruction fetch is among the largest stalls) took the GI box to 15.1 ms and
+// caustic to 7.0 ms. Bound by instruction issue (60 % of cycles, 20 warps per SM): fixed-latency
 // dependencies and instruction fetch are the largest stalls, phase A takes about a quarter of the
 // GI box's time and half of Eq. 9's. Groups of entries are 16-byte granules because the pool's
 // shared memory sets how many paths fit a batch.
@@ -2384,9 +2385,10 @@ __device__ __forceinline__ float3 replay_alone(const GroupScene& S, int depth, i
     return p.L;
 }
 
-// One render's radiance from a path's chain (without the common part). kMove: 0 no perturbed primitive, 1 only black ones (a render that meets its own
-// primitive ends there), 2 any. Tangent slot k is a parameter of channel k mod 3 (kND: 0 or a
-// multiple of 3); J.mat_slots[m] holds the slots of material m's parameters.
+// One render's radiance from a path's chain (without the common part). kMove: 0 no perturbed
+// primitive, 1 only black ones (a render that meets its own primitive ends there) with every emitter
+// among them, 2 any. Tangent slot k is a parameter of channel k mod 3 (kND: 0 or a multiple of 3);
+// J.mat_slots[m] holds the slots of material m's parameters.
 template <bool kCount, bool kMat, int kMove, int kND>
 __device__ __forceinline__ float3 replay_sample(const GroupScene& S, const TraceJob& J, const GroupLane& gl,
                                                 const float4* ent, const unsigned short* nxt, int i, unsigned pixel,
@@ -2426,7 +2428,7 @@ __device__ __forceinline__ float3 replay_sample(const GroupScene& S, const Trace
                     bool seen = true;
                     float g;
                     int lmat;
-                    if (kMove && est == 1u) {
+                    if (kMove == 1 || (kMove && est == 1u)) {
                         const float4 b = ent[i + 1];
                         float3 ns;
                         float lu, lv;
@@ -2771,7 +2773,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
             bool live = have;
 #pragma unroll 1
             while (__any_sync(kFull, live)) {
-                if (live) live = replay_vertex<kCount, kMat, (kMove != 0)>(E.scene, J.depth, J.rr_start, p, el, cnt) == kLive;
+                if (live) live = replay_vertex<kCount, kMat, kMove>(E.scene, J.depth, J.rr_start, p, el, cnt) == kLive;
             }
             const unsigned fm = __ballot_sync(kFull, el.full), hm = __ballot_sync(kFull, have);
             const int nb = fm ? __ffs(fm) - 1 : __popc(hm);  // the batch: tasks of lanes 0 .. nb - 1
