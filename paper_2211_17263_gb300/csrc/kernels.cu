@@ -2330,17 +2330,22 @@ size_t replay_smem(const TraceLaunch& L) {
 constexpr int replay_min_blocks(bool move) { return move ? 5 : 6; }
 
 // The pool takes the shared memory that replay_min_blocks CTAs per SM (the registers' limit) leave,
-// up to kReplayPoolMax granules: a pool that runs out costs part of a batch's phase A (GI box at
-// 32 renders, 224 granules of 3 float4 instead of 128: 73 -> 27 ms), a CTA less per SM more.
-constexpr int kReplayPoolMax = 512;
+// up to kReplayPoolMax granules, or that fewer CTAs leave where it would be too small to hold a
+// batch of common paths: a pool that runs out costs part of a batch's phase A (GI box at 32
+// renders, 224 granules of 3 float4 instead of 128: 73 -> 27 ms), a CTA less per SM a tenth or so
+// (Eq. 9 on the box's walls with 44 renders, whose sums fill 6 CTAs' shared memory: 232 x 274 at 50 spp
+// 29.9 ms with 24 granules, 5.2 ms with what 3 CTAs leave; 64 renders, 256 x 256 at 16 spp, 10.9 and 1.9).
+constexpr int kReplayPoolMax = 512, kReplayPoolMove = 256, kReplayPoolFixed = 128;
 int replay_pool(const TraceLaunch& L) {
-    const size_t kCta = 227 * 1024 / replay_min_blocks(L.replay_move != 0) - 1024;  // 1 KB is the system's
     const size_t head = sizeof(ReplayHead) + size_t(L.tab_rows) * 16;
     const size_t rest = replay_warp_bytes(0, L.halves, L.pixels, L.diff_nd);
+    const int need = (L.pool + 7) & ~7, want = L.replay_move ? kReplayPoolMove : kReplayPoolFixed;
     int fits = 0;
-    if (kCta > head + kReplayWarps * rest) fits = int((kCta - head - kReplayWarps * rest) / (18 * kReplayWarps));
+    for (int ctas = replay_min_blocks(L.replay_move != 0); ctas >= 2 && fits < want; --ctas) {
+        const size_t cta = 227 * 1024 / ctas - 1024;  // 1 KB of a CTA's is the system's
+        if (cta > head + kReplayWarps * rest) fits = int((cta - head - kReplayWarps * rest) / (18 * kReplayWarps));
+    }
     fits = fits < kReplayPoolMax ? fits : kReplayPoolMax;
-    const int need = (L.pool + 7) & ~7;
     return fits > need ? fits & ~7 : need;
 }
 
