@@ -456,10 +456,10 @@ int choose_replay_block(prdpt_ctx* c, int requested, int W, int H, int spp) {
 // Work items per block in replay mode: the fewest that do the same for the block size a caller asked
 // for (caustic 237 x 141 at 20 spp, 24 renders, blocks of 32 pixels: 0.68 ms whole, 0.27 ms in 8
 // parts; their sums meet in memory, which costs small blocks 5 %, so the choice above comes first).
-int replay_parts(prdpt_ctx* c, int px, int tiles, int spp) {
+int replay_parts(prdpt_ctx* c, int px, int tiles, int spp, int chunks) {
     const long long warps = (long long)c->sms * kReplayWarpsPerSm;
     int parts = 1;
-    while (2 * parts <= px && (long long)tiles * parts < 8 * warps && (long long)px / (2 * parts) * spp >= 64) parts *= 2;
+    while (chunks == 1 && 2 * parts <= px && (long long)tiles * parts < 8 * warps && (long long)px / (2 * parts) * spp >= 64) parts *= 2;
     return parts;
 }
 
@@ -520,7 +520,7 @@ int grid_for_group(prdpt_ctx* c, int items, int ctas_per_sm) {
 // Persistent grid of the replay kernel: one work item per warp of CTAs of kGroupBlock threads
 // (ctas_per_sm counts 256-thread CTAs, as above). 0: the kernel cannot run with its shared memory.
 int grid_for_replay(prdpt_ctx* c, const TraceLaunch& L, int ctas_per_sm) {
-    const unsigned long long key = (unsigned long long)replay_smem(L) << 9 | (L.halves > 1 ? 256u : 0u) | unsigned(L.diff_nd) << 4 |
+    const unsigned long long key = (unsigned long long)replay_smem(L) << 10 | (L.halves > 1 ? 256u : 0u) | (L.replay_chunked ? 512u : 0u) | unsigned(L.diff_nd) << 4 |
                                    (L.replay_mat ? 8u : 0u) | (L.counters ? 4u : 0u) | unsigned(L.replay_move);
     auto it = c->occ_replay.find(key);
     if (it == c->occ_replay.end()) it = c->occ_replay.emplace(key, trace_replay_blocks_per_sm(L)).first;
@@ -538,6 +538,7 @@ void replay_cover(TraceLaunch& L, const TraceJob& J) {
     L.halves = std::max(L.halves, J.R > 32 ? 2 : 1);
     L.tab_rows = std::max(L.tab_rows, J.R * J.gstride);
     L.pixels = std::max(L.pixels, J.bw * J.bh / J.parts);
+    L.replay_chunked |= J.chunks > 1 ? 1 : 0;
     L.pool = std::max(L.pool, replay_path_granules(J.depth, J.n_var > 0));
     if (J.diff) L.diff_nd = J.nd;
     L.pool = replay_pool(L);
@@ -546,7 +547,7 @@ void replay_cover(TraceLaunch& L, const TraceJob& J) {
 // Work items of a gradient job's render launch: pixel blocks (path sharing, replay),
 // (block, group of gsize renders) (render-group mode) or (render, block).
 long long job_items(const TraceJob& J) {
-    if (J.emit) return (long long)J.tiles * J.parts;
+    if (J.emit) return (long long)J.tiles * J.parts * J.chunks;
     if (J.share) return J.tiles;
     if (J.gsize > 0) return (long long)J.tiles * (J.R / J.gsize);
     return (long long)J.R * J.tiles;
@@ -822,8 +823,8 @@ static void fill_share(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     }
     // Only albedos bound: path sharing would trace every path that meets a bound material again
     // in every render; replay (fill_group) traces it once.
-    if (J.n_var == 0 && o->render_groups >= 0 && 2 * o->pairs <= 64 && B.n_prims <= kGroupPrims &&
-        B.n_mats <= kGroupMats) {
+    if (J.n_var == 0 && o->render_groups >= 0 && 2 * o->pairs * __builtin_popcount(J.var_mats) <= kReplayTabRows &&
+        B.n_prims <= kGroupPrims && B.n_mats <= kGroupMats) {
         J.var_mats = 0u;
         return;
     }
@@ -843,6 +844,7 @@ static void fill_share(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
 static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o) {
     J.black = 0;
     J.parts = 1;
+    J.chunks = 1;
     J.gsize = 0;
     J.gstride = 0;
     J.emit = 0;
@@ -879,7 +881,7 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     const int stride = rows + nm + (radius ? 2 : 0);
     if (n + nm == 0) return;
     const int R = J.R;
-    // Replay (k_trace_replay): at most 64 renders whose rows fit; every path is traced once and
+    // Replay (k_trace_replay): renders whose rows fit, at most 64 at a time; every path is traced once and
     // each render replays what differs (path sharing's switch turns it off). The pathwise
     // estimator's rows also hold the parameters' clamp derivatives, by tangent slot.
     int per_channel[3] = {0, 0, 0};
@@ -895,8 +897,11 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     }
     J.nd = J.nd <= 2 ? 3 * J.nd : (J.nd <= 4 ? 12 : 0);  // 0, 3, 6 or 12
     const int rstride = stride + (J.nd + 3) / 4;
-    if (!o->no_path_sharing && (!pathwise || J.nd > 0) && R >= 1 && R <= 64 && R * rstride <= kReplayTabRows) {
+    // (Beyond 64 renders only with bound materials: a path is then traced once per 64 renders, which
+    // still beats render groups -- GI box 256 x 256 at 16 spp, 80 renders: 13.6 -> 5.0 ms.)
+    if (!o->no_path_sharing && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
         J.emit = 1;
+        J.chunks = (R + 63) / 64;
         J.black = 1;
         for (int i = 0; i < B.n_prims; ++i) {
             const int m = B.prim_mat[i];
@@ -1155,7 +1160,7 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
-    if (prdpt_status st = check_items(per_block ? (long long)tiles : (long long)R * tiles)) return st;
+    if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) return st;
     if (probe.share) {
         const size_t pix = (size_t)o->width * o->height;
         if (prdpt_status st = grow(c, &c->s_share, &c->s_share_n, (size_t)tiles * 96)) return st;
@@ -1172,7 +1177,7 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
     if (prdpt_status st = grow(c, &c->s_partials, &c->s_partials_n, (size_t)R * tiles)) return st;
     if (prdpt_status st = grow(c, &c->s_losses, &c->s_losses_n, (size_t)R)) return st;
     if (probe.emit) {
-        probe.parts = replay_parts(c, px, tiles, o->spp);
+        probe.parts = replay_parts(c, px, tiles, o->spp, probe.chunks);
         if (probe.parts > 1 &&  // (without room for the parts' sums the blocks stay whole)
             (grow(c, &c->s_psums, &c->s_psums_n, replay_part_sums(probe, tiles)) != PRDPT_OK ||
              grow_zeroed(c, &c->s_pdone, &c->s_pdone_n, (size_t)tiles) != PRDPT_OK))
@@ -1453,7 +1458,7 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
     int bw, bh, tiles_x, tiles;
     tiles_for(px, W, H, &bw, &bh, &tiles_x, &tiles);
-    if (prdpt_status st = check_items(per_block ? (long long)tiles : (long long)R * tiles)) {
+    if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) {
         delete j;
         return st;
     }
@@ -1489,7 +1494,7 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     const size_t off_bs = (off_nr + (tex ? sizeof(HdNorm) * (size_t)R : 0) + 255) & ~size_t(255);
     const size_t off_ps = (off_bs + sizeof(BaseScene) + 255) & ~size_t(255);  // after the job's own copy of its scene
     // replay mode: the sums of the blocks' parts and their counters
-    if (probe.emit) probe.parts = replay_parts(c, px, tiles, o->spp);
+    if (probe.emit) probe.parts = replay_parts(c, px, tiles, o->spp, probe.chunks);
     const size_t off_pd = (off_ps + sizeof(double) * replay_part_sums(probe, tiles) + 255) & ~size_t(255);
     size_t total = off_bs + sizeof(BaseScene);
     void* base = nullptr;
@@ -1862,6 +1867,8 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
                 T.tab_rows = c->batch_replay.tab_rows;
                 T.pool = c->batch_replay.pool;
                 T.halves = c->batch_replay.halves;
+                T.replay_chunked = c->batch_replay.replay_chunked;
+                if (T.replay_chunked) T.replay_mat = 1;  // (the chunked variants replay throughputs)
                 T.pixels = c->batch_replay.pixels;
             }
             T.queue = queues[kd];

@@ -193,7 +193,7 @@ struct TraceJob {
     // a block is `parts` work items (a power of two, at most its pixels), whose sums go through
     // part_sums [tiles][parts][R][1 + nd] when there are several; part_done counts a block's finished
     // parts (zero between launches).
-    int emit, black, parts;
+    int emit, black, parts, chunks;  // chunks: of 64 renders each (several: parts is 1)
     double* part_sums;
     unsigned* part_done;
     // pathwise estimator in replay mode: tangent slot k holds parameter slot_param[k] (-1: none) of
@@ -216,6 +216,7 @@ struct TraceLaunch {
     // black ones, 2 any), float4 of the per-render table, entries of a warp's pool, 32-render
     // halves of a warp's sums, pixels of a work item at most
     int replay_mat, replay_move, tab_rows, pool, halves, pixels;
+    int replay_chunked;       // a job has more than 64 renders (bound materials)
     int fin_total;            // packed launch: finalisation CTAs (sum of R over jobs)
     unsigned* queue;          // work-queue head, zeroed by the instantiation launch
     unsigned long long* counters;  // [8] or null (null: the uncounted kernel variant runs)

@@ -2263,7 +2263,7 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
 // Under common random numbers the renders of a job differ only where a perturbed primitive
 // meets a ray, where an emitter that moved is sampled, and in the albedos that are bound. A
 // work item is one of a pixel block's J.parts parts (1/parts of the positions of the bit-reversed
-// slot order) for all R <= 64 renders, taken by one warp, which takes the part's (pixel, sample)
+// slot order) for all R <= 64 renders (more: 64 of them), taken by one warp, which takes the part's (pixel, sample)
 // tasks in batches of 32, pixels in that order:
 //   phase A  lane = task: the path is traced once in the invariant scene (replay_vertex). What
 //            is the same in every render goes into the pixel's common sum, the rest into a
@@ -2603,7 +2603,8 @@ __device__ __noinline__ void replay_combine(const TraceJob& J, unsigned item, in
     if (lane == 0) J.part_done[t] = 0u;  // ready for the next launch
 }
 
-template <bool kCount, bool kMat, int kMove, int kND>
+// kChunked: jobs of more than 64 renders (a variant of its own: the chunk costs the others 1 %).
+template <bool kCount, bool kMat, int kMove, int kND, bool kChunked>
 __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_trace_replay(const __grid_constant__ TraceLaunch L) {
     extern __shared__ __align__(16) unsigned char s_replay[];
     ReplayHead& E = *reinterpret_cast<ReplayHead*>(s_replay);
@@ -2634,11 +2635,11 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
         if (jb == 0) pdl_enter();
         __syncthreads();
     }
-    if (threadIdx.x == 0) E.left = __ldcg(J.queue) < unsigned(J.tiles * J.parts) ? 1u : 0u;
+    if (threadIdx.x == 0) E.left = __ldcg(J.queue) < unsigned(J.tiles * J.parts * J.chunks) ? 1u : 0u;
     __syncthreads();
     if (!E.left) continue;
     const int n = J.n_var, nr = J.var_rows, nm = __popc(J.var_mats), stride = J.gstride, ncl = (kND + 3) / 4;
-    if (J.R < 1 || J.R > 32 * halves || J.R * stride > L.tab_rows || stride < nr + nm + ncl || n < 0 ||
+    if (J.R < 1 || J.R > 64 * J.chunks || (!kChunked && J.chunks > 1) || (J.R > 32 && halves < 2) || (J.chunks > 1 && J.parts > 1) || J.R * stride > L.tab_rows || stride < nr + nm + ncl || n < 0 ||
         n > kMaxVariant || J.n_prims > kGroupPrims || J.n_mats > kGroupMats || (!kMat && nm) || (!kMove && n) ||
         (kMove == 1 && !J.black && n) || J.parts < 1 || J.parts > J.bw * J.bh ||
         J.bw * J.bh > L.pixels * J.parts || (J.parts & (J.parts - 1)) != 0 || replay_path_granules(J.depth, kMove != 0) > L.pool) {
@@ -2711,9 +2712,13 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
         unsigned item = 0;
         if (lane == 0) item = atomicAdd(J.queue, 1u);
         item = __shfl_sync(kFull, item, 0);
-        if (item >= unsigned(J.tiles * J.parts)) break;
+        // jobs of more than 64 renders: every block once per chunk of 64
+        const unsigned units = unsigned(J.tiles * J.parts), chunk = kChunked ? item / units : 0u;
+        if (kChunked ? int(chunk) >= J.chunks : item >= units) break;
+        if (kChunked) item -= chunk * units;
+        const int r0 = int(chunk) * 64;
         const int t = int(item) / J.parts, q0 = (int(item) - t * J.parts) * (qend << qshift);
-        const int R = J.R, nh = R > 32 ? 2 : 1, spp = J.spp;
+        const int R = kChunked ? min(J.R - r0, 64) : J.R, nh = R > 32 ? 2 : 1, spp = J.spp;
         // phase B lanes: render gi of sample group ks; with R < 32, nsg = floor(32 / R) samples
         // side by side (lanes beyond nsg R idle)
         const int G = R < 32 ? R : 32, nsg = 32 / G, gi = lane % G, ks = lane / G;
@@ -2746,7 +2751,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
 #pragma unroll 1
             for (; (q >> l) & 1; ++l) v = s[l][lane] + v;
             if (q + 1 < qend) s[l][lane] = v;
-            else if (ks == 0 && gi + 32 * h < R) replay_store<kND>(J, item, gi + 32 * h, 0, v);  // a5
+            else if (ks == 0 && gi + 32 * h < R) replay_store<kND>(J, item, r0 + gi + 32 * h, 0, v);  // a5
         };
         int k0 = 0, s0 = 0;    // the next task: pixel k0 of the block, sample s0
         int nextq = 0;         // positions below are summed
@@ -2814,8 +2819,8 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
 #pragma unroll 1
                 for (int h = 0; h < nh; ++h) {
                     const int r = gi + 32 * h;
-                    const GroupLane gl{tab + (r < R ? r : 0), J.var_prims, J.var_mats, J.var_offs, J.var_rows, areas,
-                                       nullptr, 0, R};
+                    const GroupLane gl{tab + r0 + (r < R ? r : 0), J.var_prims, J.var_mats, J.var_offs, J.var_rows, areas,
+                                       nullptr, 0, kChunked ? J.R : R};
                     unsigned hi0 = 0u, hi1 = 0u, hi2 = 0u, lo0 = 0u, lo1 = 0u, lo2 = 0u;
                     unsigned dhi[kND > 0 ? kND : 1], dlo[kND > 0 ? kND : 1];
 #pragma unroll
@@ -2906,7 +2911,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
             _Pragma("unroll 1") for (int z = nextq; z < qend; ++z) push_pair(h, z, 0.0);
             if (kND > 0 && ks == 0 && gi + 32 * h < R) {
 #pragma unroll
-                for (int k = 0; k < kND; ++k) replay_store<kND>(J, item, gi + 32 * h, 1 + k, gsum[h * kND + k][lane]);
+                for (int k = 0; k < kND; ++k) replay_store<kND>(J, item, r0 + gi + 32 * h, 1 + k, gsum[h * kND + k][lane]);
             }
         }
         __syncwarp();
@@ -3350,12 +3355,18 @@ static_assert(sizeof(ReplayHead) + kReplayTabRows * 16 +
 using ReplayKernel = void (*)(const TraceLaunch);
 template <bool kCount>
 static ReplayKernel replay_kernel_of(const TraceLaunch& L) {
-    if (L.diff_nd == 3) return k_trace_replay<kCount, true, 0, 3>;
-    if (L.diff_nd == 6) return k_trace_replay<kCount, true, 0, 6>;
-    if (L.diff_nd == 12) return k_trace_replay<kCount, true, 0, 12>;
-    if (!L.replay_mat) return L.replay_move == 2 ? k_trace_replay<kCount, false, 2, 0> : k_trace_replay<kCount, false, 1, 0>;
-    return L.replay_move == 2 ? k_trace_replay<kCount, true, 2, 0>
-                              : (L.replay_move ? k_trace_replay<kCount, true, 1, 0> : k_trace_replay<kCount, true, 0, 0>);
+    if (L.replay_chunked)
+        return L.replay_move == 2 ? k_trace_replay<kCount, true, 2, 0, true>
+                                  : (L.replay_move ? k_trace_replay<kCount, true, 1, 0, true>
+                                                   : k_trace_replay<kCount, true, 0, 0, true>);
+    if (L.diff_nd == 3) return k_trace_replay<kCount, true, 0, 3, false>;
+    if (L.diff_nd == 6) return k_trace_replay<kCount, true, 0, 6, false>;
+    if (L.diff_nd == 12) return k_trace_replay<kCount, true, 0, 12, false>;
+    if (!L.replay_mat)
+        return L.replay_move == 2 ? k_trace_replay<kCount, false, 2, 0, false> : k_trace_replay<kCount, false, 1, 0, false>;
+    return L.replay_move == 2 ? k_trace_replay<kCount, true, 2, 0, false>
+                              : (L.replay_move ? k_trace_replay<kCount, true, 1, 0, false>
+                                               : k_trace_replay<kCount, true, 0, 0, false>);
 }
 static ReplayKernel replay_kernel(const TraceLaunch& L) {
     return L.counters ? replay_kernel_of<true>(L) : replay_kernel_of<false>(L);

@@ -103,6 +103,38 @@ def test_replay_is_bit_identical(ctx, make, pairs, spp, block_pixels):
 
 
 @pytest.mark.parametrize("make", [_gi, _walls, _box_light_wall])
+@pytest.mark.parametrize("pairs,block_pixels", [(33, 8), (40, 32), (70, 0)])
+def test_more_than_64_renders_in_chunks(ctx, make, pairs, block_pixels):
+    """Jobs with bound materials replay 64 renders at a time (chunks of 64 and the rest)."""
+    wl = make(width=29, height=13, spp=5, pairs=pairs)
+    scene = ctx.upload_scene(wl.scene, wl.bindings)
+    target = _t(np.random.default_rng(1).uniform(size=(wl.height, wl.width, 4)))
+    out = []
+    for kw in ({}, dict(no_path_sharing=1, render_groups=-1)):
+        g, L = scene.smoothed_grad(_t(wl.theta0), _t(wl.sigma), target,
+                                   scene.grad_opts(wl, step=3, block_pixels=block_pixels or 8, **kw))
+        torch.cuda.synchronize()
+        out.append((g.cpu().numpy(), L.cpu().numpy()))
+    assert np.array_equal(out[0][1], out[1][1]) and np.array_equal(out[0][0], out[1][0])
+    # packed with a job of few renders: each as alone
+    from paper_2211_17263_gb300 import api
+    small = make(width=29, height=13, spp=5, pairs=3)
+    state = []
+    for packed in (False, True):
+        jobs = [api.Job(ctx.upload_scene(w.scene, w.bindings), w, target.cpu().numpy()) for w in (wl, small)]
+        if packed:
+            api.step_batch(ctx, jobs)
+        else:
+            for j in jobs:
+                j.step()
+        state.append([j.read() for j in jobs])
+        for j in jobs:
+            j.release()
+    for a, b in zip(*state):
+        assert all(np.array_equal(a[k], b[k]) for k in ("theta", "grad", "losses"))
+
+
+@pytest.mark.parametrize("make", [_gi, _walls, _box_light_wall])
 def test_long_paths_fill_the_pool(ctx, make):
     """Depth 64 without roulette: a batch's paths do not fit the pool and are taken in smaller batches."""
     wl = make(width=16, height=12, spp=32, pairs=4, depth=64, rr_start=-1)
