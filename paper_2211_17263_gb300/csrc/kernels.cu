@@ -118,8 +118,8 @@ __device__ __forceinline__ uint4 philox(uint4 c, unsigned k0, unsigned k1) {
 }
 
 // The same generator kept out of line: one copy of its code instead of one per call site,
-// for the kernels whose code outgrows the instruction cache (emitter sharing, render groups;
-// measured: caustic step 7.16 -> 6.72 ms).
+// for the kernels whose code outgrows the instruction cache (replay, render groups; measured on
+// an earlier kernel for caustic: 7.16 -> 6.72 ms a step; the per-render kernel is 4 % faster inline).
 __device__ __noinline__ uint4 philox_ool(uint4 c, unsigned k0, unsigned k1) { return philox(c, k0, k1); }
 
 // ((x >> 9) * 2 + 1) / 2^24: exact in FP32, never 0, 1 or 1/2.
@@ -2188,7 +2188,7 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
     E.rec = rec;
     if (total) {
         int i = int(atomicAdd(E.ctr, unsigned(total)));
-        if (i + total > E.cap) {
+        if (unsigned(i) >= unsigned(E.cap) || i + total > E.cap) {
             E.full = true;
             return kEnded;
         }
@@ -2300,7 +2300,7 @@ constexpr int kReplayWarps = kGroupBlock / 32;
 //   u64 acc[halves][3][32]            radiance of the current pixel, 2^-32 fixed point
 //   u64 dacc[halves][nd][32]          Eq. 9: its tangent sums
 //   double gsum[halves][nd][32]       Eq. 9: the block's gradient partials
-//   u64 common[pixels][3]             radiance common to all renders, per pixel of the block
+//   u64 common[replay_common][3]             radiance common to all renders, per pixel of the block
 //   float4 ent[pool], u16 nxt[pool], u16 first[32], unsigned ctr
 struct ReplayHead {
     GroupScene scene;  // the invariant part (render 0's records of the other primitives)
@@ -2315,9 +2315,15 @@ static_assert(sizeof(ReplayHead) % 16 == 0, "float4 arrays follow");
 __host__ __device__ constexpr int replay_levels(int pixels) {
     return pixels <= 1 ? 0 : (pixels <= 2 ? 1 : (pixels <= 4 ? 2 : (pixels <= 8 ? 3 : (pixels <= 16 ? 4 : 5))));
 }
+// Entries of `common`: the pixels, rounded up to an even number so that the pool after it is aligned.
+__host__ __device__ constexpr int replay_common(int pixels) { return pixels + (pixels & 1); }
 __host__ __device__ constexpr size_t replay_warp_bytes(int pool, int halves, int pixels, int nd) {
-    return size_t(halves) * (replay_levels(pixels) + 3 + 2 * nd) * 256 + ((size_t(pixels) * 24 + 15) & ~size_t(15)) + size_t(pool) * 18 + 80;
+    return size_t(halves) * (replay_levels(pixels) + 3 + 2 * nd) * 256 + size_t(replay_common(pixels)) * 24 + size_t(pool) * 18 + 80;
 }
+// (pool in multiples of 8: 16-byte alignment throughout)
+static_assert(replay_warp_bytes(8, 1, 1, 0) % 16 == 0 && replay_warp_bytes(8, 1, 2, 3) % 16 == 0 &&
+                  replay_warp_bytes(24, 2, 4, 6) % 16 == 0 && replay_warp_bytes(512, 2, 32, 12) % 16 == 0,
+              "the next warp's sums are aligned");
 size_t replay_smem(const TraceLaunch& L) {
     return sizeof(ReplayHead) + size_t(L.tab_rows) * 16 +
            kReplayWarps * replay_warp_bytes(L.pool, L.halves, L.pixels, L.diff_nd);
@@ -2618,7 +2624,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
     unsigned long long (*dacc)[32] = acc + halves * 3;
     double (*gsum)[32] = reinterpret_cast<double (*)[32]>(dacc + halves * kND);
     unsigned long long (*common)[3] = reinterpret_cast<unsigned long long (*)[3]>(gsum + halves * kND);
-    float4* ent = reinterpret_cast<float4*>(common + L.pixels + (L.pixels & 1));
+    float4* ent = reinterpret_cast<float4*>(common + replay_common(L.pixels));
     unsigned short* nxt = reinterpret_cast<unsigned short*>(ent + L.pool);
     unsigned short* firsts = nxt + L.pool;
     unsigned* ctr = reinterpret_cast<unsigned*>(firsts + 32);

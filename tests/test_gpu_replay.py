@@ -134,6 +134,20 @@ def test_more_than_64_renders_in_chunks(ctx, make, pairs, block_pixels):
         assert all(np.array_equal(a[k], b[k]) for k in ("theta", "grad", "losses"))
 
 
+@pytest.mark.parametrize("make", [_gi, _walls, _light, _two_lights])
+@pytest.mark.parametrize("spp,block_pixels", [(64, 0), (65, 8), (32, 0), (16, 16)])
+def test_items_of_one_two_and_four_pixels(ctx, make, spp, block_pixels):
+    """Small images with many samples: blocks, or parts of blocks, of 1, 2 and 4 pixels. With
+    block_pixels = 0 the blocks differ from the per-render kernel's, so its FP64 partial sums are
+    grouped differently: the FP32 losses may then differ in their last bit."""
+    wl = make(width=23, height=9, spp=spp, pairs=3)
+    (g, L), (g0, L0) = _compare(ctx, wl, block_pixels)
+    if block_pixels:
+        assert np.array_equal(L, L0) and np.array_equal(g, g0)
+    else:
+        assert np.allclose(L, L0, rtol=2.0**-22, atol=0.0)
+
+
 @pytest.mark.parametrize("make", [_gi, _walls, _box_light_wall])
 def test_long_paths_fill_the_pool(ctx, make):
     """Depth 64 without roulette: a batch's paths do not fit the pool and are taken in smaller batches."""
