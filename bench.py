@@ -164,8 +164,8 @@ def _profiled(workload_name, key):
 
 
 def _emitter_bound(wl):
-    """Does a position or radius binding move an emitter (the emitter-sharing mode's jobs;
-    geometry-only jobs share paths through the shared-pass pipeline)?"""
+    """Does a position or radius binding move an emitter (such jobs replay paths; jobs that move
+    other geometry only share paths through the shared-pass pipeline)?"""
     import workloads
     sc = wl.scene
     for kind, idx, _ in np.asarray(wl.bindings):
@@ -175,12 +175,20 @@ def _emitter_bound(wl):
     return False
 
 
+def _shared_pass(wl):
+    """Does the workload run path sharing's pipeline when paths are shared (geometry moves, no
+    emitter does)?"""
+    import workloads
+    moves = np.isin(np.asarray(wl.bindings)[:, 0], (workloads.BIND_PRIM_POS, workloads.BIND_SPHERE_RADIUS))
+    return bool(moves.any()) and not _emitter_bound(wl)
+
+
 def _launches_per_step(wl, sharing):
     """The library's kernel launches in one resident step: sampler, render kernel,
     finalisation; path sharing adds the per-render and epilogue passes (replay and
     render groups run one render kernel); texture scenes add the D-dimensional draws and gradient kernels."""
     import workloads
-    n = 5 if sharing and not _emitter_bound(wl) else 3
+    n = 5 if sharing and _shared_pass(wl) else 3
     if wl.D > 64:
         n += 3 if wl.sampler == workloads.SAMPLER_RADIAL else 2
     return n
@@ -521,9 +529,8 @@ def main():
         achieved = fp32_counted / (trace_avg_ms * 1e-3) / 1e12 if fp32_counted else model_achieved
         value = world * 1000.0 / step_ms
         traffic = _profiled(wl.name, "dram_bytes_per_step")
-        replayed = (wl.crn and wl.D <= 64 and wl.renders <= 64 and shape["render_groups"] >= 0
-                    and not shape["no_path_sharing"])
-        if sharing and not _emitter_bound(wl):
+        replayed = sharing and not _shared_pass(wl)  # each path traced once for all renders
+        if sharing and _shared_pass(wl):
             kernels = "render pipeline (k_trace shared pass, k_trace_affected, k_shared_epilogue, k_finalize)"
         elif replayed:
             kernels = "replay kernel k_trace_replay + k_finalize"

@@ -6,8 +6,8 @@ persistent grid keeps per SM (the number of live warps), whether renders are tra
 by side in one warp (render_groups = 0: automatic group size; -1: one render per work
 item), and whether paths are shared across renders where the job allows it
 (no_path_sharing = 0: paths no perturbation can reach traced once for geometry-only
-perturbations; each path traced once with each render's own next-event estimates when only
-emitters move) or every render traces its own. Each
+perturbations; each path traced once and replayed by every render for the other jobs) or
+every render traces its own. Each
 candidate is timed with CUDA events on the render launches of a throwaway resident job of
 the same shape; the fastest is cached in a JSON file keyed by the shape, so later jobs of
 that shape start from the tuned launch (api.Job looks it up when given no shape). The CTA
