@@ -463,6 +463,13 @@ int replay_parts(prdpt_ctx* c, int px, int tiles, int spp, int chunks) {
     return parts;
 }
 
+// The per-render kernel's block size where replay's own choice is a smaller one, else 0. Smaller
+// blocks have more partials: a call whose partials the memory budget then refuses takes this size.
+int choose_whole_block(prdpt_ctx* c, const prdpt_grad_opts* o, int px) {
+    const int whole = choose_block(c, o->block_pixels, 2 * o->pairs, o->width, o->height, false);
+    return px < whole ? whole : 0;
+}
+
 size_t replay_part_sums(const TraceJob& J, int tiles) {  // doubles of a replay job's part sums
     return J.parts > 1 ? size_t(tiles) * J.parts * J.R * (1 + J.nd) : 0;
 }
@@ -1142,9 +1149,10 @@ struct AdamDev {
     float lr, b1, b2, eps;
 };
 
-prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* theta_dev, const float* sigma_dev,
+// *whole: replay chose smaller blocks than the per-render kernel would take (choose_whole_block).
+prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* theta_dev, const float* sigma_dev,
                                   const prdpt_grad_opts* o, const float* target_dev, float* grad_dev,
-                                  float* losses_dev, void* stream, const AdamDev* adam = nullptr) {
+                                  float* losses_dev, void* stream, const AdamDev* adam, int* whole) {
     Scene* s = get_scene(c, scene_id);
     if (!s) return fail(PRDPT_E_NOT_FOUND, "unknown scene");
     if (prdpt_status st = check_grad_opts(o)) return st;
@@ -1158,6 +1166,7 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
     const bool per_block = probe.share || probe.emit;
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
+    *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
     if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) return st;
@@ -1306,6 +1315,18 @@ prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* t
     return PRDPT_OK;
 }
 
+prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* theta_dev, const float* sigma_dev,
+                                  const prdpt_grad_opts* o, const float* target_dev, float* grad_dev,
+                                  float* losses_dev, void* stream, const AdamDev* adam = nullptr) {
+    int whole = 0;
+    const prdpt_status st = smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, o, target_dev, grad_dev, losses_dev,
+                                                 stream, adam, &whole);
+    if (st != PRDPT_E_OUT_OF_BUDGET || !whole) return st;  // (refused before anything was enqueued)
+    prdpt_grad_opts w = *o;
+    w.block_pixels = whole;
+    return smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, &w, target_dev, grad_dev, losses_dev, stream, adam, &whole);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1434,10 +1455,9 @@ prdpt_status prdpt_adam_step(prdpt_ctx* c, int32_t D, float* theta_dev, float* m
     return PRDPT_OK;
 }
 
-prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_desc* d, int32_t* job_out) {
-    if (!c || !d || !job_out || !d->theta0_host || !d->sigma0_host)
-        return fail(PRDPT_E_INVALID_ARG, "NULL argument");
-    std::lock_guard<std::mutex> lk(c->mu);
+// prdpt_job_create with the context's mutex held; *whole as for smoothed_grad_blocks
+static prdpt_status job_create_blocks(prdpt_ctx* c, int32_t scene_id, const prdpt_job_desc* d, int32_t* job_out,
+                                      int* whole) {
     Scene* s = get_scene(c, scene_id);
     if (!s) return fail(PRDPT_E_NOT_FOUND, "unknown scene");
     const prdpt_grad_opts* o = &d->grad;
@@ -1456,6 +1476,7 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     const bool per_block = probe.share || probe.emit;
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
+    *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, W, H, &bw, &bh, &tiles_x, &tiles);
     if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) {
@@ -1667,6 +1688,18 @@ prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_de
     c->jobs.push_back(j);
     *job_out = (int)c->jobs.size() - 1;
     return PRDPT_OK;
+}
+
+prdpt_status prdpt_job_create(prdpt_ctx* c, int32_t scene_id, const prdpt_job_desc* d, int32_t* job_out) {
+    if (!c || !d || !job_out || !d->theta0_host || !d->sigma0_host)
+        return fail(PRDPT_E_INVALID_ARG, "NULL argument");
+    std::lock_guard<std::mutex> lk(c->mu);
+    int whole = 0;
+    const prdpt_status st = job_create_blocks(c, scene_id, d, job_out, &whole);
+    if (st != PRDPT_E_OUT_OF_BUDGET || !whole) return st;
+    prdpt_job_desc w = *d;
+    w.grad.block_pixels = whole;
+    return job_create_blocks(c, scene_id, &w, job_out, &whole);
 }
 
 // Draws of a texture job's step by the high-dimensional kernels (from its sampler setup).

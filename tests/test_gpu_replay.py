@@ -167,3 +167,38 @@ def test_pathwise_replay(ctx, slots, pairs, spp):
     (g, L), (g0, L0) = _compare(ctx, wl, 8)
     assert np.array_equal(L, L0)
     assert np.linalg.norm(g - g0) <= 3 * 8 * 2.0**-24 * 8 * np.linalg.norm(g0)
+
+
+def test_whole_blocks_where_the_budget_refuses_small_ones(gpu_lib):
+    """A small image's one-pixel blocks have up to 32 times the partials; a call that the memory
+    budget would then refuse takes the per-render kernel's blocks instead, as a job and as a gradient."""
+    from paper_2211_17263_gb300 import api
+    wl = _gi(width=120, height=100, spp=64, pairs=32)
+    target = _t(np.random.default_rng(1).uniform(size=(wl.height, wl.width, 4)))
+
+    def run(ctx, job):
+        scene = ctx.upload_scene(wl.scene, wl.bindings)
+        if job:
+            j = api.Job(scene, wl, target.cpu().numpy(), use_tuned=False)
+            j.step()
+            return j.read()["grad"]
+        g, _ = scene.smoothed_grad(_t(wl.theta0), _t(wl.sigma), target, scene.grad_opts(wl))
+        torch.cuda.synchronize()
+        return g.cpu().numpy()
+
+    for job in (True, False):
+        ctx = api.Context(0, hbm_budget_bytes=200 << 20)
+        try:
+            grad = run(ctx, job)
+            used = ctx.memory_used()
+        finally:
+            ctx.close()
+        # one-pixel blocks: 12000 x 64 FP64 partials, 6.1 MB; the per-render kernel's hold 8 to 32 pixels
+        ctx = api.Context(0, hbm_budget_bytes=used - (3 << 20))
+        try:
+            small = run(ctx, job)
+            assert ctx.memory_used() <= used - (3 << 20)
+        finally:
+            ctx.close()
+        # differences of losses that are rounded to FP64 sums in another order
+        assert np.allclose(small, grad, rtol=1e-6, atol=1e-6 * np.abs(grad).max())
