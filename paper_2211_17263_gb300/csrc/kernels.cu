@@ -2285,7 +2285,8 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
 // Tracing a path once instead of once per render leaves per render only its estimates (light
 // sample, occlusion by the few primitives the cull leaves, geometry term) and products of
 // albedos. Before, the GI box's renders retraced every path side by side (k_trace_group) and Eq. 9
-// traced each render alone (k_trace): GI box 512 x 512, 32 renders at 32 spp 40.9 -> 16.2 ms, its
+// traced each render alone (k_trace; Eq. 10 with albedos only shared paths, but nearly every path meets a
+// bound wall): GI box 512 x 512, 32 renders at 32 spp 40.9 -> 16.2 ms, its
 // walls by Eq. 9 87.6 -> 7.5 ms, by Eq. 10 at 256 x 256 11.3 -> 1.26 ms, caustic 512 x 512, 64 renders at
 // 64 spp 7.8 -> 7.3 ms. Leaving fixed emitters out of the variant for jobs whose emitters all move
 // (80 -> 74 KB of code: instruction fetch is among the largest stalls) took the GI box to 15.1 ms and
@@ -2300,7 +2301,7 @@ constexpr int kReplayWarps = kGroupBlock / 32;
 //   u64 acc[halves][3][32]            radiance of the current pixel, 2^-32 fixed point
 //   u64 dacc[halves][nd][32]          Eq. 9: its tangent sums
 //   double gsum[halves][nd][32]       Eq. 9: the block's gradient partials
-//   u64 common[replay_common][3]             radiance common to all renders, per pixel of the block
+//   u64 common[replay_common][3]      radiance common to all renders, per pixel of the block
 //   float4 ent[pool], u16 nxt[pool], u16 first[32], unsigned ctr
 struct ReplayHead {
     GroupScene scene;  // the invariant part (render 0's records of the other primitives)
