@@ -142,7 +142,7 @@ struct prdpt_ctx {
     // per-render ones, then the replay jobs: jobs and work items of each kind (one render
     // launch per kind)
     int batch_jobs[4] = {0, 0, 0, 0}, batch_items[4] = {0, 0, 0, 0};
-    TraceLaunch batch_replay{};  // variant, table and pool of the packed replay launch
+    std::vector<TraceLaunch> batch_replay;  // the packed step's replay launches, by class of job
     // optional CUDA-event timing of the render kernel, recorded on its launch stream
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_used, ev_free;
@@ -549,6 +549,14 @@ void replay_cover(TraceLaunch& L, const TraceJob& J) {
     L.pool = std::max(L.pool, replay_path_granules(J.depth, J.n_var > 0));
     if (J.diff) L.diff_nd = J.nd;
     L.pool = replay_pool(L);
+}
+
+// Jobs that share a packed replay launch: one class per kernel variant and number of renders per
+// lane. One launch for all of them would run the most general variant with the largest sums, and so
+// the smallest pool, on every job (12 jobs of the serving mix, GI boxes of 16 to 128 renders among
+// them: 137 job-steps/s in one launch, 145.5 by class, p99 step latency 46 and 36 ms).
+int replay_class(const TraceJob& J) {
+    return (J.chunks > 1 ? 16 : 0) | (J.R > 32 ? 8 : 0) | (J.var_mats ? 4 : 0) | (J.n_var > 0 ? (J.black ? 1 : 2) : 0);
 }
 
 // Work items of a gradient job's render launch: pixel blocks (path sharing, replay),
@@ -1803,10 +1811,13 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
                 Job* j = get_job(c, ids[i]);
                 if (kind(j) == pass) order.push_back(j);
             }
+        std::stable_sort(order.begin(), order.end(), [&](const Job* a, const Job* b) {  // replay jobs, by class
+            return kind(a) == 3 && kind(b) == 3 && replay_class(a->trace) < replay_class(b->trace);
+        });
         std::vector<InstJob> inst(n);
         std::vector<TraceJob> trace(n);
         int blocks = 0, jobs_of[4] = {0, 0, 0, 0}, items_of[4] = {0, 0, 0, 0};
-        TraceLaunch cover{};  // the replay launch's variant, table and pool
+        std::vector<TraceLaunch> replays;  // per class: its jobs, items, variant, table and pool
         for (int i = 0; i < n; ++i) {
             Job* j = order[i];
             const int kd = kind(j);
@@ -1818,7 +1829,16 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
             trace[i].fin_begin = blocks - j->R;  // same prefix as the sampler CTAs
             const long long it = job_items(j->trace);
             if (prdpt_status st = check_items((long long)items_of[kd] + it)) return st;
-            if (kd == 3) replay_cover(cover, j->trace);
+            if (kd == 3) {
+                if (jobs_of[kd] == 0 || replay_class(j->trace) != replay_class(order[i - 1]->trace)) {
+                    replays.emplace_back();
+                    items_of[kd] = 0;
+                }
+                TraceLaunch& T = replays.back();
+                replay_cover(T, j->trace);
+                T.njobs++;
+                T.total_items += int(it);
+            }
             items_of[kd] += int(it);
             jobs_of[kd]++;
         }
@@ -1868,7 +1888,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
         PRDPT_CUDA(cudaEventRecord(c->h_desc_ev[k], st_));
         c->batch_ids = ids;
         c->batch_blocks = blocks;
-        c->batch_replay = cover;
+        c->batch_replay = std::move(replays);
         for (int q = 0; q < 4; ++q) {
             c->batch_jobs[q] = jobs_of[q];
             c->batch_items[q] = items_of[q];
@@ -1883,31 +1903,29 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
     IL.queue_reset3 = c->s_ctl + 8;
     IL.queue_reset4 = c->s_ctl + 9;
     PRDPT_CUDA(launch_instantiate(IL, st_));
-    TraceLaunch TL[4] = {};
-    int nL = 0, first = 0;
-    unsigned* queues[4] = {c->s_ctl + 2, c->s_ctl + 3, c->s_ctl + 8, c->s_ctl + 9};
-    for (int kd = 0; kd < 4; ++kd) {  // path-sharing, render-group, per-render, replay jobs
+    std::vector<TraceLaunch> TL;
+    int first = 0;
+    unsigned* queues[3] = {c->s_ctl + 2, c->s_ctl + 3, c->s_ctl + 8};
+    for (int kd = 0; kd < 3; ++kd) {  // path-sharing, render-group, per-render jobs
         if (c->batch_jobs[kd] > 0) {
-            TraceLaunch& T = TL[nL++];
+            TraceLaunch T{};
             T.jobs = c->d_trace + first;
             T.njobs = c->batch_jobs[kd];
             T.total_items = c->batch_items[kd];
             T.share = kd == 0 ? 1 : 0;
-            T.group = kd == 1 ? 1 : (kd == 3 ? 2 : 0);
-            if (kd == 3) {
-                T.replay_mat = c->batch_replay.replay_mat;
-                T.replay_move = c->batch_replay.replay_move;
-                T.tab_rows = c->batch_replay.tab_rows;
-                T.pool = c->batch_replay.pool;
-                T.halves = c->batch_replay.halves;
-                T.replay_chunked = c->batch_replay.replay_chunked;
-                if (T.replay_chunked) T.replay_mat = 1;  // (the chunked variants replay throughputs)
-                T.pixels = c->batch_replay.pixels;
-            }
+            T.group = kd == 1 ? 1 : 0;
             T.queue = queues[kd];
+            TL.push_back(T);
         }
         first += c->batch_jobs[kd];
     }
+    for (TraceLaunch T : c->batch_replay) {  // replay jobs (each has its own queue)
+        T.jobs = c->d_trace + first;
+        T.group = 2;
+        first += T.njobs;
+        TL.push_back(T);
+    }
+    const int nL = int(TL.size());
     for (int i = 0; i < nL; ++i) {
         TL[i].counters = c->counting ? c->counters : nullptr;
         TL[i].status = c->status;
@@ -1917,7 +1935,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
     FL.njobs = n;
     FL.fin_total = c->batch_blocks;
     FL.status = c->status;
-    PRDPT_CUDA(timed_trace(c, TL, nL, &FL, false, st_, 0));
+    PRDPT_CUDA(timed_trace(c, TL.data(), nL, &FL, false, st_, 0));
     for (int i = 0; i < n; ++i) {  // every job's buffers are in use until here
         Job* j = get_job(c, ids[i]);
         PRDPT_CUDA(mark_use(j->last, &j->used, &j->captured, st_));

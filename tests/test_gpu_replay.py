@@ -202,3 +202,28 @@ def test_whole_blocks_where_the_budget_refuses_small_ones(gpu_lib):
             ctx.close()
         # differences of losses that are rounded to FP64 sums in another order
         assert np.allclose(small, grad, rtol=1e-6, atol=1e-6 * np.abs(grad).max())
+
+
+def test_packed_step_of_every_class(ctx):
+    """Replay jobs of all variants (renders per lane, chunks, bound albedos, moving emitters, parting
+    renders), in mixed order, in one packed step: each equals the job stepped alone, bit for bit."""
+    from paper_2211_17263_gb300 import api
+    shapes = [(_gi, 3, 33, 18), (_walls, 20, 24, 11), (_light, 24, 16, 9), (_gi, 40, 13, 8), (_box_light_wall, 5, 21, 10),
+              (_gi, 2, 40, 6), (_two_lights, 17, 12, 12), (_walls, 4, 9, 9), (_light, 8, 31, 7)]
+    wls = [make(width=w, height=h, spp=6, pairs=p) for make, p, w, h in shapes]
+    scenes = [ctx.upload_scene(wl.scene, wl.bindings) for wl in wls]
+    rng = np.random.default_rng(5)
+    targets = [rng.uniform(size=(wl.height, wl.width, 4)).astype(np.float32) for wl in wls]
+    make = lambda: [api.Job(s, wl, t, use_tuned=False, block_pixels=8) for s, wl, t in zip(scenes, wls, targets)]
+    alone, packed = make(), make()
+    for _ in range(2):
+        for j in alone:
+            j.step()
+        api.step_batch(ctx, packed)
+    for a, b in zip(alone, packed):
+        x, y = a.read(), b.read()
+        assert x["steps"] == y["steps"] == 2
+        for k in ("theta", "grad", "losses"):
+            assert np.array_equal(x[k], y[k])
+        a.release()
+        b.release()
