@@ -436,19 +436,25 @@ int choose_block(prdpt_ctx* c, int requested, int R, int W, int H, bool render) 
     return 8;
 }
 
-// Pixels per block in replay mode when the caller does not say: the most that give every resident
-// warp eight items, while each still fills two batches of paths (32 each). A small image would
-// otherwise end in a half-empty round (GI box walls 256 x 256 at 32 spp, 24 warps per SM: blocks of 8
-// pixels 1.55 ms, of 4 pixels 1.25 ms).
-int choose_replay_block(prdpt_ctx* c, int requested, int W, int H, int spp) {
+// Is a replay work item of px pixels worth splitting in two? Up to eight items per resident warp while
+// each half still fills two batches of paths (32 each); a small image would otherwise end in a
+// half-empty round (GI box walls 256 x 256 at 32 spp, 24 warps per SM: blocks of 8 pixels 1.55 ms, of 4
+// pixels 1.25 ms). While there are fewer items than warps, down to 8 paths: idle warps cost more
+// than half-empty batches (GI box 86 x 86 at 3 spp, 78 renders: 484 items of 32 pixels 3.06 ms, split to
+// 4 pixels 0.23 ms; render groups 2.01 ms).
+bool replay_split(prdpt_ctx* c, long long items, int px, int spp) {
+    const long long warps = (long long)c->sms * kReplayWarpsPerSm, paths = (long long)(px / 2) * spp;
+    return px > 1 && ((items < 8 * warps && paths >= 64) || (items < warps && paths >= 8));
+}
+
+// Pixels per block in replay mode when the caller does not say.
+int choose_replay_block(prdpt_ctx* c, int requested, int W, int H, int spp, int chunks) {
     if (requested == 8 || requested == 16 || requested == 32) return requested;
-    const long long warps = (long long)c->sms * kReplayWarpsPerSm;
     int px = 32;
     for (; px > 1; px /= 2) {
         int bw, bh;
         block_shape(px, &bw, &bh);
-        const long long items = (long long)((W + bw - 1) / bw) * ((H + bh - 1) / bh);
-        if (items >= 8 * warps || px / 2 * spp < 64) break;
+        if (!replay_split(c, (long long)((W + bw - 1) / bw) * ((H + bh - 1) / bh) * chunks, px, spp)) break;
     }
     return px;
 }
@@ -457,9 +463,8 @@ int choose_replay_block(prdpt_ctx* c, int requested, int W, int H, int spp) {
 // for (caustic 237 x 141 at 20 spp, 24 renders, blocks of 32 pixels: 0.68 ms whole, 0.27 ms in 8
 // parts; their sums meet in memory, which costs small blocks 5 %, so the choice above comes first).
 int replay_parts(prdpt_ctx* c, int px, int tiles, int spp, int chunks) {
-    const long long warps = (long long)c->sms * kReplayWarpsPerSm;
     int parts = 1;
-    while (chunks == 1 && 2 * parts <= px && (long long)tiles * parts < 8 * warps && (long long)px / (2 * parts) * spp >= 64) parts *= 2;
+    while (chunks == 1 && replay_split(c, (long long)tiles * parts, px / parts, spp)) parts *= 2;
     return parts;
 }
 
@@ -1172,7 +1177,7 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
     fill_share(probe, s->host, o);  // path sharing or replay: items are blocks, not (render, block)
     fill_group(probe, s->host, o);
     const bool per_block = probe.share || probe.emit;
-    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp)
+    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp, probe.chunks)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
@@ -1482,7 +1487,7 @@ static prdpt_status job_create_blocks(prdpt_ctx* c, int32_t scene_id, const prdp
     j->R = 2 * o->pairs;
     const int D = j->D, R = j->R, W = o->width, H = o->height;
     const bool per_block = probe.share || probe.emit;
-    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp)
+    const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp, probe.chunks)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;

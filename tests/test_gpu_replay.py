@@ -227,3 +227,18 @@ def test_packed_step_of_every_class(ctx):
             assert np.array_equal(x[k], y[k])
         a.release()
         b.release()
+
+
+@pytest.mark.parametrize("make", [_gi, _walls, _two_lights])
+@pytest.mark.parametrize("pairs,spp,width,height", [(39, 3, 86, 86), (20, 1, 33, 7), (3, 8, 29, 31), (35, 2, 5, 3)])
+def test_few_samples_on_small_images(ctx, make, pairs, spp, width, height):
+    """Fewer work items than warps: blocks go down to 8 paths, less than a batch. The per-render
+    kernel's blocks are larger, so FP64 partial sums are grouped differently: an FP32 loss may differ
+    in its last bit."""
+    wl = make(width=width, height=height, spp=spp, pairs=pairs)
+    scene = ctx.upload_scene(wl.scene, wl.bindings)
+    target = _t(np.random.default_rng(2).uniform(size=(height, width, 4)))
+    L = []
+    for kw in ({}, dict(no_path_sharing=1, render_groups=-1)):
+        L.append(scene.smoothed_grad(_t(wl.theta0), _t(wl.sigma), target, scene.grad_opts(wl, step=1, **kw))[1].cpu().numpy())
+    assert np.allclose(L[0], L[1], rtol=2.0**-22, atol=0.0)
