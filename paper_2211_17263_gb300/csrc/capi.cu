@@ -919,18 +919,28 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     const int rstride = stride + (J.nd + 3) / 4;
     // (Beyond 64 renders only with bound materials: a path is then traced once per 64 renders, which
     // still beats render groups -- GI box 256 x 256 at 16 spp, 80 renders: 13.6 -> 5.0 ms.)
-    if (!o->no_path_sharing && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
+    // Where the renders part from the path (a perturbed primitive that is not black is seen) they trace
+    // the rest one lane each, so groups of 4 or more stay faster beside bound albedos or fixed emitters
+    // (GI box with a grey box moving, 400 x 400: 8 renders at 2 spp 1.29 ms in groups, 2.54 ms replayed; 6
+    // renders, groups of 2, 2.28 and 1.60 ms). With 2 renders the chains cost more than a second trace
+    // from 16 spp on (GI box 1.81 and 1.99 ms), and for Eq. 9 with fewer samples or 4 renders too
+    // (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16 spp 1.94 and 1.74; 4 renders at
+    // 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
+    bool parts = false, fixed_light = false;
+    for (int i = 0; i < B.n_prims; ++i) {
+        const int m = B.prim_mat[i];
+        const float* mp = B.mat_param[m];
+        const bool moves = (prims >> B.prim_slot[i]) & 1u;
+        fixed_light |= !moves && (mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f);
+        parts |= moves && (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f);
+    }
+    const bool grouped = !pathwise && ((parts && (nm > 0 || fixed_light) && R % 4 == 0 && 4 * stride <= kGroupTabRows) ||
+                                       (n > 0 && R == 2 && o->spp >= 16));
+    const bool few = pathwise && R < 6 && R * R * o->spp < 64;
+    if (!o->no_path_sharing && !grouped && !few && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
         J.emit = 1;
         J.chunks = (R + 63) / 64;
-        J.black = 1;
-        for (int i = 0; i < B.n_prims; ++i) {
-            const int m = B.prim_mat[i];
-            const float* mp = B.mat_param[m];
-            if ((mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f) && !((prims >> B.prim_slot[i]) & 1u)) J.black = 0;
-            if (((prims >> B.prim_slot[i]) & 1u) &&
-                (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f))
-                J.black = 0;
-        }
+        J.black = !parts && !fixed_light;
         J.gstride = rstride;
         J.n_var = n;
         J.var_prims = prims;
