@@ -74,9 +74,10 @@ __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
     return f3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
 // The approximate reciprocal, quotient and reciprocal root of the path tracer, without the code
-// that the plain intrinsics carry for subnormal operands: their operands here are never subnormal
-// (directions, cosines, roulette probabilities, distances; a subnormal under the root of the
-// sphere test gives a miss), and for the others the results are the same.
+// that the plain intrinsics carry for subnormal operands: their operands in the tracer are never
+// subnormal (directions, cosines, roulette probabilities, distances; a subnormal under the root of
+// the sphere test gives a miss), and for the others the results are the same. A quad's u x v can
+// have a subnormal square: k_instantiate takes the plain root for its normal.
 __device__ __forceinline__ float rcp_fast(float a) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
@@ -407,7 +408,8 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
             P[1] = make_float4(g[3] * g[3], 1.0f / g[3], __int_as_float(mat), __int_as_float(i));
         } else if (type == kQuad) {
             const float3 u = f3(g[3], g[4], g[5]), v = f3(g[6], g[7], g[8]);
-            const float3 n = normalized(cross3(u, v));
+            const float3 uv = cross3(u, v);
+            const float3 n = uv * rsqrtf(dot3(uv, uv));  // subnormal for |u x v| < 1.1e-19: not rsqrt_fast
             float uw = 1.0f / dot3(u, u), vw = 1.0f / dot3(v, v);
             bool plain = true;  // textured quads: the first keeps 1/(u.u), 1/(v.v) in the scene's header
             for (int k = 0; k < i && mat == B.tex_mat; ++k)
