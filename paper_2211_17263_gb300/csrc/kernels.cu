@@ -204,8 +204,9 @@ __device__ __forceinline__ float half_extent(float e, float w) {
 
 // An axis-aligned quad (unit normal along one axis, edges along the other two): returns 1 + the
 // normal's axis and replaces uw, vw by the half extents along the lower and the higher edge axis, for
-// quad_any_t's short test; 0 for any other quad.
-__device__ __forceinline__ int axis_quad(float3 n, float3 u, float3 v, float& uw, float& vw) {
+// quad_any_t's short test; 0 for any other quad, and for one whose plane the camera's eye is `near`.
+template <class Near>
+__device__ __forceinline__ int axis_quad(float3 n, float3 u, float3 v, float& uw, float& vw, const Near& near) {
     const float nn[3] = {n.x, n.y, n.z}, uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z};
     int a = -1, b = -1, c = -1;
     float eu = 0.0f, ev = 0.0f;
@@ -218,7 +219,7 @@ __device__ __forceinline__ int axis_quad(float3 n, float3 u, float3 v, float& uw
     }
     if (a < 0 || b < 0 || c < 0) return 0;
     const float hu = half_extent(eu, uw), hv = half_extent(ev, vw);
-    if (!(hu > 1e-30f && hu < 1e30f && hv > 1e-30f && hv < 1e30f)) return 0;
+    if (!(hu > 1e-30f && hu < 1e30f && hv > 1e-30f && hv < 1e30f) || near(a)) return 0;
     uw = b < c ? hu : hv;
     vw = b < c ? hv : hu;
     return 1 + a;
@@ -418,7 +419,16 @@ __global__ void __launch_bounds__(kInstBlock) k_instantiate(const InstLaunch L) 
                 s_tex[0] = uw;
                 s_tex[1] = vw;
             }
-            const int axis = plain ? axis_quad(n, u, v, uw, vw) : 0;
+            // The eye within 1e-6 of the quad's plane (see quad_any_t). Renders share the rows of a moving
+            // quad that no binding changes, so one that moves along its normal is judged in forward
+            // renders only.
+            auto near = [&](int a) {
+                if (!(fabsf(g[a] - B.eye[a]) < 1e-6f)) return false;
+                for (int d = 0; d < B.D && !J.render_mode && B.tex_mat < 0; ++d)
+                    if (B.bind_kind[d] == kBindPos && B.bind_index[d] == i && B.bind_comp[d] == a) return false;
+                return true;
+            };
+            const int axis = plain ? axis_quad(n, u, v, uw, vw, near) : 0;
             P[0] = make_float4(c.x, c.y, c.z, __int_as_float(mat | (axis << 8)));
             P[1] = make_float4(n.x, n.y, n.z, __int_as_float(i));
             P[2] = make_float4(u.x, u.y, u.z, uw);
@@ -558,6 +568,12 @@ __device__ __forceinline__ float quad_t(const Rec& P, float3 o, float3 d) {
 // instructions and one reciprocal per axis and ray instead of 38 and one per quad: four 512 x 512
 // renders of the GI box at 32 spp 6.35 -> 6.06 ms, occlusion with independent samples 478 -> 468 us
 // (together with div_fast and its kin).
+// quad_t's bound on the cosine (1e-12) is left out: with a smaller one that is not zero, t > kEps
+// needs a ray that starts within 1e-12 t of the plane but not in it. Points on surfaces lie kEps off
+// parallel planes and anywhere beside the others; the camera's eye can lie so near, and then the
+// quad takes the general test (k_instantiate). Testing the bound here costs 1 to 5 % (per quad: GI box
+// 512 x 512, 32 renders 14.58 -> 15.03 ms, Eq. 9 on 256 x 256 walls 2.02 -> 2.10; per ray, with the
+// reciprocal cleared: 14.91 and 2.10).
 template <class Rec>
 __device__ __forceinline__ float quad_any_t(const Rec& P, float3 o, float3 d, float3 inv) {
     const float4 a = P[0];
