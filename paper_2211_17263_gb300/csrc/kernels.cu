@@ -2745,7 +2745,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
         const int t = int(item) / J.parts, q0 = (int(item) - t * J.parts) * (qend << qshift);
         const int R = kChunked ? min(J.R - r0, 64) : J.R, nh = R > 32 ? 2 : 1, spp = J.spp;
         // phase B lanes: render gi of sample group ks; with R < 32, nsg = floor(32 / R) samples
-        // side by side (lanes beyond nsg R idle)
+        // side by side (lanes beyond nsg R repeat the last group's; they are not counted)
         const int G = R < 32 ? R : 32, nsg = 32 / G, gi = lane % G, ks = lane / G;
         const int areas = !kND && J.gstride > J.var_rows + __popc(J.var_mats) ? 1 : 0;
         const int x0 = (t % J.tiles_x) * J.bw, y0 = (t / J.tiles_x) * J.bh;
@@ -2806,12 +2806,14 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
                 start_path<true>(E.scene, J.W, J.H, px, py, sp, slot, p);
             }
             bool live = have;
+            const Counters before = cnt;
 #pragma unroll 1
             while (__any_sync(kFull, live)) {
                 if (live) live = replay_vertex<kCount, kMat, kMove>(E.scene, J.depth, J.rr_start, p, el, cnt) == kLive;
             }
             const unsigned fm = __ballot_sync(kFull, el.full), hm = __ballot_sync(kFull, have);
             const int nb = fm ? __ffs(fm) - 1 : __popc(hm);  // the batch: tasks of lanes 0 .. nb - 1
+            if (kCount && lane >= nb) cnt = before;  // traced again in the next batch
             if (nb == 0) {
                 if (alone) {  // cannot happen: the host sizes the pool for any one path
                     if (lane == 0) atomicOr(L.status, kStatusBadItem);
@@ -2860,7 +2862,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
                             if (i <= ks) jj = __ffs(todo) - 1;
                             todo &= todo - 1u;
                         }
-                        if (jj < 0 || r >= R) continue;
+                        if (jj < 0 || r >= R || (kCount && ks >= nsg)) continue;
                         Tangents<kND> tn;
                         if (kND > 0) tan_reset(tn);
                         const float3 v = replay_sample<kCount, kMat, kMove, kND>(

@@ -1,0 +1,71 @@
+"""Replay mode (every path traced once, replayed by each render) at the edges of what it takes."""
+import numpy as np
+import pytest
+
+import workloads
+from test_gpu_replay import _light, _t, _walls
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def ctx(gpu_lib):
+    from paper_2211_17263_gb300 import api
+    c = api.Context(0)
+    yield c
+    c.close()
+
+
+def _grad(ctx, wl, step=3, **kw):
+    scene = ctx.upload_scene(wl.scene, wl.bindings)
+    target = _t(np.random.default_rng(1).uniform(size=(wl.height, wl.width, 4)))
+    g, L = scene.smoothed_grad(_t(wl.theta0), _t(wl.sigma), target, scene.grad_opts(wl, step=step, **kw))
+    torch.cuda.synchronize()
+    return g.cpu().numpy(), L.cpu().numpy()
+
+
+def _count(ctx, wl, **kw):
+    ctx.counters_enable(True)
+    _grad(ctx, wl, **kw)
+    n = np.array(ctx.counters_read())
+    ctx.counters_enable(False)
+    return n
+
+
+@pytest.mark.parametrize("pairs", [3, 5, 6, 9, 12])
+def test_shadow_rays_are_counted_once_per_render(ctx, pairs):
+    """The renders of a job, and the same renders one pair at a time, trace the same shadow rays
+    (6, 10, 12, 18 and 24 renders leave lanes of a warp without a render)."""
+    wl = _light(width=19, height=11, spp=5, pairs=pairs)
+    whole = _count(ctx, wl)
+    one = [_count(ctx, workloads.scaled(wl, pairs=1), pair_begin=p) for p in range(pairs)]
+    assert whole[5] == sum(n[5] for n in one) > 0
+
+
+def _closed_walls(**kw):
+    """The box with its camera inside and a front wall: no path leaves it."""
+    wl = _walls(**kw)
+    sc = wl.scene
+    lo, hi = sc.prim_geom[:5, :3].min(0), sc.prim_geom[:5, :3].max(0)
+    side = int(np.argmax(np.abs(sc.camera[3:6] - sc.camera[:3])))  # the open side faces the camera
+    outside = sc.camera[side] < (lo[side] + hi[side]) / 2
+    front = (lo + hi) / 2
+    front[side] = lo[side] - 0.5 if outside else hi[side] + 0.5
+    u, v = 20 * np.eye(3)[(side + 1) % 3], 20 * np.eye(3)[(side + 2) % 3]
+    geom = np.concatenate([sc.prim_geom, [np.concatenate([front, u, v])]]).astype(np.float32)
+    camera = sc.camera.copy()
+    camera[side] = front[side] + (0.3 if outside else -0.3)
+    wl.scene = workloads.Scene(np.append(sc.prim_type, 1).astype(np.int32), np.append(sc.prim_mat, 0).astype(np.int32),
+                               geom, sc.mat_type, sc.mat_param, camera, sc.background)
+    return wl
+
+
+def test_work_is_counted_once_where_the_pool_runs_out(ctx):
+    """Paths that did not fit their batch's pool are traced again in the next one; their rays and
+    vertices count once. Without roulette every render's paths are the shared ones."""
+    wl = _closed_walls(width=16, height=12, spp=32, pairs=4, depth=64, rr_start=-1)
+    shared, alone = _count(ctx, wl, block_pixels=8), _count(ctx, wl, block_pixels=8, no_path_sharing=1, render_groups=-1)
+    for k in (3, 4, 5, 6):
+        assert shared[k] * 8 == alone[k] > 0, k
+    assert shared[6] > 16 * 12 * 32 * 20  # long paths: 32 of them exceed the pool's 512 granules
