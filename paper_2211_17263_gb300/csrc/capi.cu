@@ -493,12 +493,17 @@ void tiles_for(int pixels, int W, int H, int* bw, int* bh, int* tiles_x, int* ti
     *tiles = *tiles_x * ((H + *bh - 1) / *bh);
 }
 
-// Zero-initialised device array that grows on demand (kernels leave it zeroed).
+// Zero-initialised device array that grows on demand (kernels leave it zeroed). Cleared before the
+// call goes on: a clear on the default stream is not ordered before the caller's when that does not
+// wait for it.
 template <typename T>
 prdpt_status grow_zeroed(prdpt_ctx* c, T** p, size_t* cap, size_t n) {
     if (*cap >= n) return PRDPT_OK;
     if (prdpt_status st = grow(c, p, cap, n)) return st;
-    if (cudaMemset(*p, 0, n * sizeof(T)) != cudaSuccess) return fail(PRDPT_E_CUDA, "cudaMemset failed");
+    if (cudaMemsetAsync(*p, 0, n * sizeof(T), c->io) != cudaSuccess || cudaStreamSynchronize(c->io) != cudaSuccess) {
+        *cap = 0;
+        return fail(PRDPT_E_CUDA, "clearing scratch memory failed");
+    }
     return PRDPT_OK;
 }
 

@@ -69,3 +69,22 @@ def test_work_is_counted_once_where_the_pool_runs_out(ctx):
     for k in (3, 4, 5, 6):
         assert shared[k] * 8 == alone[k] > 0, k
     assert shared[6] > 16 * 12 * 32 * 20  # long paths: 32 of them exceed the pool's 512 granules
+
+
+def test_parts_on_a_side_stream(gpu_lib):
+    """The first call of a context on a stream that does not wait for the legacy default stream:
+    the counters of finished parts are zero before it."""
+    from paper_2211_17263_gb300 import api
+    wl = _walls(width=64, height=48, spp=16, pairs=4)
+    want = None
+    for _ in range(6):
+        ctx = api.Context(0)
+        try:
+            side = torch.cuda.Stream()
+            with torch.cuda.stream(side):
+                got = [_grad(ctx, wl, block_pixels=32) for _ in range(2)]
+        finally:
+            ctx.close()
+        want = want or got[0]
+        for g, L in got:
+            assert np.array_equal(g, want[0]) and np.array_equal(L, want[1])
