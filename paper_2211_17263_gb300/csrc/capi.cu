@@ -132,6 +132,9 @@ struct prdpt_ctx {
     size_t s_pdone_n = 0;
     double* s_rgrads = nullptr;   // pathwise estimator: [R][kMaxDiff] per-render gradients
     size_t s_rgrads_n = 0;
+    // Scratch whose size depends on the blocks (s_partials, s_gpart, s_psums, s_pdone) is given back
+    // when memory runs out, but not to the call that is growing it, and not once a graph holds it.
+    bool scratch_held = false, scratch_captured = false;
     // packed launches
     std::vector<int> batch_ids;
     InstJob* d_inst = nullptr;
@@ -184,14 +187,19 @@ struct prdpt_ctx {
 
 namespace {
 
+bool release_block_scratch(prdpt_ctx* c);
+
 prdpt_status dev_alloc(prdpt_ctx* c, void** p, size_t bytes) {
     if (bytes == 0) bytes = 16;
-    if (c->budget && c->used + bytes > c->budget)
+    if (c->budget && c->used + bytes > c->budget) {
+        if (release_block_scratch(c)) return dev_alloc(c, p, bytes);
         return fail(PRDPT_E_OUT_OF_BUDGET, "allocation of " + std::to_string(bytes) + " bytes exceeds the HBM budget (" +
                                                std::to_string(c->used) + " of " + std::to_string(c->budget) + " used)");
+    }
     cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();  // an out-of-memory result is not sticky: keep it from later launch checks
+        if (release_block_scratch(c)) return dev_alloc(c, p, bytes);
         return fail(PRDPT_E_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     }
     c->allocs[*p] = bytes;
@@ -206,7 +214,25 @@ void dev_free(prdpt_ctx* c, void* p) {
     if (it == c->allocs.end()) return;
     c->used -= it->second;
     c->allocs.erase(it);
-    cudaFree(p);
+    cudaFree(p);  // waits for the kernels that use it
+}
+
+template <typename T>
+bool drop(prdpt_ctx* c, T** p, size_t* cap) {
+    const bool held = *p != nullptr;
+    dev_free(c, *p);
+    *p = nullptr;
+    *cap = 0;
+    return held;
+}
+
+// Replay's small blocks and parts take more scratch than whole blocks: where that keeps another
+// allocation from the budget, it is given back.
+bool release_block_scratch(prdpt_ctx* c) {
+    if (c->scratch_held || c->scratch_captured) return false;
+    const bool a = drop(c, &c->s_partials, &c->s_partials_n), b = drop(c, &c->s_gpart, &c->s_gpart_n);
+    const bool d = drop(c, &c->s_psums, &c->s_psums_n), e = drop(c, &c->s_pdone, &c->s_pdone_n);
+    return a || b || d || e;
 }
 
 constexpr size_t kZeroBytes = size_t(4) << 20;
@@ -1198,6 +1224,21 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
     if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) return st;
+    const size_t n_w = std::max((size_t)R * D, (size_t)kMaxD), n_gpart = probe.diff ? (size_t)R * tiles * D : 0;
+    if (*whole && c->budget) {  // refused before anything grows: whole blocks may fit
+        auto more = [](size_t cap, size_t n, size_t bytes) { return cap < n ? (n - cap) * bytes : 0; };
+        if (c->used + more(c->s_scenes_n, R, sizeof(InstScene)) + more(c->s_w_n, n_w, sizeof(float)) +
+                more(c->s_partials_n, (size_t)R * tiles, sizeof(double)) + more(c->s_losses_n, R, sizeof(double)) +
+                more(c->s_gpart_n, n_gpart, sizeof(double)) +
+                (probe.diff ? more(c->s_rgrads_n, (size_t)R * kMaxDiff, sizeof(double)) : 0) >
+            c->budget)
+            return fail(PRDPT_E_OUT_OF_BUDGET, "the scratch of small blocks exceeds the HBM budget");
+    }
+    struct Hold {  // the block scratch is this call's until it has been launched
+        prdpt_ctx* c;
+        explicit Hold(prdpt_ctx* ctx) : c(ctx) { c->scratch_held = true; }
+        ~Hold() { c->scratch_held = false; }
+    } hold(c);
     if (probe.share) {
         const size_t pix = (size_t)o->width * o->height;
         if (prdpt_status st = grow(c, &c->s_share, &c->s_share_n, (size_t)tiles * 96)) return st;
@@ -1209,20 +1250,21 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
         if (prdpt_status st = grow(c, &c->s_flags, &c->s_flags_n, (size_t)R * ((pix + 31) / 32))) return st;
     }
     if (prdpt_status st = grow(c, &c->s_scenes, &c->s_scenes_n, (size_t)R)) return st;
-    if (prdpt_status st = grow(c, &c->s_w, &c->s_w_n, (size_t)R * D > (size_t)kMaxD ? (size_t)R * D : (size_t)kMaxD))
-        return st;
+    if (prdpt_status st = grow(c, &c->s_w, &c->s_w_n, n_w)) return st;
     if (prdpt_status st = grow(c, &c->s_partials, &c->s_partials_n, (size_t)R * tiles)) return st;
     if (prdpt_status st = grow(c, &c->s_losses, &c->s_losses_n, (size_t)R)) return st;
-    if (probe.emit) {
+    if (probe.diff) {
+        if (prdpt_status st = grow(c, &c->s_gpart, &c->s_gpart_n, n_gpart)) return st;
+        if (prdpt_status st = grow(c, &c->s_rgrads, &c->s_rgrads_n, (size_t)R * kMaxDiff)) return st;
+    }
+    if (probe.emit) {  // last: they may only take what the buffers above leave
         probe.parts = replay_parts(c, px, tiles, o->spp, probe.chunks);
         if (probe.parts > 1 &&  // (without room for the parts' sums the blocks stay whole)
             (grow(c, &c->s_psums, &c->s_psums_n, replay_part_sums(probe, tiles)) != PRDPT_OK ||
-             grow_zeroed(c, &c->s_pdone, &c->s_pdone_n, (size_t)tiles) != PRDPT_OK))
+             grow_zeroed(c, &c->s_pdone, &c->s_pdone_n, (size_t)tiles) != PRDPT_OK)) {
             probe.parts = 1;
-    }
-    if (probe.diff) {
-        if (prdpt_status st = grow(c, &c->s_gpart, &c->s_gpart_n, (size_t)R * tiles * D)) return st;
-        if (prdpt_status st = grow(c, &c->s_rgrads, &c->s_rgrads_n, (size_t)R * kMaxDiff)) return st;
+            g_err = "no error";
+        }
     }
     const bool tex = s->host.tex_mat >= 0;
     cudaStream_t st_ = static_cast<cudaStream_t>(stream);
@@ -1340,19 +1382,28 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
         PRDPT_CUDA(launch_hd_grad(G, st_));
     }
     PRDPT_CUDA(mark_use(s->use, &s->used, &s->captured, st_));  // the scene block is in use until here
+    c->scratch_captured |= s->captured;
     return PRDPT_OK;
 }
 
 prdpt_status smoothed_grad_locked(prdpt_ctx* c, int32_t scene_id, const float* theta_dev, const float* sigma_dev,
                                   const prdpt_grad_opts* o, const float* target_dev, float* grad_dev,
                                   float* losses_dev, void* stream, const AdamDev* adam = nullptr) {
+    // (refused before anything was enqueued) whole blocks where small ones do not fit, and then with
+    // the block scratch of earlier calls given back
     int whole = 0;
-    const prdpt_status st = smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, o, target_dev, grad_dev, losses_dev,
-                                                 stream, adam, &whole);
-    if (st != PRDPT_E_OUT_OF_BUDGET || !whole) return st;  // (refused before anything was enqueued)
     prdpt_grad_opts w = *o;
-    w.block_pixels = whole;
-    return smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, &w, target_dev, grad_dev, losses_dev, stream, adam, &whole);
+    prdpt_status st = smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, &w, target_dev, grad_dev, losses_dev, stream,
+                                           adam, &whole);
+    if (st == PRDPT_E_OUT_OF_BUDGET && whole) {
+        w.block_pixels = whole;
+        st = smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, &w, target_dev, grad_dev, losses_dev, stream, adam,
+                                  &whole);
+    }
+    if (st == PRDPT_E_OUT_OF_BUDGET && !capturing(static_cast<cudaStream_t>(stream)) && release_block_scratch(c))
+        st = smoothed_grad_blocks(c, scene_id, theta_dev, sigma_dev, &w, target_dev, grad_dev, losses_dev, stream, adam,
+                                  &whole);
+    return st;
 }
 
 }  // namespace

@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import workloads
-from test_gpu_replay import _light, _t, _walls
+from test_gpu_replay import _gi, _light, _t, _walls
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -69,6 +69,68 @@ def test_work_is_counted_once_where_the_pool_runs_out(ctx):
     for k in (3, 4, 5, 6):
         assert shared[k] * 8 == alone[k] > 0, k
     assert shared[6] > 16 * 12 * 32 * 20  # long paths: 32 of them exceed the pool's 512 granules
+
+
+def _eq9(**kw):
+    return workloads.scaled(workloads.config_gi_albedo(), **kw)
+
+
+@pytest.mark.parametrize("block_pixels", [0, 32])
+@pytest.mark.parametrize("room", ["whole blocks", "small blocks' losses", "parts' sums"])
+def test_pathwise_gradient_within_the_budget_of_whole_blocks(gpu_lib, block_pixels, room):
+    """Eq. 9 under memory budgets that hold the partials of whole blocks, but not those of smaller
+    blocks or the sums of blocks in parts beside them: neither may take the gradient partials' room."""
+    from paper_2211_17263_gb300 import api
+    wl = _eq9(width=120, height=100, spp=64, pairs=32)
+    R, D, tiles, pixels = 64, 6, 15 * 25, 120 * 100  # blocks of 32 pixels, at most one part a pixel
+    losses, grads, sums = 8 * R * tiles, 8 * R * tiles * D, 8 * R * tiles * 32 * (1 + D)
+    extra = {"whole blocks": losses + grads, "small blocks' losses": 8 * R * pixels + grads // 2,
+             "parts' sums": losses + sums + grads // 2}[room]
+    ctx = api.Context(0)
+    try:
+        want, _ = _grad(ctx, wl, block_pixels=32)
+    finally:
+        ctx.close()
+    # everything else a call allocates: control words, scene, instances, weights, losses, gradients
+    ctx = api.Context(0, hbm_budget_bytes=1 << 30)
+    try:
+        _grad(ctx, _eq9(width=8, height=4, spp=1, pairs=32), block_pixels=32)
+        budget = ctx.memory_used() + extra + 4096
+    finally:
+        ctx.close()
+    ctx = api.Context(0, hbm_budget_bytes=budget)
+    try:
+        for _ in range(2):
+            got, _ = _grad(ctx, wl, block_pixels=block_pixels)
+            assert ctx.memory_used() <= budget
+            # blocks of another size group the FP64 partial sums differently
+            assert np.allclose(got, want, rtol=1e-6, atol=1e-6 * np.abs(want).max())
+    finally:
+        ctx.close()
+
+
+def test_optional_sums_make_room(gpu_lib):
+    """The part sums of one call do not keep a later call, job or render from the budget."""
+    from paper_2211_17263_gb300 import api
+    wl = _gi(width=120, height=100, spp=64, pairs=32)
+    ctx = api.Context(0, hbm_budget_bytes=64 << 20)
+    try:
+        want, _ = _grad(ctx, wl, block_pixels=32)
+        used = ctx.memory_used()
+    finally:
+        ctx.close()
+    big = _light(width=512, height=512, spp=1, pairs=2)
+    sums = 8 * 64 * (1 << 13)  # at least 8192 parts of 64 renders
+    ctx = api.Context(0, hbm_budget_bytes=used + 16 * 512 * 512 - sums)
+    try:
+        assert np.array_equal(_grad(ctx, wl, block_pixels=32)[0], want)
+        job = api.Job(ctx.upload_scene(big.scene, big.bindings), big, None, use_tuned=False)
+        job.step()
+        job.read()
+        job.release()
+        assert np.array_equal(_grad(ctx, wl, block_pixels=32)[0], want)
+    finally:
+        ctx.close()
 
 
 def test_parts_on_a_side_stream(gpu_lib):
