@@ -505,7 +505,8 @@ size_t replay_part_sums(const TraceJob& J, int tiles) {  // doubles of a replay 
     return J.parts > 1 ? size_t(tiles) * J.parts * J.R * (1 + J.nd) : 0;
 }
 
-// The render kernels number their work items (render x pixel block) with 32-bit integers.
+// The render kernels number their work items (render x pixel block) with 32-bit integers. (Replay
+// numbers blocks, but a call of more partials is refused all the same: 34 GB at 2^32.)
 prdpt_status check_items(long long items) {
     if (items > 0x7fffffffLL)
         return fail(PRDPT_E_INVALID_ARG, "more than 2^31 - 1 work items (renders x pixel blocks): use larger "
@@ -1217,13 +1218,12 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
     probe.R = R;
     fill_share(probe, s->host, o);  // path sharing or replay: items are blocks, not (render, block)
     fill_group(probe, s->host, o);
-    const bool per_block = probe.share || probe.emit;
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp, probe.chunks)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
-    if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) return st;
+    if (prdpt_status st = check_items(probe.share ? (long long)tiles : (long long)R * tiles)) return st;
     const size_t n_w = std::max((size_t)R * D, (size_t)kMaxD), n_gpart = probe.diff ? (size_t)R * tiles * D : 0;
     if (*whole && c->budget) {  // refused before anything grows: whole blocks may fit
         auto more = [](size_t cap, size_t n, size_t bytes) { return cap < n ? (n - cap) * bytes : 0; };
@@ -1552,13 +1552,12 @@ static prdpt_status job_create_blocks(prdpt_ctx* c, int32_t scene_id, const prdp
     j->D = s->D;
     j->R = 2 * o->pairs;
     const int D = j->D, R = j->R, W = o->width, H = o->height;
-    const bool per_block = probe.share || probe.emit;
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp, probe.chunks)
                               : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, W, H, &bw, &bh, &tiles_x, &tiles);
-    if (prdpt_status st = check_items(per_block ? (long long)tiles * probe.chunks : (long long)R * tiles)) {
+    if (prdpt_status st = check_items(probe.share ? (long long)tiles : (long long)R * tiles)) {
         delete j;
         return st;
     }

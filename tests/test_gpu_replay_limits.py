@@ -150,3 +150,24 @@ def test_parts_on_a_side_stream(gpu_lib):
         want = want or got[0]
         for g, L in got:
             assert np.array_equal(g, want[0]) and np.array_equal(L, want[1])
+
+
+def test_more_work_items_than_numbers_stay_refused(ctx):
+    """512 renders of 8192^2 pixels in 8-pixel blocks: (render, block) pairs beyond 32-bit numbers,
+    refused as a job and as a gradient, with or without sharing, before anything is allocated."""
+    from paper_2211_17263_gb300 import capi
+    wl = _walls()  # two bound materials: 512 renders' rows fit
+    scene = ctx.upload_scene(wl.scene, wl.bindings)
+    small, dev = np.zeros(16, np.float32), _t(np.zeros(16))
+    for kw in ({}, dict(no_path_sharing=1)):
+        opts = scene.grad_opts(wl, pairs=256, block_pixels=8, **kw)
+        opts.width = opts.height = 8192
+        desc = capi.prdpt_job_desc(grad=opts, theta0_host=small.ctypes.data, sigma0_host=small.ctypes.data,
+                                   target_host=small.ctypes.data, lr=0.01, beta1=0.9, beta2=0.999, eps=1e-8,
+                                   sigma_min=0.01, anneal=0, total_steps=1)
+        before = ctx.memory_used()
+        with pytest.raises(capi.PrdptError, match="work items"):
+            capi.prdpt_job_create(ctx.handle, scene.id, desc)
+        with pytest.raises(capi.PrdptError, match="work items"):
+            scene.smoothed_grad(dev[:6], dev[:6], dev, opts)
+        assert ctx.memory_used() == before
