@@ -575,19 +575,6 @@ int grid_for_replay(prdpt_ctx* c, const TraceLaunch& L, int ctas_per_sm) {
     return need < cap ? need : cap;
 }
 
-// Add a job to a replay launch: the variant, table and pool that cover every job of it.
-void replay_cover(TraceLaunch& L, const TraceJob& J) {
-    L.replay_mat |= J.var_mats ? 1 : 0;
-    L.replay_move = std::max(L.replay_move, J.n_var > 0 ? (J.black ? 1 : 2) : 0);
-    L.halves = std::max(L.halves, J.R > 32 ? 2 : 1);
-    L.tab_rows = std::max(L.tab_rows, J.R * J.gstride);
-    L.pixels = std::max(L.pixels, J.bw * J.bh / J.parts);
-    L.replay_chunked |= J.chunks > 1 ? 1 : 0;
-    L.pool = std::max(L.pool, replay_path_granules(J.depth, J.n_var > 0));
-    if (J.diff) L.diff_nd = J.nd;
-    L.pool = replay_pool(L);
-}
-
 // Jobs that share a packed replay launch: one class per kernel variant and number of renders per
 // lane. One launch for all of them would run the most general variant with the largest sums, and so
 // the smallest pool, on every job (12 jobs of the serving mix, GI boxes of 16 to 128 renders among

@@ -213,9 +213,10 @@ struct TraceLaunch {
     int group;                // 1: every job of the launch runs in render-group mode (k_trace_group),
                               // 2: in replay mode (k_trace_replay)
     // replay mode, covering every job of the launch: bound materials, perturbed primitives (1 only
-    // black ones, 2 any), float4 of the per-render table, entries of a warp's pool, 32-render
+    // black ones, 2 any), float4 of the per-render table, granules of a warp's pool, 32-render
     // halves of a warp's sums, pixels of a work item at most
     int replay_mat, replay_move, tab_rows, pool, halves, pixels;
+    int granules;             // entries of the pool that any one path may need
     int replay_chunked;       // a job has more than 64 renders (bound materials)
     int fin_total;            // packed launch: finalisation CTAs (sum of R over jobs)
     unsigned* queue;          // work-queue head, zeroed by the instantiation launch
@@ -301,7 +302,8 @@ int trace_group_blocks_per_sm();
 int trace_replay_blocks_per_sm(const TraceLaunch& L);
 constexpr int kReplayWarpsPerSm = 20;  // resident warps of the replay kernel
 size_t replay_smem(const TraceLaunch& L);
-int replay_pool(const TraceLaunch& L);  // pool of a launch that needs at least L.pool granules
+// Add a job to a replay launch: the variant, table and pool that cover every job of it.
+void replay_cover(TraceLaunch& L, const TraceJob& J);
 constexpr int kGroupBlock = 128;    // render-group CTAs: 4 warps (their per-warp tables fit 48 KB)
 constexpr int kGroupTabRows = 192;  // float4 of a warp's per-render record table (render-group mode)
 constexpr int kReplayTabRows = 1024;  // float4 of a CTA's per-render record table (replay mode), at most

@@ -2361,10 +2361,10 @@ constexpr int replay_min_blocks(bool move) { return move ? 5 : 6; }
 // (Eq. 9 on the box's walls with 44 renders, whose sums fill 6 CTAs' shared memory: 232 x 274 at 50 spp
 // 29.9 ms with 24 granules, 5.2 ms with what 3 CTAs leave; 64 renders, 256 x 256 at 16 spp, 10.9 and 1.9).
 constexpr int kReplayPoolMax = 512, kReplayPoolMove = 256, kReplayPoolFixed = 128;
-int replay_pool(const TraceLaunch& L) {
+static int replay_pool(const TraceLaunch& L) {
     const size_t head = sizeof(ReplayHead) + size_t(L.tab_rows) * 16;
     const size_t rest = replay_warp_bytes(0, L.halves, L.pixels, L.diff_nd);
-    const int need = (L.pool + 7) & ~7, want = L.replay_move ? kReplayPoolMove : kReplayPoolFixed;
+    const int need = (L.granules + 7) & ~7, want = L.replay_move ? kReplayPoolMove : kReplayPoolFixed;
     int fits = 0;
     for (int ctas = replay_min_blocks(L.replay_move != 0); ctas >= 2 && fits < want; --ctas) {
         const size_t cta = 227 * 1024 / ctas - 1024;  // 1 KB of a CTA's is the system's
@@ -2372,6 +2372,22 @@ int replay_pool(const TraceLaunch& L) {
     }
     fits = fits < kReplayPoolMax ? fits : kReplayPoolMax;
     return fits > need ? fits & ~7 : need;
+}
+
+// The pool is fitted anew to the tables, sums and pixels of all jobs so far: taken as the least pool
+// for the next job, the first one's would keep the launch to fewer CTAs than its jobs need (8
+// renders on one pixel, then 32 on 4: 4 CTAs per SM instead of the reverse order's 5).
+void replay_cover(TraceLaunch& L, const TraceJob& J) {
+    auto most = [](int& a, int b) { a = a > b ? a : b; };
+    L.replay_mat |= J.var_mats ? 1 : 0;
+    most(L.replay_move, J.n_var > 0 ? (J.black ? 1 : 2) : 0);
+    most(L.halves, J.R > 32 ? 2 : 1);
+    most(L.tab_rows, J.R * J.gstride);
+    most(L.pixels, J.bw * J.bh / J.parts);
+    L.replay_chunked |= J.chunks > 1 ? 1 : 0;
+    most(L.granules, replay_path_granules(J.depth, J.n_var > 0));
+    if (J.diff) L.diff_nd = J.nd;
+    L.pool = replay_pool(L);
 }
 
 // A render's clamp derivatives (Eq. 9) in its row of the table.
