@@ -1868,9 +1868,9 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
                 Job* j = get_job(c, ids[i]);
                 if (kind(j) == pass) order.push_back(j);
             }
-        std::stable_sort(order.begin(), order.end(), [&](const Job* a, const Job* b) {  // replay jobs, by class
-            return kind(a) == 3 && kind(b) == 3 && replay_class(a->trace) < replay_class(b->trace);
-        });
+        const auto replay = std::find_if(order.begin(), order.end(), [&](const Job* j) { return kind(j) == 3; });
+        std::stable_sort(replay, order.end(),  // replay jobs (the last), by class
+                         [](const Job* a, const Job* b) { return replay_class(a->trace) < replay_class(b->trace); });
         std::vector<InstJob> inst(n);
         std::vector<TraceJob> trace(n);
         int blocks = 0, jobs_of[4] = {0, 0, 0, 0}, items_of[4] = {0, 0, 0, 0};
