@@ -37,11 +37,22 @@ CANDIDATES = [(px, cps, rg, nps) for px in (32, 16, 8) for cps in (3, 2) for rg,
 _lock = threading.Lock()
 
 
+# The kernels that a job's candidates run (render groups, path sharing, replay, ...) change with the
+# library's routing rules: entries tuned under other rules are not taken up.
+ROUTES = 2
+
+
 def shape_key(wl) -> str:
+    """Key of everything that a job's route and launch depend on."""
     sc = wl.scene
     counts = [int((sc.prim_type == t).sum()) for t in range(3)]
     mats = sorted(set(int(m) for m in sc.mat_type))
-    return (f"W{wl.width}xH{wl.height}_spp{wl.spp}_d{wl.depth}_rr{wl.rr_start}_R{wl.renders}_D{wl.D}"
+    binds = np.asarray(getattr(wl, "bindings", ())).reshape(-1, 3)
+    if len(binds) == 1 and int(binds[0, 0]) == 4:  # one texture
+        bound = f"tex{int(binds[0, 1])}"
+    else:  # which fields of which primitives and materials are bound
+        bound = "-".join(f"{k}.{i}" for k, i in sorted({(int(k), int(i)) for k, i, _ in binds}))
+    return (f"routes{ROUTES}_e{getattr(wl, 'estimator', 0)}_crn{int(getattr(wl, 'crn', 1))}_b{bound}_W{wl.width}xH{wl.height}_spp{wl.spp}_d{wl.depth}_rr{wl.rr_start}_R{wl.renders}_D{wl.D}"
             f"_prims{counts[0]}-{counts[1]}-{counts[2]}_mats{'-'.join(map(str, mats))}")
 
 
