@@ -81,7 +81,7 @@ struct Job {
 struct prdpt_ctx {
     int device = 0;
     int sms = 0;
-    int occ_grad = 1, occ_render = 1, occ_diff = 1, occ_group = 1;
+    int occ_grad = 1, occ_render = 1, occ_diff = 1, occ_group = 1, occ_prefix = 1;
     std::map<unsigned long long, int> occ_replay;  // resident CTAs per SM by kernel variant and shared memory
     uint64_t budget = 0, used = 0;
     std::map<void*, size_t> allocs;
@@ -105,7 +105,7 @@ struct prdpt_ctx {
     double* s_losses = nullptr;
     size_t s_losses_n = 0;
     unsigned* s_ctl = nullptr;    // [0] queue, [1] done counter, [2..3], [8], [9] batch queues, [4..7] sharing
-                                  // counters, [8] third batch queue (16 words)
+                                  // counters (16 words)
     unsigned long long* s_share = nullptr;  // path sharing: [tiles][96] shared radiance
     size_t s_share_n = 0;
     int* s_aff = nullptr;         // path sharing: list of blocks with affected paths
@@ -142,9 +142,9 @@ struct prdpt_ctx {
     size_t batch_cap = 0;
     int batch_blocks = 0;
     // the packed arrays hold the path-sharing jobs, then the render-group jobs, then the
-    // per-render ones, then the replay jobs: jobs and work items of each kind (one render
-    // launch per kind)
-    int batch_jobs[4] = {0, 0, 0, 0}, batch_items[4] = {0, 0, 0, 0};
+    // per-render ones, the prefix-sharing ones, then the replay jobs: jobs and work items of
+    // each kind (one render launch per kind)
+    int batch_jobs[5] = {}, batch_items[5] = {};
     std::vector<TraceLaunch> batch_replay;  // the packed step's replay launches, by class of job
     // optional CUDA-event timing of the render kernel, recorded on its launch stream
     bool timing = false;
@@ -561,6 +561,14 @@ int grid_for_group(prdpt_ctx* c, int items, int ctas_per_sm) {
     return need < cap ? need : cap;
 }
 
+// Persistent grid of the prefix-sharing kernel: one work item per CTA of kGroupBlock threads
+// (ctas_per_sm counts 256-thread CTAs, as above).
+int grid_for_prefix(prdpt_ctx* c, int items, int ctas_per_sm) {
+    const int per_sm = (ctas_per_sm > 0 && 2 * ctas_per_sm < c->occ_prefix) ? 2 * ctas_per_sm : c->occ_prefix;
+    const int cap = c->sms * per_sm;
+    return items < cap ? items : cap;
+}
+
 // Persistent grid of the replay kernel: one work item per warp of CTAs of kGroupBlock threads
 // (ctas_per_sm counts 256-thread CTAs, as above). 0: the kernel cannot run with its shared memory.
 int grid_for_replay(prdpt_ctx* c, const TraceLaunch& L, int ctas_per_sm) {
@@ -583,11 +591,11 @@ int replay_class(const TraceJob& J) {
     return (J.chunks > 1 ? 16 : 0) | (J.R > 32 ? 8 : 0) | (J.var_mats ? 4 : 0) | (J.n_var > 0 ? (J.black ? 1 : 2) : 0);
 }
 
-// Work items of a gradient job's render launch: pixel blocks (path sharing, replay),
+// Work items of a gradient job's render launch: pixel blocks (path and prefix sharing, replay),
 // (block, group of gsize renders) (render-group mode) or (render, block).
 long long job_items(const TraceJob& J) {
     if (J.emit) return (long long)J.tiles * J.parts * J.chunks;
-    if (J.share) return J.tiles;
+    if (J.share || J.prefix) return J.tiles;
     if (J.gsize > 0) return (long long)J.tiles * (J.R / J.gsize);
     return (long long)J.R * J.tiles;
 }
@@ -615,6 +623,7 @@ cudaError_t timed_trace(prdpt_ctx* c, const TraceLaunch* Ls, int nL, const Trace
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < nL; ++i) {
         const int grid = (Ls[i].group == 2 && !render) ? grid_for_replay(c, Ls[i], ctas_per_sm)
+                         : (Ls[i].group == 3 && !render) ? grid_for_prefix(c, Ls[i].total_items, ctas_per_sm)
                          : Ls[i].diff_nd ? grid_for_diff(c, Ls[i].total_items, ctas_per_sm)
                          : (Ls[i].group && !render) ? grid_for_group(c, Ls[i].total_items, ctas_per_sm)
                                                     : grid_for(c, Ls[i].total_items, render, ctas_per_sm);
@@ -674,6 +683,7 @@ prdpt_status prdpt_create(prdpt_ctx** out, int32_t device, uint64_t hbm_budget_b
     c->occ_render = trace_blocks_per_sm(true);
     c->occ_diff = trace_diff_blocks_per_sm();
     c->occ_group = trace_group_blocks_per_sm();
+    c->occ_prefix = trace_prefix_blocks_per_sm();
     e = cudaStreamCreateWithFlags(&c->io, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         delete c;
@@ -887,6 +897,7 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     J.gsize = 0;
     J.gstride = 0;
     J.emit = 0;
+    J.prefix = 0;
     if (J.share || o->render_groups < 0 || !o->crn || B.tex_mat >= 0 || B.n_prims > kGroupPrims ||
         B.n_mats > kGroupMats)
         return;
@@ -952,6 +963,18 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         const bool moves = (prims >> B.prim_slot[i]) & 1u;
         fixed_light |= !moves && (mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f);
         parts |= moves && (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f);
+    }
+    // Where every emitter moves and no material is bound, such renders share each path's prefix instead
+    // (k_trace_prefix; its table holds whole records' worth of rows).
+    const int wide = 4 * n + nm + (radius ? 2 : 0);
+    const bool lights_move = n > 0 && nm == 0 && !fixed_light && R <= 64;
+    if (!pathwise && !o->no_path_sharing && parts && lights_move && R * wide <= kPrefixTabRows) {
+        J.prefix = 1;
+        J.gstride = stride;
+        J.n_var = n;
+        J.var_prims = prims;
+        J.var_mats = 0u;
+        return;
     }
     const bool grouped = !pathwise && ((parts && (nm > 0 || fixed_light) && R % 4 == 0 && 4 * stride <= kGroupTabRows) ||
                                        (n > 0 && R == 2 && o->spp >= 16));
@@ -1206,7 +1229,7 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
     fill_share(probe, s->host, o);  // path sharing or replay: items are blocks, not (render, block)
     fill_group(probe, s->host, o);
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, o->width, o->height, o->spp, probe.chunks)
-                              : choose_block(c, o->block_pixels, probe.share ? 1 : R, o->width, o->height, false);
+                              : choose_block(c, o->block_pixels, probe.share || probe.prefix ? 1 : R, o->width, o->height, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, o->width, o->height, &bw, &bh, &tiles_x, &tiles);
@@ -1336,7 +1359,7 @@ prdpt_status smoothed_grad_blocks(prdpt_ctx* c, int32_t scene_id, const float* t
     J.parts = probe.parts;
     TL.total_items = int(job_items(J));
     TL.share = J.share;
-    TL.group = J.emit ? 2 : (J.gsize > 0 ? 1 : 0);
+    TL.group = J.emit ? 2 : (J.prefix ? 3 : (J.gsize > 0 ? 1 : 0));
     TL.diff_nd = diff_slots(J);
     if (J.emit) {
         J.queue = c->s_ctl + 0;
@@ -1540,7 +1563,7 @@ static prdpt_status job_create_blocks(prdpt_ctx* c, int32_t scene_id, const prdp
     j->R = 2 * o->pairs;
     const int D = j->D, R = j->R, W = o->width, H = o->height;
     const int px = probe.emit ? choose_replay_block(c, o->block_pixels, W, H, o->spp, probe.chunks)
-                              : choose_block(c, o->block_pixels, probe.share ? 1 : R, W, H, false);
+                              : choose_block(c, o->block_pixels, probe.share || probe.prefix ? 1 : R, W, H, false);
     *whole = probe.emit ? choose_whole_block(c, o, px) : 0;
     int bw, bh, tiles_x, tiles;
     tiles_for(px, W, H, &bw, &bh, &tiles_x, &tiles);
@@ -1828,7 +1851,7 @@ prdpt_status prdpt_step(prdpt_ctx* c, int32_t job_id, void* stream) {
     TL.job0 = j->trace;
     TL.total_items = int(job_items(j->trace));
     TL.share = j->trace.share;
-    TL.group = j->trace.emit ? 2 : (j->trace.gsize > 0 ? 1 : 0);
+    TL.group = j->trace.emit ? 2 : (j->trace.prefix ? 3 : (j->trace.gsize > 0 ? 1 : 0));
     TL.diff_nd = diff_slots(j->trace);
     if (j->trace.emit) replay_cover(TL, j->trace);
     TL.queue = j->queue;
@@ -1861,19 +1884,20 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
             if (j->tex) return fail(PRDPT_E_INVALID_ARG, "texture jobs step alone (prdpt_step)");
         }
         auto kind = [](const Job* j) {
-            return j->trace.share ? 0 : (j->trace.gsize > 0 ? 1 : (j->trace.emit ? 3 : 2));
+            const TraceJob& T = j->trace;
+            return T.share ? 0 : (T.gsize > 0 ? 1 : (T.prefix ? 3 : (T.emit ? 4 : 2)));
         };
-        for (int pass = 0; pass < 4; ++pass)
+        for (int pass = 0; pass < 5; ++pass)
             for (int i = 0; i < n; ++i) {
                 Job* j = get_job(c, ids[i]);
                 if (kind(j) == pass) order.push_back(j);
             }
-        const auto replay = std::find_if(order.begin(), order.end(), [&](const Job* j) { return kind(j) == 3; });
+        const auto replay = std::find_if(order.begin(), order.end(), [&](const Job* j) { return kind(j) == 4; });
         std::stable_sort(replay, order.end(),  // replay jobs (the last), by class
                          [](const Job* a, const Job* b) { return replay_class(a->trace) < replay_class(b->trace); });
         std::vector<InstJob> inst(n);
         std::vector<TraceJob> trace(n);
-        int blocks = 0, jobs_of[4] = {0, 0, 0, 0}, items_of[4] = {0, 0, 0, 0};
+        int blocks = 0, jobs_of[5] = {}, items_of[5] = {};
         std::vector<TraceLaunch> replays;  // per class: its jobs, items, variant, table and pool
         for (int i = 0; i < n; ++i) {
             Job* j = order[i];
@@ -1886,7 +1910,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
             trace[i].fin_begin = blocks - j->R;  // same prefix as the sampler CTAs
             const long long it = job_items(j->trace);
             if (prdpt_status st = check_items((long long)items_of[kd] + it)) return st;
-            if (kd == 3) {
+            if (kd == 4) {
                 if (jobs_of[kd] == 0 || replay_class(j->trace) != replay_class(order[i - 1]->trace)) {
                     replays.emplace_back();
                     items_of[kd] = 0;
@@ -1946,7 +1970,7 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
         c->batch_ids = ids;
         c->batch_blocks = blocks;
         c->batch_replay = std::move(replays);
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 5; ++q) {
             c->batch_jobs[q] = jobs_of[q];
             c->batch_items[q] = items_of[q];
         }
@@ -1962,15 +1986,15 @@ prdpt_status prdpt_step_batch(prdpt_ctx* c, const int32_t* job_ids, int32_t n, v
     PRDPT_CUDA(launch_instantiate(IL, st_));
     std::vector<TraceLaunch> TL;
     int first = 0;
-    unsigned* queues[3] = {c->s_ctl + 2, c->s_ctl + 3, c->s_ctl + 8};
-    for (int kd = 0; kd < 3; ++kd) {  // path-sharing, render-group, per-render jobs
+    unsigned* queues[4] = {c->s_ctl + 2, c->s_ctl + 3, c->s_ctl + 8, c->s_ctl + 9};
+    for (int kd = 0; kd < 4; ++kd) {  // path-sharing, render-group, per-render, prefix-sharing jobs
         if (c->batch_jobs[kd] > 0) {
             TraceLaunch T{};
             T.jobs = c->d_trace + first;
             T.njobs = c->batch_jobs[kd];
             T.total_items = c->batch_items[kd];
             T.share = kd == 0 ? 1 : 0;
-            T.group = kd == 1 ? 1 : 0;
+            T.group = kd == 1 ? 1 : (kd == 3 ? 3 : 0);
             T.queue = queues[kd];
             TL.push_back(T);
         }

@@ -185,7 +185,10 @@ struct TraceJob {
     int gsize, gstride, var_rows;
     unsigned var_offs;
     unsigned char row_src[2 * kMaxVariant];
-    // Replay mode (k_trace_replay): 1 when the job's paths are traced once for all its renders
+    // Prefix mode (k_trace_prefix): `prefix` is 1 when the job's paths are traced once for all its renders
+    // up to the first ray that could meet a perturbed primitive (gstride as above; items are pixel
+    // blocks of all renders).
+    // Replay mode (k_trace_replay): `emit` is 1 when the job's paths are traced once for all its renders
     // and each render replays what differs (gstride as above, plus two rows of clamp derivatives
     // for the pathwise estimator; items are pixel blocks of all renders, taken from `queue`);
     // black: every perturbed primitive's material is diffuse and black (and not bound), and every
@@ -193,7 +196,9 @@ struct TraceJob {
     // a block is `parts` work items (a power of two, at most its pixels), whose sums go through
     // part_sums [tiles][parts][R][1 + nd] when there are several; part_done counts a block's finished
     // parts (zero between launches).
-    int emit, black, parts, chunks;  // chunks: of 64 renders each (several: parts is 1)
+    int emit;
+    short black, prefix;
+    int parts, chunks;        // chunks: of 64 renders each (several: parts is 1)
     double* part_sums;
     unsigned* part_done;
     // pathwise estimator in replay mode: tangent slot k holds parameter slot_param[k] (-1: none) of
@@ -211,7 +216,7 @@ struct TraceLaunch {
     int diff_nd;              // pathwise estimator: tangent slots of the kernel variant (0; k_trace 4, 6, 8;
                               // k_trace_replay 3, 6, 12)
     int group;                // 1: every job of the launch runs in render-group mode (k_trace_group),
-                              // 2: in replay mode (k_trace_replay)
+                              // 2: in replay mode (k_trace_replay), 3: in prefix mode (k_trace_prefix)
     // replay mode, covering every job of the launch: bound materials, perturbed primitives (1 only
     // black ones, 2 any), float4 of the per-render table, granules of a warp's pool, 32-render
     // halves of a warp's sums, pixels of a work item at most
@@ -297,6 +302,7 @@ cudaError_t launch_philox(unsigned long long seed, unsigned c0, unsigned c1, uns
 // kDiffBlock threads.
 int trace_blocks_per_sm(bool render_mode);
 int trace_group_blocks_per_sm();
+int trace_prefix_blocks_per_sm();
 // Resident CTAs per SM of a replay launch's kernel variant with its shared memory (0: it does
 // not fit).
 int trace_replay_blocks_per_sm(const TraceLaunch& L);
@@ -306,6 +312,7 @@ size_t replay_smem(const TraceLaunch& L);
 void replay_cover(TraceLaunch& L, const TraceJob& J);
 constexpr int kGroupBlock = 128;    // render-group CTAs: 4 warps (their per-warp tables fit 48 KB)
 constexpr int kGroupTabRows = 192;  // float4 of a warp's per-render record table (render-group mode)
+constexpr int kPrefixTabRows = 256;   // float4 of a CTA's per-render record table (prefix mode)
 constexpr int kReplayTabRows = 1024;  // float4 of a CTA's per-render record table (replay mode), at most
 // Granules (float4) of a warp's pool that one path may need in replay mode with and without
 // perturbed primitives: per vertex a segment (3), emission (1) and estimate (3; without perturbed

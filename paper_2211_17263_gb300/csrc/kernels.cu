@@ -25,6 +25,8 @@
 //   k_trace_replay  replay: each path traced once for all renders of a job, recording the
 //                   events that can differ; each render replays them with its own
 //                   primitives, albedos and (Eq. 9) tangents.
+//   k_trace_prefix  paths shared up to the first ray that could meet a moving object that is not
+//                   black; from there the renders go on side by side.
 //   k_finalize      one CTA per render: L_r from the block partials (fixed order); the
 //                   CTA completing a job's last render forms the gradient of Eq. 10
 //                   (or the mean of Eq. 9's pathwise gradients) and applies Adam.
@@ -2050,7 +2052,8 @@ __device__ __forceinline__ float4 prim_ball(const float4* P, int type) {
 // box strictly on one side. The margins exceed the FP32 rounding of the intersection tests and
 // of the approximate roots and quotients here, so leaving these primitives out never changes a
 // shadow ray's outcome.
-__device__ __forceinline__ unsigned shadow_cull(const GroupScene& S, const ReplayLane& E, float3 po, int slot) {
+template <class Lane>
+__device__ __forceinline__ unsigned shadow_cull(const GroupScene& S, const Lane& E, float3 po, int slot) {
     const int k = __popc(E.skip & ((1u << slot) - 1u));
     const float3 lo = xyz(E.ulo[k]), hi = xyz(E.uhi[k]);
     const float3 bc = (lo + hi) * 0.5f, bh = (hi - lo) * 0.5f;
@@ -2084,8 +2087,8 @@ __device__ __forceinline__ unsigned shadow_cull(const GroupScene& S, const Repla
 }
 
 // Does the segment o + t d, 0 <= t <= tmax, touch a union box of the perturbed primitives?
-template <bool kCount>
-__device__ __forceinline__ bool replay_touch(const ReplayLane& E, float3 o, float3 d, float tmax, Counters& cnt) {
+template <bool kCount, class Lane>
+__device__ __forceinline__ bool replay_touch(const Lane& E, float3 o, float3 d, float tmax, Counters& cnt) {
     const float3 inv = rcp3(d);
     const float tm = tmax * 1.0001f + 1e-3f;
     bool hit = false;
@@ -2970,6 +2973,369 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
     }
 }
 
+// ---------------------------------------------------------------------------
+// k_trace_prefix: path vertices shared up to the first ray that could meet a moving object (a3-a5)
+// ---------------------------------------------------------------------------
+// For a job of R <= 64 renders whose perturbed primitives include every emitter and at least one
+// that is not black, and whose materials are not bound (e.g. a moving ball and light): the renders'
+// paths agree until one of their rays could meet a perturbed primitive, and differ before that only
+// in the next-event estimates. A work item is one pixel block of all renders, taken by a
+// CTA of kPrefixWarps warps; warp w takes the pixel slots of positions q = 8w .. 8w + 7 of
+// the bit-reversed order. For each pixel, 32 samples at a time:
+//   phase A  lane = sample: the path is traced once in the invariant scene, keeping its
+//            diffuse vertices (PrefixLane) and its end: left the scene (the background term),
+//            ended, or stopped where a ray could meet a perturbed primitive;
+//   phase B  lane = render (lane and lane + 32; with R <= 16, render lane mod G of sample
+//            group lane / G, G the power of two >= R): for each sample that adds anything,
+//            the render's own next-event estimates at the kept vertices (occlusion tested
+//            against the primitives the vertex's cull mask leaves), then the background term
+//            or, for a stopped path, the rest of the path traced in the render's scene (as in
+//            k_trace_group).
+// Each render's radiance is the same sum, term by term and in the same order, as tracing
+// the path in that render alone, so with the same block shape every partial is
+// bit-identical to the per-render kernel's; the warps' subtrees of the pairwise pixel sum
+// are combined as that sum's top two levels.
+// Replay shares such a path further, but where some renders part from it and others do not, a warp
+// waits for both; here all renders of a stopped path go on side by side (237 x 141, 16 renders at 16 spp,
+// replayed and here: a glass ball moving beside the light 540 and 337 us, a grey box beside the GI box's
+// light 4.06 and 1.77 ms). Bound by instruction issue like the other render kernels.
+constexpr int kPrefixCap = 2;      // diffuse vertices kept per path
+constexpr int kPrefixFields = 13;  // po, ns, beta * albedo, the emitter point (lu, lv), emitter li, cull mask
+constexpr int kPrefixWarps = kGroupBlock / 32;
+constexpr int kPrefixSlots = 32 / kPrefixWarps;
+static_assert(kPrefixSlots == 8, "the warps' subtrees are the pairwise sum's levels 0-2");
+constexpr int kPrefixMinBlocks = 5;  // <= 102 registers: 20 resident warps per SM
+
+struct PrefixLane {
+    const float4* ulo;   // as ReplayLane's
+    const float4* uhi;
+    const float4* ball;
+    int n_var;
+    unsigned skip;
+    float* ent;          // the warp's kept vertices: ent[(k * kPrefixFields + field) * 32 + lane]
+    int lane;
+    int n;               // vertices kept by this lane's path
+    bool miss;           // the path ended by leaving the scene
+};
+struct PrefixWarp {
+    float ent[kPrefixCap * kPrefixFields * 32];  // kept vertices of the warp's 32 paths
+    float st[10][32];                            // end state: o, d, beta, vertex b (bits)
+    int n[32];                                   // vertices kept
+    int kind[32];                                // 0 ended, 1 left the scene, 2 stopped (specular flag: 4)
+    double pair[2][3][32];                       // pairwise-sum stacks of the lane's two renders
+};
+struct PrefixSmem {
+    GroupScene scene;  // the invariant part (render 0's records of the other primitives)
+    TraceJob job;
+    float4 tab[kPrefixTabRows];  // per-render rows (as k_trace_group's), R x gstride
+    float4 ulo[kMaxVariant], uhi[kMaxVariant];
+    float4 ball[kGroupPrims];
+    double sub[kPrefixWarps][64];
+    PrefixWarp w[kPrefixWarps];
+    unsigned item;
+    int job_index;
+};
+
+// One vertex of a path in the invariant scene (as advance; no invariant primitive emits): kAffected
+// where the renders trace on themselves, from the path's present ray.
+template <bool kCount>
+__device__ __forceinline__ int prefix_vertex(const GroupScene& S, int depth, int rr_start, Path& p, PrefixLane& E,
+                                             Counters& cnt) {
+    const Hit h = closest_hit<kCount, true>(S, p.o, p.d, cnt, E.skip);
+    if (replay_touch<kCount>(E, p.o, p.d, h.slot < 0 ? 3.0e38f : h.t, cnt)) return kAffected;
+    if (h.slot < 0) {
+        E.miss = true;  // the background term is added per render, after its vertex terms
+        return kEnded;
+    }
+    if (kCount) ++cnt.vertices;
+    const float3 pt = p.o + p.d * h.t;
+    int mat;
+    const float3 ng = surface_normal(static_cast<const float4*>(S.prim[h.slot]), h.type, pt, p.o, p.d, mat);
+    const float4 m0 = S.mat[mat][0];
+    const int mtype = as_int(m0.w);
+    const float3 albedo = xyz(m0);
+    const bool last = p.b + 1 >= depth, rr = !last && rr_start >= 0 && p.b >= rr_start;
+    uint4 w1 = make_uint4(0u, 0u, 0u, 0u);
+    if (mtype == kDiffuse) {
+        const float3 ns = dot3(ng, p.d) < 0.0f ? ng : ng * -1.0f;
+        const float3 po = pt + ns * kEps;
+        const uint4 w0 = path_words<true>(S, p.pixel, p.s, p.b, 0);
+        if (S.n_lights > 1 || rr) w1 = path_words<true>(S, p.pixel, p.s, p.b, 1);
+        if (S.n_lights > 0) {  // kept for the renders' own estimates (the renders' emitters differ)
+            if (E.n == kPrefixCap) return kAffected;
+            float* e = E.ent + E.n * kPrefixFields * 32 + E.lane;
+            const float3 ba = p.beta * albedo;
+            const int li = nee_light(S, w1.x);
+            e[0] = po.x; e[32] = po.y; e[64] = po.z;
+            e[96] = ns.x; e[128] = ns.y; e[160] = ns.z;
+            e[192] = ba.x; e[224] = ba.y; e[256] = ba.z;
+            e[288] = u01(w0.x); e[320] = u01(w0.y); e[352] = __int_as_float(li);
+            e[384] = __uint_as_float(shadow_cull(S, E, po, S.light[li].y));
+            ++E.n;
+        }
+        if (last) return kEnded;
+        p.d = normalized(diffuse_dir(ns, u01(w0.z), u01(w0.w)));
+        p.o = po;
+        p.specular = false;
+    } else {
+        if (last) return kEnded;
+        if (rr || mtype == kDielectric) w1 = path_words<true>(S, p.pixel, p.s, p.b, 1);
+        if (mtype == kMirror) {
+            const float3 ns = dot3(ng, p.d) < 0.0f ? ng : ng * -1.0f;
+            p.d = normalized(p.d - ns * (2.0f * dot3(p.d, ns)));
+            p.o = pt + ns * kEps;
+        } else {
+            dielectric(p, pt, ng, S.mat[mat][1].w, u01(w1.z));
+        }
+        p.specular = true;
+    }
+    p.beta = p.beta * albedo;
+    if (maxc(p.beta) <= 0.0f) return kEnded;
+    if (rr) {  // Russian roulette on slot 1's second uniform
+        const float q = fminf(0.95f, maxc(p.beta));
+        if (u01(w1.y) >= q) return kEnded;
+        p.beta = p.beta * rcp_fast(q);
+    }
+    ++p.b;
+    return kLive;
+}
+
+template <bool kCount>
+__global__ void __launch_bounds__(kGroupBlock, kPrefixMinBlocks) k_trace_prefix(const __grid_constant__ TraceLaunch L) {
+    __shared__ PrefixSmem E;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    PrefixWarp& Wp = E.w[warp];
+    const TraceJob& J = E.job;
+    int cur_job = -1;
+    Counters cnt{0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (!L.jobs) {  // a single job's descriptor is host data: copied before the wait
+        const unsigned* src = reinterpret_cast<const unsigned*>(&L.job0);
+        unsigned* dst = reinterpret_cast<unsigned*>(&E.job);
+        for (int i = threadIdx.x; i < int(sizeof(TraceJob) / 4); i += kGroupBlock) dst[i] = src[i];
+    }
+    __syncthreads();
+    pdl_enter();
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const unsigned item = atomicAdd(L.queue, 1u);
+            int j = 0;
+            if (item < unsigned(L.total_items) && L.jobs) {
+                int lo = 0, hi = L.njobs - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) / 2;
+                    if (L.jobs[mid].item_begin <= int(item)) lo = mid; else hi = mid - 1;
+                }
+                j = lo;
+            }
+            E.item = item;
+            E.job_index = j;
+        }
+        __syncthreads();
+        const unsigned item = E.item;
+        const int j = E.job_index;
+        if (item >= unsigned(L.total_items)) break;
+        if (j != cur_job) {  // stage the job, its invariant scene, per-render rows and union bounds
+            if (L.jobs) {
+                const unsigned* src = reinterpret_cast<const unsigned*>(L.jobs + j);
+                unsigned* dst = reinterpret_cast<unsigned*>(&E.job);
+                for (int i = threadIdx.x; i < int(sizeof(TraceJob) / 4); i += kGroupBlock) dst[i] = src[i];
+                __syncthreads();
+            }
+            if (J.R < 1 || J.R > 64 || J.R * J.gstride > kPrefixTabRows || J.gstride < J.var_rows || J.n_var < 1 ||
+                J.n_var > kMaxVariant || J.n_prims > kGroupPrims || J.n_mats > kGroupMats) {
+                if (threadIdx.x == 0) atomicOr(L.status, kStatusBadItem);
+                break;
+            }
+            if (warp == 0) stage_group_scene(E.scene, J, 0, lane);
+            const int stride = J.gstride, n = J.n_var, nr = J.var_rows;
+            for (int i = threadIdx.x; i < J.R * stride; i += kGroupBlock) {
+                const int r = i / stride, q = i - r * stride;
+                const InstScene& R = J.scenes[r];
+                float4 v;
+                if (q < nr) v = __ldg(&R.prim[J.row_src[q] >> 1][J.row_src[q] & 1]);
+                else v = __ldg(reinterpret_cast<const float4*>(R.light_area) + (q - nr));  // emitter areas
+                E.tab[q * J.R + r] = v;  // field-major, as k_trace_group's table
+            }
+            __syncthreads();
+            if (warp == 1 && lane < J.n_prims && lane < kCullBits)
+                E.ball[lane] = prim_ball(E.scene.prim[lane], lane < E.scene.n_sph ? kSphere
+                                                             : (lane < E.scene.n_sph + E.scene.n_quad ? kQuad : kBox));
+            if (warp == 0) {
+                for (int k = 0; k < n; ++k) {
+                    const int slot = nth_set_bit(J.var_prims, k);
+                    const int type = slot < E.scene.n_sph ? kSphere : (slot < E.scene.n_sph + E.scene.n_quad ? kQuad : kBox);
+                    float3 lo = f3(INFINITY, INFINITY, INFINITY), hi = f3(-INFINITY, -INFINITY, -INFINITY);
+                    for (int r = lane; r < J.R; r += 32) {
+                        float3 a, c;
+                        const SRec own{E.tab + ((J.var_offs >> (8 * k)) & 255u) * J.R + r, J.R, type == kQuad ? 1 : 2, E.scene.prim[slot]};
+                        prim_bounds(own, type, a, c);
+                        lo = f3(fminf(lo.x, a.x), fminf(lo.y, a.y), fminf(lo.z, a.z));
+                        hi = f3(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        lo.x = fminf(lo.x, __shfl_xor_sync(kFull, lo.x, o));
+                        lo.y = fminf(lo.y, __shfl_xor_sync(kFull, lo.y, o));
+                        lo.z = fminf(lo.z, __shfl_xor_sync(kFull, lo.z, o));
+                        hi.x = fmaxf(hi.x, __shfl_xor_sync(kFull, hi.x, o));
+                        hi.y = fmaxf(hi.y, __shfl_xor_sync(kFull, hi.y, o));
+                        hi.z = fmaxf(hi.z, __shfl_xor_sync(kFull, hi.z, o));
+                    }
+                    if (lane == 0) {
+                        E.ulo[k] = make_float4(lo.x, lo.y, lo.z, 0.f);
+                        E.uhi[k] = make_float4(hi.x, hi.y, hi.z, 0.f);
+                    }
+                }
+            }
+            __syncthreads();
+            cur_job = j;
+        }
+        const int t = int(item) - J.item_begin;
+        if (t < 0 || t >= J.tiles) {
+            if (threadIdx.x == 0) atomicOr(L.status, kStatusBadItem);
+            break;
+        }
+        const int R = J.R, nh = R > 32 ? 2 : 1, stride = J.gstride;
+        // phase B lanes: render gi = lane mod G of sample group ks = lane / G (G the power of
+        // two >= R, at most 32): with few renders a warp takes 32 / G samples at a time
+        const int G = R >= 32 ? 32 : (R <= 1 ? 1 : 1 << (32 - __clz(R - 1)));
+        const int nsg = 32 / G, gi = lane % G, ks = lane / G;
+        const int areas = stride > J.var_rows ? 1 : 0;
+        const int x0 = (t % J.tiles_x) * J.bw, y0 = (t / J.tiles_x) * J.bh;
+        const int vw = min(J.bw, J.W - x0), vh = min(J.bh, J.H - y0);
+        const int npx = vw * vh;
+        const unsigned magic_w = 0xffffffffu / unsigned(vw) + 1u;
+        const float inv = mean_scale(J.spp);
+        PrefixLane el{E.ulo, E.uhi, E.ball, J.n_var, J.var_prims, Wp.ent, lane, 0, false};
+        const bool bg_nonzero = E.scene.bg.x != 0.0f || E.scene.bg.y != 0.0f || E.scene.bg.z != 0.0f;
+        double sub[2] = {0.0, 0.0};
+        // The loops below stay rolled: unrolled copies of the tracer overflow the instruction
+        // cache (measured on the caustic step: 13.1 ms unrolled, 11.0 ms rolled).
+#pragma unroll 1
+        for (int qq = 0; qq < kPrefixSlots; ++qq) {
+            const int slot = brev5(warp * kPrefixSlots + qq);  // pixels in bit-reversed slot order
+            double e[2] = {0.0, 0.0};
+            if (slot < npx) {
+                const int row = div_magic(slot, vw, magic_w);
+                const int px = x0 + slot - row * vw, py = y0 + row;
+                unsigned long long acc[2][3] = {{0ull, 0ull, 0ull}, {0ull, 0ull, 0ull}};
+                for (int s0 = 0; s0 < J.spp; s0 += 32) {
+                    // ---- phase A: one path per lane, traced once for all renders ----------
+                    __syncwarp();  // phase B of the previous samples is done with the table
+                    bool work = false;  // does the sample add anything to a render?
+                    if (s0 + lane < J.spp) {
+                        Path p;
+                        start_path<true>(E.scene, J.W, J.H, px, py, s0 + lane, slot, p);
+                        if (kCount) ++cnt.paths;
+                        el.n = 0;
+                        el.miss = false;
+                        int res;
+                        while ((res = prefix_vertex<kCount>(E.scene, J.depth, J.rr_start, p, el, cnt)) == kLive) {
+                        }
+                        Wp.n[lane] = el.n;
+                        Wp.kind[lane] = (res == kAffected ? 2 : (el.miss ? 1 : 0)) | (p.specular ? 4 : 0);
+                        Wp.st[0][lane] = p.o.x;
+                        Wp.st[1][lane] = p.o.y;
+                        Wp.st[2][lane] = p.o.z;
+                        Wp.st[3][lane] = p.d.x;
+                        Wp.st[4][lane] = p.d.y;
+                        Wp.st[5][lane] = p.d.z;
+                        Wp.st[6][lane] = p.beta.x;
+                        Wp.st[7][lane] = p.beta.y;
+                        Wp.st[8][lane] = p.beta.z;
+                        Wp.st[9][lane] = __int_as_float(p.b);
+                        work = el.n > 0 || res == kAffected || (el.miss && bg_nonzero);
+                    }
+                    // ---- phase B: each render's terms of each sample, in sample order -----
+                    // (samples that add nothing to any render -- no kept vertex, not stopped,
+                    // no background term -- are passed over: their sums would add zero)
+                    __syncwarp();
+                    unsigned todo = __ballot_sync(kFull, work);
+#pragma unroll 1
+                    while (todo) {
+                        int jj = -1;  // sample group ks takes the ks-th of the next nsg samples
+                        for (int i = 0; i < nsg && todo; ++i) {
+                            if (i == ks) jj = __ffs(todo) - 1;
+                            todo &= todo - 1u;
+                        }
+                        if (jj < 0) continue;
+                        const int nk = Wp.n[jj], kind = Wp.kind[jj];
+#pragma unroll 1
+                        for (int h = 0; h < nh; ++h) {
+                            const int r = gi + 32 * h;
+                            if (r >= R) continue;
+                            const GroupLane gl{E.tab + r, J.var_prims, 0u, J.var_offs, J.var_rows, areas, nullptr, 0, R};
+                            float3 Lr = f3(0.f, 0.f, 0.f);
+#pragma unroll 1
+                            for (int k = 0; k < nk; ++k) {
+                                const float* en = Wp.ent + k * kPrefixFields * 32 + jj;
+                                const float3 po = f3(en[0], en[32], en[64]), nsv = f3(en[96], en[128], en[160]);
+                                float3 wi;
+                                float dist, g;
+                                int lmat;
+                                if (nee_to<kCount, false, true>(E.scene, po, nsv, en[288], en[320],
+                                                                __float_as_int(en[352]), cnt, __float_as_uint(en[384]),
+                                                                &gl, wi, dist, g, lmat))
+                                    Lr = nee_add(Lr, f3(en[192], en[224], en[256]), xyz(E.scene.mat[lmat][1]), g);
+                            }
+                            const float3 beta = f3(Wp.st[6][jj], Wp.st[7][jj], Wp.st[8][jj]);
+                            if ((kind & 3) == 1) {
+                                Lr = bg_add(Lr, beta, xyz(E.scene.bg));
+                            } else if ((kind & 3) == 2) {  // the rest of the path in render r's scene
+                                Path p;
+                                p.o = f3(Wp.st[0][jj], Wp.st[1][jj], Wp.st[2][jj]);
+                                p.d = f3(Wp.st[3][jj], Wp.st[4][jj], Wp.st[5][jj]);
+                                p.beta = beta;
+                                p.L = Lr;
+                                p.pixel = unsigned(py * J.W + px);
+                                p.s = s0 + jj;
+                                p.b = __float_as_int(Wp.st[9][jj]);
+                                p.slot = slot;
+                                p.specular = (kind & 4) != 0;
+                                p.seg = 0u;
+                                Lr = replay_alone<kCount>(E.scene, J.depth, J.rr_start, gl, p, cnt);
+                            }
+                            if (Lr.x != 0.0f || Lr.y != 0.0f || Lr.z != 0.0f) {
+                                acc[h][0] += to_fixed(Lr.x);
+                                acc[h][1] += to_fixed(Lr.y);
+                                acc[h][2] += to_fixed(Lr.z);
+                            }
+                        }
+                    }
+                }
+                for (int o = G; o < 32; o <<= 1) {  // the render's other sample groups
+                    acc[0][0] += __shfl_xor_sync(kFull, acc[0][0], o);
+                    acc[0][1] += __shfl_xor_sync(kFull, acc[0][1], o);
+                    acc[0][2] += __shfl_xor_sync(kFull, acc[0][2], o);
+                }
+                const float4 T = __ldg(J.target + size_t(py) * J.W + px);
+                for (int h = 0; h < nh; ++h)
+                    e[h] = pixel_sq_error(acc[h][0], acc[h][1], acc[h][2], T, unsigned(J.spp), inv);
+            }
+            for (int h = 0; h < 2; ++h) {  // levels 0-2 of the pairwise sum over this warp's slots
+                double v = e[h];
+                int l = 0;
+                for (; (qq >> l) & 1; ++l) v = Wp.pair[h][l][lane] + v;
+                if (l < 3) Wp.pair[h][l][lane] = v;
+                else sub[h] = v;
+            }
+        }
+        for (int h = 0; h < nh; ++h)
+            if (ks == 0 && gi + 32 * h < R) E.sub[warp][gi + 32 * h] = sub[h];
+        __syncthreads();
+        for (int r = threadIdx.x; r < R; r += kGroupBlock)  // a5: levels 3 and 4
+            J.partials[size_t(r) * J.tiles + t] = (E.sub[0][r] + E.sub[1][r]) + (E.sub[2][r] + E.sub[3][r]);
+        __syncthreads();
+    }
+    if (kCount) {
+        const unsigned v[kNumCounters] = {warp_sum_u(cnt.sph), warp_sum_u(cnt.quad), warp_sum_u(cnt.box),
+                                          warp_sum_u(cnt.paths), warp_sum_u(cnt.vertices), warp_sum_u(cnt.shadow),
+                                          warp_sum_u(cnt.rays), 0u};
+        if (lane == 0)
+            for (int i = 0; i < kNumCounters; ++i) atomicAdd(L.counters + i, (unsigned long long)v[i]);
+    }
+}
+
 // Per-render pass of a path-sharing job: render r traces again each recorded path one of
 // whose kept segments touches render r's bounds of a perturbed primitive, and adds its radiance minus the shared-pass radiance (2^-32 fixed point,
 // modulo 2^64) to the render's image-sized buffer with global atomic adds -- integer
@@ -3427,9 +3793,17 @@ int trace_replay_blocks_per_sm(const TraceLaunch& L) {
     return n;
 }
 
+int trace_prefix_blocks_per_sm() {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace_prefix<false>, kGroupBlock, 0);
+    return n > 0 ? n : 1;
+}
+
 cudaError_t launch_trace(const TraceLaunch& L, bool render_mode, int grid, cudaStream_t stream) {
     if (L.total_items <= 0) return cudaSuccess;
     const bool count = L.counters != nullptr;
+    if (L.group == 3 && !render_mode)
+        return launch_pdl(count ? k_trace_prefix<true> : k_trace_prefix<false>, grid, kGroupBlock, stream, L);
     if (L.group == 2 && !render_mode)
         return launch_pdl_smem(replay_kernel(L), grid, kGroupBlock, replay_smem(L), stream, L);
     if (L.group && !render_mode)
