@@ -949,13 +949,17 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     const int rstride = stride + (J.nd + 3) / 4;
     // (Beyond 64 renders only with bound materials: a path is then traced once per 64 renders, which
     // still beats render groups -- GI box 256 x 256 at 16 spp, 80 renders: 13.6 -> 5.0 ms.)
-    // Where the renders part from the path (a perturbed primitive that is not black is seen) they trace
-    // the rest one lane each, so groups of 4 or more stay faster beside bound albedos or fixed emitters
-    // (GI box with a grey box moving, 400 x 400: 8 renders at 2 spp 1.29 ms in groups, 2.54 ms replayed; 6
-    // renders, groups of 2, 2.28 and 1.60 ms). With 2 renders the chains cost more than a second trace
-    // from 16 spp on (GI box 1.81 and 1.99 ms), and for Eq. 9 with fewer samples or 4 renders too
-    // (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16 spp 1.94 and 1.74; 4 renders at
-    // 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
+    // Where the renders part from the path (a perturbed primitive that is not black is seen) a warp waits
+    // for those that do and those that do not, so beside bound albedos or fixed emitters they run in
+    // groups; but groups of two (render counts that 4 does not divide) take ceil(spp / 16) passes for
+    // each pair, and a small image's replay has few lanes to wait for. GI box with a grey box moving, 300 x
+    // 300, groups and replay in ms: 10 renders at 2 spp 2.60, 1.37; at 8 spp 3.48, 4.31; 30 renders at
+    // 8 spp 9.61, 6.56; at 16 spp 11.0, 11.8; 37 x 21, 10 renders at 13 spp 0.23, 0.21.
+    // Where nothing parts, replay's chains cost more than the few renders' traces: beside fixed emitters with
+    // up to 4 renders (400 x 400, 4 renders at 8 spp 0.35 ms in groups, 0.46 replayed; 6 renders 0.87,
+    // 0.47), with bound albedos 2 renders from 16 spp on (GI box 1.81 and 1.99 ms), and for Eq. 9 with
+    // fewer samples or 4 renders too (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16
+    // spp 1.94 and 1.74; 4 renders at 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
     bool parts = false, fixed_light = false;
     for (int i = 0; i < B.n_prims; ++i) {
         const int m = B.prim_mat[i];
@@ -976,8 +980,10 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         J.var_mats = 0u;
         return;
     }
-    const bool grouped = !pathwise && ((parts && (nm > 0 || fixed_light) && R % 4 == 0 && 4 * stride <= kGroupTabRows) ||
-                                       (n > 0 && R == 2 && o->spp >= 16));
+    const bool narrow = R % 4 == 2 && (5LL * o->spp * ((R + 31) / 32) < 2LL * R * ((o->spp + 15) / 16) ||
+                                       (R <= 10 && (long long)o->width * o->height * o->spp <= 24000));
+    const bool grouped = !pathwise && n > 0 &&
+                         (parts ? !narrow : (nm > 0 ? R == 2 && o->spp >= 16 : fixed_light && R <= 4));
     const bool few = pathwise && R < 6 && R * R * o->spp < 64;
     if (!o->no_path_sharing && !grouped && !few && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
         J.emit = 1;
@@ -990,13 +996,16 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         return;
     }
     if (pathwise) return;
+    // The largest group whose records would fit with all four rows each. (Only the rows that differ are
+    // kept, so more would fit, but larger groups leave fewer work items and part more: the above at 96 x
+    // 95 and 2 spp, 32 renders in groups of 16 0.68 ms, of 32 1.18; 300 x 295 at 8 spp 5.31 and 5.68.)
     int G = 0;
     if (o->render_groups > 0) {
         const int g = o->render_groups;
-        if ((g & (g - 1)) == 0 && g >= 2 && g <= 32 && R % g == 0 && g * stride <= kGroupTabRows) G = g;
+        if ((g & (g - 1)) == 0 && g >= 2 && g <= 32 && R % g == 0 && g * wide <= kGroupTabRows) G = g;
     } else {
         for (int g = 32; g >= 2; g >>= 1)
-            if (R % g == 0 && g * stride <= kGroupTabRows) {
+            if (R % g == 0 && g * wide <= kGroupTabRows) {
                 G = g;
                 break;
             }

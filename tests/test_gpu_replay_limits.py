@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 import workloads
-from test_gpu_replay import _gi, _light, _t, _walls
+from test_gpu_replay import _bind, _box_light_wall, _gi, _light, _t, _two_lights, _walls
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -171,3 +171,23 @@ def test_more_work_items_than_numbers_stay_refused(ctx):
         with pytest.raises(capi.PrdptError, match="work items"):
             scene.smoothed_grad(dev[:6], dev[:6], dev, opts)
         assert ctx.memory_used() == before
+
+
+def _moving_and_fixed_light(**kw):  # one emitter moves, the other is fixed: no render parts from a path
+    wl = _two_lights(**kw)
+    return _bind(wl, wl.bindings[:3], wl.theta0[:3], wl.sigma[:3])
+
+
+@pytest.mark.parametrize("make,pairs,spp,grouped", [
+    (_box_light_wall, 1, 40, True), (_box_light_wall, 3, 16, True), (_box_light_wall, 13, 16, True),
+    (_box_light_wall, 3, 2, False), (_box_light_wall, 13, 2, False), (_two_lights, 5, 16, True),
+    (_moving_and_fixed_light, 1, 8, True), (_moving_and_fixed_light, 2, 8, True), (_moving_and_fixed_light, 3, 8, False),
+    (_gi, 1, 16, True), (_gi, 1, 8, False), (_light, 1, 32, False)])
+def test_routes_where_replay_is_slower(ctx, make, pairs, spp, grouped):
+    """Jobs whose renders part from the paths, and few renders beside fixed emitters, run in groups,
+    which count every render's paths; where replay pays it counts each path once. Same results."""
+    wl = make(width=96, height=60, spp=spp, pairs=pairs)
+    paths = wl.width * wl.height * wl.spp * (2 * pairs if grouped else 1)
+    assert _count(ctx, wl, block_pixels=8)[3] == paths
+    (g, L), (g0, L0) = (_grad(ctx, wl, block_pixels=8, **kw) for kw in ({}, dict(no_path_sharing=1, render_groups=-1)))
+    assert np.array_equal(L, L0) and np.array_equal(g, g0)
