@@ -465,12 +465,16 @@ int choose_block(prdpt_ctx* c, int requested, int R, int W, int H, bool render) 
 // Is a replay work item of px pixels worth splitting in two? Up to eight items per resident warp while
 // each half still fills two batches of paths (32 each); a small image would otherwise end in a
 // half-empty round (GI box walls 256 x 256 at 32 spp, 24 warps per SM: blocks of 8 pixels 1.55 ms, of 4
-// pixels 1.25 ms). While there are fewer items than warps, down to 8 paths: idle warps cost more
-// than half-empty batches (GI box 86 x 86 at 3 spp, 78 renders: 484 items of 32 pixels 3.06 ms, split to
-// 4 pixels 0.23 ms; render groups 2.01 ms).
+// pixels 1.25 ms); up to four per warp where each half is one full batch (GI box with only its light
+// moving, 96 x 96 at 32 spp, 2 renders: 1.5 items per warp 402 us, split 211). While there are fewer items
+// than warps, down to 8 paths: idle warps cost more than half-empty batches (GI box 86 x 86 at 3 spp,
+// 78 renders: 484 items of 32 pixels 3.06 ms, split to 4 pixels 0.23 ms; render groups 2.01 ms); while the
+// halves still have a warp each, down to one pixel: a warp replays its pixels one after another (caustic
+// 24 x 24 at 1 spp, 2 renders: 8 pixels an item 45 us, one pixel 27, emitter sharing 29).
 bool replay_split(prdpt_ctx* c, long long items, int px, int spp) {
     const long long warps = (long long)c->sms * kReplayWarpsPerSm, paths = (long long)(px / 2) * spp;
-    return px > 1 && ((items < 8 * warps && paths >= 64) || (items < warps && paths >= 8));
+    return px > 1 && ((items < 8 * warps && paths >= 64) || (items < 4 * warps && paths == 32) ||
+                      (items < warps && paths >= 8) || 2 * items <= warps);
 }
 
 // Pixels per block in replay mode when the caller does not say.

@@ -191,3 +191,16 @@ def test_routes_where_replay_is_slower(ctx, make, pairs, spp, grouped):
     assert _count(ctx, wl, block_pixels=8)[3] == paths
     (g, L), (g0, L0) = (_grad(ctx, wl, block_pixels=8, **kw) for kw in ({}, dict(no_path_sharing=1, render_groups=-1)))
     assert np.array_equal(L, L0) and np.array_equal(g, g0)
+
+
+@pytest.mark.parametrize("make", [_gi, _walls, _light, _eq9])
+@pytest.mark.parametrize("width,height,spp,pairs", [(1, 1, 1, 1), (24, 24, 1, 1), (5, 3, 3, 24), (40, 33, 3, 5),
+                                                    (64, 47, 1, 16), (96, 60, 32, 1), (76, 41, 32, 3)])
+def test_items_down_to_one_pixel(ctx, make, width, height, spp, pairs):
+    """Small images in items of one pixel, and items of one full batch each. In parts of 8-pixel
+    blocks the losses are the per-render kernel's bit for bit (Eq. 9's too); with automatic blocks its
+    FP64 partial sums are grouped differently, and an FP32 loss may differ in its last bit."""
+    wl = make(width=width, height=height, spp=spp, pairs=pairs)
+    want = _grad(ctx, wl, block_pixels=8, no_path_sharing=1, render_groups=-1)[1]
+    assert np.array_equal(_grad(ctx, wl, block_pixels=8)[1], want)
+    assert np.allclose(_grad(ctx, wl)[1], want, rtol=2.0**-22, atol=0.0)
