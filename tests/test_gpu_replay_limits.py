@@ -204,3 +204,11 @@ def test_items_down_to_one_pixel(ctx, make, width, height, spp, pairs):
     want = _grad(ctx, wl, block_pixels=8, no_path_sharing=1, render_groups=-1)[1]
     assert np.array_equal(_grad(ctx, wl, block_pixels=8)[1], want)
     assert np.allclose(_grad(ctx, wl)[1], want, rtol=2.0**-22, atol=0.0)
+
+
+@pytest.mark.parametrize("pairs", [1, 2, 3, 5, 6, 15, 16, 17])
+def test_sample_groups_side_by_side(ctx, pairs):
+    """1 to 16 sample groups in a warp, powers of two and others, summed by halves."""
+    wl = _light(width=45, height=23, spp=37, pairs=pairs)
+    (g, L), (g0, L0) = (_grad(ctx, wl, block_pixels=16, **kw) for kw in ({}, dict(no_path_sharing=1, render_groups=-1)))
+    assert np.array_equal(L, L0) and np.array_equal(g, g0)
