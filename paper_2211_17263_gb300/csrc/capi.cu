@@ -958,7 +958,8 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     // groups; but groups of two (render counts that 4 does not divide) take ceil(spp / 16) passes for
     // each pair, and a small image's replay has few lanes to wait for. GI box with a grey box moving, 300 x
     // 300, groups and replay in ms: 10 renders at 2 spp 2.60, 1.37; at 8 spp 3.48, 4.31; 30 renders at
-    // 8 spp 9.61, 6.56; at 16 spp 11.0, 11.8; 37 x 21, 10 renders at 13 spp 0.23, 0.21.
+    // 8 spp 9.61, 6.56; at 16 spp 11.0, 11.8; 37 x 21, 10 renders at 13 spp 0.23, 0.21; 64 x 64, 2 renders
+    // at 2 spp 0.155, 0.129; 96 x 95 0.178, 0.211.
     // Where nothing parts, replay's chains cost more than the few renders' traces: beside fixed emitters with
     // up to 4 renders (400 x 400, 4 renders at 8 spp 0.35 ms in groups, 0.46 replayed; 6 renders 0.87,
     // 0.47), with bound albedos 2 renders from 16 spp on (GI box 1.81 and 1.99 ms), and for Eq. 9 with
@@ -985,7 +986,7 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         return;
     }
     const bool narrow = R % 4 == 2 && (5LL * o->spp * ((R + 31) / 32) < 2LL * R * ((o->spp + 15) / 16) ||
-                                       (R <= 10 && (long long)o->width * o->height * o->spp <= 24000));
+                                       (R <= 10 && o->width * o->height <= 4096 && o->width * o->height * o->spp <= 24000));
     const bool grouped = !pathwise && n > 0 &&
                          (parts ? !narrow : (nm > 0 ? R == 2 && o->spp >= 16 : fixed_light && R <= 4));
     const bool few = pathwise && R < 6 && R * R * o->spp < 64;

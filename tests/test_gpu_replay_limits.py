@@ -179,7 +179,7 @@ def _moving_and_fixed_light(**kw):  # one emitter moves, the other is fixed: no 
 
 
 @pytest.mark.parametrize("make,pairs,spp,grouped", [
-    (_box_light_wall, 1, 40, True), (_box_light_wall, 3, 16, True), (_box_light_wall, 13, 16, True),
+    (_box_light_wall, 1, 40, True), (_box_light_wall, 1, 2, True), (_box_light_wall, 3, 16, True), (_box_light_wall, 13, 16, True),
     (_box_light_wall, 3, 2, False), (_box_light_wall, 13, 2, False), (_two_lights, 5, 16, True),
     (_moving_and_fixed_light, 1, 8, True), (_moving_and_fixed_light, 2, 8, True), (_moving_and_fixed_light, 3, 8, False),
     (_gi, 1, 16, True), (_gi, 1, 8, False), (_light, 1, 32, False)])
