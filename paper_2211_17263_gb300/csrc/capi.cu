@@ -962,9 +962,10 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     // at 2 spp 0.155, 0.129; 96 x 95 0.178, 0.211.
     // Where nothing parts, replay's chains cost more than the few renders' traces: beside fixed emitters with
     // up to 4 renders (400 x 400, 4 renders at 8 spp 0.35 ms in groups, 0.46 replayed; 6 renders 0.87,
-    // 0.47), with bound albedos 2 renders from 16 spp on (GI box 1.81 and 1.99 ms), and for Eq. 9 with
-    // fewer samples or 4 renders too (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16
-    // spp 1.94 and 1.74; 4 renders at 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
+    // 0.47), with bound albedos 2 renders from 12 spp on (GI box 400 x 400 at 16 spp 1.81 and 1.99 ms, 281 x 103
+    // at 13 spp 0.33 and 0.35, 300 x 295 at 8 spp 0.84 and 0.72), and for Eq. 9 with fewer samples or 4
+    // renders too (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16 spp 1.94 and 1.74;
+    // 4 renders at 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
     bool parts = false, fixed_light = false;
     for (int i = 0; i < B.n_prims; ++i) {
         const int m = B.prim_mat[i];
@@ -988,7 +989,7 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     const bool narrow = R % 4 == 2 && (5LL * o->spp * ((R + 31) / 32) < 2LL * R * ((o->spp + 15) / 16) ||
                                        (R <= 10 && o->width * o->height <= 4096 && o->width * o->height * o->spp <= 24000));
     const bool grouped = !pathwise && n > 0 &&
-                         (parts ? !narrow : (nm > 0 ? R == 2 && o->spp >= 16 : fixed_light && R <= 4));
+                         (parts ? !narrow : (nm > 0 ? R == 2 && o->spp >= 12 : fixed_light && R <= 4));
     const bool few = pathwise && R < 6 && R * R * o->spp < 64;
     if (!o->no_path_sharing && !grouped && !few && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
         J.emit = 1;
