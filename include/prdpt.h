@@ -137,13 +137,17 @@ typedef struct {
     int32_t ctas_per_sm;       /* resident render CTAs per SM, counted as 256-thread CTAs (kernels with
                                   smaller CTAs keep proportionally more; capped at the occupancy
                                   limit); 0 = occupancy limit */
-    int32_t no_path_sharing;   /* 0: with crn = 1, trace paths that no perturbation can touch once for
-                                  all renders (geometry-only perturbations), or, for the other jobs
-                                  without texture or emission bindings (at most 64 renders), trace
-                                  each path once and let every render replay what differs: its own
-                                  next-event estimates, primitives, albedos and tangents (replay);
-                                  same result, bit for bit (Eq. 9's tangents to rounding); 1: trace
-                                  every render */
+    int32_t no_path_sharing;   /* 0: with crn = 1, share path samples between the renders where that
+                                  is the faster way: paths that no perturbation can touch are traced
+                                  once for all renders (no emitter moves); each path is traced once and
+                                  every render replays what differs, its own next-event estimates,
+                                  primitives, albedos and tangents (replay: an emitter moves or albedos
+                                  are bound; no texture or emission bindings, at most 16 primitives, 16
+                                  materials and 4 moving primitives; up to 64 renders, more with bound
+                                  albedos under Eq. 10 while their rows fit; Eq. 9 with up to 4 albedos
+                                  per channel); or up to the first ray that could meet a moving object
+                                  (every emitter and an object that is not black move). Same result, bit
+                                  for bit (Eq. 9's tangents to rounding); 1: trace every render */
     int32_t estimator;         /* PRDPT_ESTIMATOR_*: 0 = Eq. 10 (kernel-gradient weights times render
                                   losses); 1 = Eq. 9 (mean over the renders of each render's pathwise
                                   loss gradient: requires sampler = GAUSS, every binding an albedo or
@@ -158,7 +162,8 @@ typedef struct {
                                   and whose per-render records fit), -1 = off (one render per work
                                   item), or 2, 4, 8, 16, 32. Used with crn = 1, the Eq. 10 estimator
                                   and no texture or emission bindings; ignored otherwise, and when
-                                  replay applies (see no_path_sharing; -1 turns replay off too) */
+                                  paths are shared (see no_path_sharing; -1 turns all but the first
+                                  way of sharing off too) */
 } prdpt_grad_opts;
 #define PRDPT_ESTIMATOR_KERNEL_GRADIENT 0 /* Eq. 10: sum_r w_r L_r */
 #define PRDPT_ESTIMATOR_PATHWISE 1        /* Eq. 9: mean_r dL/dtheta (theta + tau_r) */

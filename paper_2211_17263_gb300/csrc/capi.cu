@@ -966,12 +966,22 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
     // at 13 spp 0.33 and 0.35, 300 x 295 at 8 spp 0.84 and 0.72), and for Eq. 9 with fewer samples or 4
     // renders too (walls, 2 renders at 4 spp 0.60 per render and 0.84 replayed, at 16 spp 1.94 and 1.74;
     // 4 renders at 2 spp 0.66 and 0.70, at 4 spp 1.08 and 0.72).
-    bool parts = false, fixed_light = false;
+    // Where lights stay and an object moves (jobs that path sharing does not take, beyond 64 samples or its
+    // scratch), few paths meet it: replay beats groups but for the fewest renders of large images
+    // (occlusion at 65 spp, groups and replay in ms: 96 x 93, 2 renders 0.40, 0.23; 16 4.35, 0.60; 32 15.9,
+    // 0.90; 200 x 197, 2 renders 0.56, 0.74; 512 x 512 at 64 spp, 4 renders 4.10, 4.56; 16 13.5, 8.37)
+    // and 17 to 31 renders of the smallest (small scene 40 x 37, 20 renders 0.17, 0.23). With bound albedos
+    // as well every path is replayed in full, and groups of 2 or 4 win up to 16 renders (GI box with a grey
+    // box and its walls, 96 x 93: 4 renders 1.70, 1.50; 6 1.33, 1.89; 8 2.95, 2.02; 12 2.25, 2.81; 20 4.16,
+    // 3.74; 200 x 197, 4 renders 3.92, 5.98; 40 x 37, 6 renders 0.94, 0.65).
+    bool parts = false, fixed_light = false, light_moves = false;
     for (int i = 0; i < B.n_prims; ++i) {
         const int m = B.prim_mat[i];
         const float* mp = B.mat_param[m];
         const bool moves = (prims >> B.prim_slot[i]) & 1u;
-        fixed_light |= !moves && (mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f);
+        const bool emits = mp[3] > 0.f || mp[4] > 0.f || mp[5] > 0.f;
+        fixed_light |= emits && !moves;
+        light_moves |= emits && moves;
         parts |= moves && (B.mat_type[m] != kDiffuse || ((mats >> m) & 1u) || mp[0] > 0.f || mp[1] > 0.f || mp[2] > 0.f);
     }
     // Where every emitter moves and no material is bound, such renders share each path's prefix instead
@@ -986,10 +996,16 @@ static void fill_group(TraceJob& J, const BaseScene& B, const prdpt_grad_opts* o
         J.var_mats = 0u;
         return;
     }
+    const long long pixels = (long long)o->width * o->height;
     const bool narrow = R % 4 == 2 && (5LL * o->spp * ((R + 31) / 32) < 2LL * R * ((o->spp + 15) / 16) ||
-                                       (R <= 10 && o->width * o->height <= 4096 && o->width * o->height * o->spp <= 24000));
-    const bool grouped = !pathwise && n > 0 &&
-                         (parts ? !narrow : (nm > 0 ? R == 2 && o->spp >= 12 : fixed_light && R <= 4));
+                                       (R <= 10 && pixels <= 4096 && pixels * o->spp <= 24000));
+    bool grouped = false;
+    if (!pathwise && n > 0) {
+        if (!parts) grouped = nm > 0 ? R == 2 && o->spp >= 12 : fixed_light && R <= 4;
+        else if (light_moves) grouped = !narrow;
+        else if (nm > 0) grouped = R % 8 != 0 && R < 18 && pixels > (R == 4 ? 9216 : 2048) && !narrow;
+        else grouped = R <= 4 ? pixels > 4096 * R * R : R > 16 && R < 32 && R % 8 != 0 && pixels <= 4096;
+    }
     const bool few = pathwise && R < 6 && R * R * o->spp < 64;
     if (!o->no_path_sharing && !grouped && !few && (!pathwise || J.nd > 0) && R >= 1 && (R <= 64 || (nm > 0 && !pathwise)) && R * rstride <= kReplayTabRows) {
         J.emit = 1;

@@ -189,8 +189,8 @@ struct TraceJob {
     // up to the first ray that could meet a perturbed primitive (gstride as above; items are pixel
     // blocks of all renders).
     // Replay mode (k_trace_replay): `emit` is 1 when the job's paths are traced once for all its renders
-    // and each render replays what differs (gstride as above, plus two rows of clamp derivatives
-    // for the pathwise estimator; items are pixel blocks of all renders, taken from `queue`);
+    // and each render replays what differs (gstride as above, plus (nd + 3) / 4 rows of clamp
+    // derivatives for the pathwise estimator; items are pixel blocks of all renders, taken from `queue`);
     // black: every perturbed primitive's material is diffuse and black (and not bound), and every
     // emitter is perturbed
     // a block is `parts` work items (a power of two, at most its pixels), whose sums go through

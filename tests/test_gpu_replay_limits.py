@@ -178,14 +178,26 @@ def _moving_and_fixed_light(**kw):  # one emitter moves, the other is fixed: no 
     return _bind(wl, wl.bindings[:3], wl.theta0[:3], wl.sigma[:3])
 
 
+def _box_moves(**kw):  # the occlusion task: a box moves under a fixed light
+    return workloads.scaled(workloads.config_occlusion(), **kw)
+
+
+def _box_and_walls(**kw):  # a grey box and two walls' albedos under a fixed light
+    wl = _box_light_wall(**kw)
+    keep = [0, 1, 2, 6, 7]
+    return _bind(wl, wl.bindings[keep], wl.theta0[keep], wl.sigma[keep])
+
+
 @pytest.mark.parametrize("make,pairs,spp,grouped", [
     (_box_light_wall, 1, 40, True), (_box_light_wall, 1, 2, True), (_box_light_wall, 3, 16, True), (_box_light_wall, 13, 16, True),
     (_box_light_wall, 3, 2, False), (_box_light_wall, 13, 2, False), (_two_lights, 5, 16, True),
     (_moving_and_fixed_light, 1, 8, True), (_moving_and_fixed_light, 2, 8, True), (_moving_and_fixed_light, 3, 8, False),
-    (_gi, 1, 16, True), (_gi, 1, 8, False), (_light, 1, 32, False)])
+    (_gi, 1, 16, True), (_gi, 1, 8, False), (_light, 1, 32, False), (_box_moves, 1, 65, False), (_box_moves, 8, 65, False),
+    (_box_and_walls, 3, 65, True), (_box_and_walls, 4, 65, False), (_box_and_walls, 10, 65, False)])
 def test_routes_where_replay_is_slower(ctx, make, pairs, spp, grouped):
     """Jobs whose renders part from the paths, and few renders beside fixed emitters, run in groups,
-    which count every render's paths; where replay pays it counts each path once. Same results."""
+    which count every render's paths; where replay pays it counts each path once (beyond 64 samples
+    also where path sharing would). Same results."""
     wl = make(width=96, height=60, spp=spp, pairs=pairs)
     paths = wl.width * wl.height * wl.spp * (2 * pairs if grouped else 1)
     assert _count(ctx, wl, block_pixels=8)[3] == paths
