@@ -2023,7 +2023,7 @@ struct ReplayLane {
     bool rec;            // recording (the renders may differ from here on)
     bool varied;         // a bound material was met: p.beta is an upper bound over the renders
     bool full;           // the pool ran out: the path is traced again in a later batch
-    bool cull;           // look for primitives that no render's shadow ray can meet (without bound materials)
+    bool cull;           // look for primitives that no render's shadow ray can meet (kMove 1, no bound materials)
 };
 
 // Enclosing ball of a primitive record, inflated beyond the FP32 rounding of its test.
@@ -2157,7 +2157,7 @@ __device__ __forceinline__ int replay_vertex(const GroupScene& S, int depth, int
                 if (kMove == 1 || (kMove && ((E.skip >> lslot) & 1u))) {  // each render's own estimate
                     est = 1u;
                     rec = true;
-                    if (kMat || E.cull) vert = shadow_cull(S, E, po, lslot) << (32 - kCullBits);
+                    if (kMat || kMove != 1 || E.cull) vert = shadow_cull(S, E, po, lslot) << (32 - kCullBits);
                     v0 = make_float4(po.x, po.y, po.z, 0.f);
                     if (kMat) {
                         v1 = make_float4(lu, lv, urr, 0.f);
@@ -2917,7 +2917,7 @@ __global__ void __launch_bounds__(kGroupBlock, replay_min_blocks(kMove != 0)) k_
                     // the pixel is complete: add its sample groups and the common part, form the error
                     auto groups = [&](unsigned long long v) {
                         unsigned long long sum = v;
-                        if (kMat) {
+                        if (kMat || kMove != 1) {
                             _Pragma("unroll 1") for (int q = 1; q < nsg; ++q) sum += __shfl_sync(kFull, v, (lane + q * G) & 31);
                         } else {  // by halves (caustic 400 x 400 at 32 spp, 2 renders: 16 groups, 679 -> 612 us)
                             _Pragma("unroll 1") for (int q = 1; q < nsg; q *= 2) {
