@@ -534,7 +534,8 @@ def main():
             kernels = "render pipeline (k_trace shared pass, k_trace_affected, k_shared_epilogue, k_finalize)"
         elif replayed:
             kernels = "replay kernel k_trace_replay + k_finalize"
-        elif shape["render_groups"] >= 0 and wl.crn and wl.D <= 64:
+        elif (shape["render_groups"] >= 0 and wl.crn and wl.D <= 64 and getattr(wl, "estimator", 0) == 0 and
+              not (np.asarray(wl.bindings)[:, 0] == workloads.BIND_MAT_EMISSION).any()):
             kernels = "render-group kernel k_trace_group + k_finalize"
         else:
             kernels = "render kernel k_trace + k_finalize"
